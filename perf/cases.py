@@ -24,6 +24,7 @@ import functools
 import math
 import types
 
+import numpy as np
 import torch
 
 from paper_2509_26538_b200 import binding as hb
@@ -159,18 +160,25 @@ def _normal(c, S, g, gain=1.0):
     return t
 
 
+def _inputs(c, seed):
+    """([[q, k, v] per layer], gradient of the output or None) on the GPU, from the seed alone."""
+    S = c["text"] + c["frames"] * c["H"] * c["W"]
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    qkv = [[_normal(c, S, g, c["gain"]), _normal(c, S, g), _normal(c, S, g)] for _ in range(c["layers"])]
+    return qkv, _normal(c, S, g) if c["kind"] == "train" else None
+
+
 def prepare(case, seed):
     c = dict(case)
     st = types.SimpleNamespace(case=c)
-    g = torch.Generator(device="cuda")
-    g.manual_seed(seed)
     if c["kind"] == "plan":
         # another request: the offset is what changes from layer to layer and from seed to seed
         c["offset"] += 1 + seed % 997
         return st
     st.plans = [_new_plan(c, layer) for layer in range(c["layers"])]
     S = st.plans[0].S
-    st.qkv = [[_normal(c, S, g, c["gain"]), _normal(c, S, g), _normal(c, S, g)] for _ in range(c["layers"])]
+    st.qkv, st.dout = _inputs(c, seed)
     out_dtype = torch.bfloat16 if c["dtype"] == "fp8" else _DTYPES[c["dtype"]]
     st.out = [_empty(c, S, out_dtype) for _ in range(c["layers"])]
     for p in st.plans:
@@ -179,7 +187,6 @@ def prepare(case, seed):
         st.first = [_empty(c, S, _DTYPES[c["dtype"]]) for _ in range(3)]
     elif c["kind"] == "train":
         st.lse = torch.empty((c["batch"], c["heads"], S), dtype=torch.float32, device="cuda")
-        st.dout = _normal(c, S, g)
         st.grads = [_empty(c, S, out_dtype) for _ in range(3)]
     elif c["kind"] == "host":
         st.qkv = [[t.cpu().pin_memory() for t in st.qkv[0]]]
@@ -250,3 +257,119 @@ def tolerance(case):
     if case["dtype"] == "fp8":
         return {"rel": 8e-2}    # weights rounded to 3 mantissa bits: 1.6e-2 ... 2.5e-2
     return {"rel": 1e-2}        # weights and results rounded to 8 bits: 1.9e-3 ... 2.8e-3
+
+
+# What the path computes, from its definition, in 64 bits.
+
+
+def _curve(k):
+    """[4^k, 2]: (row, col) of the cells of a 2^k x 2^k grid along the Hilbert curve from (0, 0) to (0, 2^k - 1)."""
+    x = y = np.zeros(1, dtype=np.int64)
+    for level in range(k):
+        s = 1 << level
+        x, y = (np.concatenate([y, x, x + s, 2 * s - 1 - y]), np.concatenate([x, y + s, y + s, s - 1 - x]))
+    return np.stack([y, x], 1)
+
+
+def _curve3(k):
+    """[8^k, 3]: (frame, row, col) along the 3-D curve of Skilling's transpose construction."""
+    d = np.arange(1 << (3 * k), dtype=np.int64)
+    X = [np.zeros_like(d) for _ in range(3)]
+    for bit in range(3 * k):
+        X[bit % 3] |= ((d >> (3 * k - 1 - bit)) & 1) << (k - 1 - bit // 3)
+    t = X[2] >> 1
+    X[2], X[1], X[0] = X[2] ^ X[1], X[1] ^ X[0], X[0] ^ t
+    for q in range(1, k):
+        Q = 1 << q
+        for i in (2, 1, 0):
+            up = (X[i] & Q) != 0
+            t = np.where(up, 0, (X[0] ^ X[i]) & (Q - 1))
+            X[0] = np.where(up, X[0] ^ (Q - 1), X[0] ^ t)
+            X[i] = X[i] ^ t
+    return np.stack(X, 1)
+
+
+def _curve_index(c):
+    """Position on the padded curve of every image token, [frames, H, W]."""
+    F, H, W = c["frames"], c["H"], c["W"]
+    a, b = max(1, (F - 1).bit_length()), (max(H, W) - 1).bit_length()
+    if F == 1:
+        cells = np.insert(_curve(b), 0, 0, axis=1)
+    elif a >= b:
+        cells = _curve3(a)
+    else:   # the plane in macro cells of 2^a x 2^a, the cube of all frames above each walked by the 3-D curve
+        cells = (np.insert(_curve(b - a) << a, 0, 0, axis=1)[:, None, :] + _curve3(a)[None]).reshape(-1, 3)
+    index = np.full(cells.max(0) + 1, -1, dtype=np.int64)
+    index[tuple(cells.T)] = np.arange(len(cells))
+    return index[:F, :H, :W], len(cells)
+
+
+def _order(c, layer):
+    """(physical position -> original token, prefix length, [physical positions of each tile's own tokens])."""
+    index, length = _curve_index(c)
+    shared = np.zeros(index.shape, dtype=bool)
+    s, f = c["shared"], c["shared_frames"] if c["frames"] > 1 else 1
+    f0, r0, c0 = c["frames"] // 2 - f // 2, c["H"] // 2 - s // 2, c["W"] // 2 - s // 2
+    shared[f0:f0 + f, r0:r0 + s, c0:c0 + s] = True
+    index, shared = index.ravel(), shared.ravel()
+    cells = np.lexsort((index, ~shared))    # shared ones first, each part along the curve
+    prefix = c["text"] + int(shared.sum())
+    tile = (index[cells[int(shared.sum()):]] + c["offset"] + layer * c["tile"] // 4) // c["tile"] % (length // c["tile"])
+    by_tile = np.argsort(tile, kind="stable")
+    cuts = np.flatnonzero(np.diff(tile[by_tile])) + 1
+    members = [prefix + m for m in np.split(by_tile, cuts) if len(m)]
+    return np.concatenate([np.arange(c["text"]), c["text"] + cells]), prefix, members
+
+
+def _attend(q, k, v, prefix, members, dout=None):
+    """Masked softmax attention on [units, S, D] in physical order: out, log-sum-exp and, with dout, dq, dk, dv."""
+    units, S, D = q.shape
+    out, lse = torch.empty_like(q), q.new_empty((units, S))
+    grads = [] if dout is None else [torch.zeros_like(q) for _ in range(3)]
+    # prefix rows see everything; the rows of a tile see the prefix and the tile
+    blocks = [(slice(0, prefix), slice(None))] if prefix else []
+    first = torch.arange(prefix, device=q.device)
+    for m in members:
+        m = torch.from_numpy(m).to(q.device)
+        blocks.append((m, torch.cat([first, m])))
+    for rows, keys in blocks:
+        n = prefix * S if isinstance(rows, slice) else len(rows) * len(keys)
+        some = max(1, int(2e8 / n))
+        for u in (slice(i, i + some) for i in range(0, units, some)):
+            qb, kb, vb = q[u][:, rows], k[u][:, keys], v[u][:, keys]
+            s = qb @ kb.transpose(1, 2) / math.sqrt(D)
+            l = torch.logsumexp(s, 2)
+            p = s.sub_(l[:, :, None]).exp_()
+            o = p @ vb
+            out[u, rows], lse[u, rows] = o, l
+            if dout is not None:
+                do = dout[u][:, rows]
+                grads[2][u, keys] += p.transpose(1, 2) @ do
+                ds = (do @ vb.transpose(1, 2) - (do * o).sum(2, keepdim=True)).mul_(p).div_(math.sqrt(D))
+                grads[0][u, rows] = ds @ kb
+                grads[1][u, keys] += ds.transpose(1, 2) @ qb
+    return [out, lse] + grads
+
+
+def exact(case, seed):
+    """What run() returns for these inputs, in 64 bits on the GPU (the largest takes a second or two)."""
+    c = case
+    if c["kind"] == "plan":
+        return None
+    qkv, dout = _inputs(c, seed)
+    S = qkv[0][0].shape[2]
+    results = []
+    for layer in range(c["layers"]):
+        order, prefix, members = _order(c, layer)
+        order = torch.from_numpy(order).to("cuda")
+        q, k, v = (t.double().reshape(-1, S, c["dim"]) for t in qkv[layer])
+        if c["kind"] != "train" and layer == 0:
+            q, k, v = (t[:, order] for t in (q, k, v))
+        if c["kind"] == "train":
+            got = _attend(q, k, v, prefix, members, dout.double().reshape(-1, S, c["dim"]))
+        else:
+            got = _attend(q, k, v, prefix, members)[:1]
+            if layer == c["layers"] - 1:
+                got = [torch.empty_like(got[0]).index_copy_(1, order, got[0])]
+        results += [t.reshape((c["batch"], c["heads"]) + t.shape[1:]) for t in got]
+    return results[0] if c["kind"] in ("fused", "host") else results
