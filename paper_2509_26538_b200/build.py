@@ -10,7 +10,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libhilberta.so")
 SOURCES = ["plan.cu", "schedule.cu", "permute.cu", "attn_fp32.cu", "attn_fp32_bwd.cu", "attn_bf16_sm100.cu", "attn_bf16_pair_sm100.cu", "attn_bf16_solo_sm100.cu", "attn_bwd_sm100.cu"]
-HEADERS = ["common.cuh", "sm100_ptx.cuh", "attn_softmax_math.cuh"]
+HEADERS = ["common.cuh", "sm100_ptx.cuh", "attn_softmax_math.cuh", "attn_fp32_tile.cuh"]
 
 
 def _newest_source() -> float:

@@ -1,141 +1,243 @@
-// fp32 forward for fp32 inputs: plain FMA arithmetic (no tensor cores, whose
-// fp32 modes round operands to tf32 and could not meet a 1e-5 tolerance).
-// One warp per query row; every lane runs its own online softmax over the keys
-// j = lane, lane + 32, ... of the row's key ranges, and the 32 partial states
-// are merged at the end.  Key ranges are those of Algorithm 1: the global prefix
-// plus the row's slid tile, or the whole sequence for prefix rows.
+// fp32 forward for fp32 inputs: online softmax over register-tiled products on the FMA pipes
+// (attn_fp32_tile.cuh).  A CTA owns 64 query rows that share a key list (Algorithm 1: the global prefix
+// plus the rows' slid tile, or the whole sequence for prefix rows) and walks it in blocks of 32 keys; the
+// next block's K and V tiles arrive (cp.async) while this block is worked on, and a block costs one barrier.
+// Bound: the FMA pipes and, next to them, shared memory.  Measured (B200): 32 x 32 + 64 tokens, 8 heads of 64,
+// forward + backward 1500 -> 190 us (16 TFLOP/s useful; one warp per query row with a key per lane before,
+// every lane reading whole rows of its own); 16 x 16 tokens, 2 heads of 64, 26 -> 10 us a call.
 #include <math.h>
 
-#include "common.cuh"
+#include <algorithm>
+#include <mutex>
+
+#include "attn_fp32_tile.cuh"
 
 namespace hilberta {
 
-constexpr int kRowsPerBlock = 4;
+using namespace fp32t;
+
+namespace {
 
 template <int D>
-__global__ void __launch_bounds__(kRowsPerBlock * 32)
+constexpr int fwd_smem() { return (res_floats(D) + 4 * blk_floats(D) + BR * PS + 2 * BR) * (int)sizeof(float); }
+
+template <int D>
+__global__ void __launch_bounds__(kThreads, D == 128 ? 2 : 3)
 attn_fp32_kernel(const float *__restrict__ q, const float *__restrict__ k, const float *__restrict__ v,
                  float *__restrict__ out, long long stride_b, long long stride_h, long long stride_s,
-                 int heads, int S, int P, const int *__restrict__ row_window,
-                 const Window *__restrict__ windows, const int *__restrict__ out_map,
-                 const int *__restrict__ in_map, float *__restrict__ lse, float scale) {
-    __shared__ float sq[kRowsPerBlock][D];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row = blockIdx.x * kRowsPerBlock + warp;
-    if (row >= S) return;  // whole warp leaves together; no block-wide barrier below
-    const int bh = blockIdx.y;
+                 int heads, int bhs, int S, const WorkItem *__restrict__ work, int n_items, int n_split, int cluster,
+                 const int *__restrict__ out_map, const int *__restrict__ in_map, float *__restrict__ lse, float scale) {
+    extern __shared__ float4 smem4[];
+    constexpr int C = D / 8;
+    float *sQ = reinterpret_cast<float *>(smem4), *sKV = sQ + res_floats(D);
+    float *sP = sKV + 4 * blk_floats(D), *sM = sP + BR * PS, *sL = sM + BR;
+    const Share share(n_items, n_split, cluster, bhs);
+    if (share.item < 0) return;
+    const WorkItem it = work[share.item];
+    const KeyList kl(it);
+    const int bh = share.column;
     const long long base = (long long)(bh / heads) * stride_b + (long long)(bh % heads) * stride_h;
+    const int nb = (kl.total + BC - 1) / BC;
+    const int j0 = (int)((long long)nb * share.rank / share.parts), j1 = (int)((long long)nb * (share.rank + 1) / share.parts);
+    const int lane = threadIdx.x & 31, rg = lane >> 3, cg = lane & 7;
+    const int wrow = (threadIdx.x >> 5) * 16 + rg;   // this lane's rows: wrow + 2 i
+
     // in_map: q, k, v are in original order and physical row p lives at row in_map[p]
-    const float *qrow = q + base + (long long)(in_map ? in_map[row] : row) * stride_s;
-    for (int d = lane; d < D; d += 32) sq[warp][d] = qrow[d];
-    __syncwarp();
-
-    int seg_start[3], seg_len[3], n_seg;
-    const int w = row_window[row];
-    if (w < 0) {
-        n_seg = 1;
-        seg_start[0] = 0;
-        seg_len[0] = S;
-    } else {
-        const Window win = windows[w];
-        n_seg = 3;
-        seg_start[0] = 0;
-        seg_len[0] = P;
-        seg_start[1] = win.seg0_start;
-        seg_len[1] = win.seg0_len;
-        seg_start[2] = win.seg1_start;
-        seg_len[2] = win.seg1_len;
+    load_rows<D>(sQ, q + base, stride_s, it.q_start, it.q_rows, in_map);
+    if (j0 < j1) {
+        load_block<D>(sKV, k + base, stride_s, kl, j0, in_map);
+        load_block<D>(sKV + blk_floats(D), v + base, stride_s, kl, j0, in_map);
     }
+    cp_commit();
 
-    float m = -INFINITY, l = 0.f;
-    float acc[D];
+    float m[4], l[4], o[4][C];
 #pragma unroll
-    for (int d = 0; d < D; ++d) acc[d] = 0.f;
+    for (int i = 0; i < 4; ++i) {
+        m[i] = -INFINITY;
+        l[i] = 0.f;
+#pragma unroll
+        for (int c = 0; c < C; ++c) o[i][c] = 0.f;
+    }
+    for (int j = j0; j < j1; ++j) {
+        const float *sK = sKV + ((j - j0) & 1) * 2 * blk_floats(D), *sV = sK + blk_floats(D);
+        cp_wait<0>();
+        __syncthreads();     // this block's tiles are in, and every warp is done with the other pair
+        if (j + 1 < j1) {
+            float *nK = sKV + ((j + 1 - j0) & 1) * 2 * blk_floats(D);
+            load_block<D>(nK, k + base, stride_s, kl, j + 1, in_map);
+            load_block<D>(nK + blk_floats(D), v + base, stride_s, kl, j + 1, in_map);
+        }
+        cp_commit();
+        float x[4][4];
+        dot_tile<D>(x, sQ + wrow * (D + 4), sK + cg * (D + 4));
+        const int valid = kl.total - j * BC;   // >= 1
+        float corr[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float mx = -INFINITY;
+#pragma unroll
+            for (int jj = 0; jj < 4; ++jj) {
+                x[i][jj] = 8 * jj + cg < valid ? x[i][jj] * scale : -INFINITY;
+                mx = fmaxf(mx, x[i][jj]);
+            }
+#pragma unroll
+            for (int off = 4; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+            const float mn = fmaxf(m[i], mx);
+            corr[i] = m[i] == mn ? 1.f : expf(m[i] - mn);   // exp(-inf) = 0 on the first block
+            m[i] = mn;
+            float sum = 0.f;
+#pragma unroll
+            for (int jj = 0; jj < 4; ++jj) {
+                const float p = 8 * jj + cg < valid ? expf(x[i][jj] - mn) : 0.f;
+                sP[(wrow + 4 * i) * PS + 8 * jj + cg] = p;
+                sum += p;
+            }
+            l[i] = fmaf(l[i], corr[i], sum);   // this lane's share of the row sum
+        }
+        __syncwarp();        // a warp's weights stay within the warp
+        acc_tile<D>(o, corr, sP + wrow * PS, sV, cg);
+        __syncwarp();
+    }
+    cp_wait<0>();
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], off);
 
-    for (int s = 0; s < n_seg; ++s) {
-        const int end = seg_start[s] + seg_len[s];
-        for (int j = seg_start[s] + lane; j < end; j += 32) {
-            const long long jrow = in_map ? in_map[j] : j;
-            const float4 *kj = reinterpret_cast<const float4 *>(k + base + jrow * stride_s);
-            float dot = 0.f;
+    if (share.parts == 1) {
 #pragma unroll
-            for (int d4 = 0; d4 < D / 4; ++d4) {
-                const float4 kk = __ldg(kj + d4);
-                dot = fmaf(sq[warp][4 * d4 + 0], kk.x, dot);
-                dot = fmaf(sq[warp][4 * d4 + 1], kk.y, dot);
-                dot = fmaf(sq[warp][4 * d4 + 2], kk.z, dot);
-                dot = fmaf(sq[warp][4 * d4 + 3], kk.w, dot);
-            }
-            const float x = dot * scale;
-            if (x > m) {
-                const float corr = expf(m - x);  // exp(-inf) = 0 on the first key
-                l *= corr;
+        for (int i = 0; i < 4; ++i) {
+            const int r = wrow + 4 * i;
+            if (r >= it.q_rows) continue;
+            const int out_row = out_map ? out_map[it.q_start + r] : it.q_start + r;   // optional fused exit scatter
+            const float inv = 1.f / l[i];
 #pragma unroll
-                for (int d = 0; d < D; ++d) acc[d] *= corr;
-                m = x;
-            }
-            const float p = expf(x - m);
-            l += p;
-            const float4 *vj = reinterpret_cast<const float4 *>(v + base + jrow * stride_s);
+            for (int c = 0; c < C; ++c) o[i][c] *= inv;
+            store_cols<D>(out + base + (long long)out_row * stride_s, cg, o[i]);
+            if (lse && cg == 0) lse[(long long)bh * S + out_row] = m[i] + logf(l[i]);
+        }
+        return;
+    }
+    // Merge of the cluster's partial states: every CTA leaves (m, l, O) of its share in shared memory,
+    // rank c writes rows [64 c / parts, 64 (c + 1) / parts).
+    __syncthreads();
+    float *sO = sKV;   // 64 rows take the space of two K / V tiles
 #pragma unroll
-            for (int d4 = 0; d4 < D / 4; ++d4) {
-                const float4 vv = __ldg(vj + d4);
-                acc[4 * d4 + 0] = fmaf(p, vv.x, acc[4 * d4 + 0]);
-                acc[4 * d4 + 1] = fmaf(p, vv.y, acc[4 * d4 + 1]);
-                acc[4 * d4 + 2] = fmaf(p, vv.z, acc[4 * d4 + 2]);
-                acc[4 * d4 + 3] = fmaf(p, vv.w, acc[4 * d4 + 3]);
-            }
+    for (int i = 0; i < 4; ++i) {
+        const int r = wrow + 4 * i;
+        store_cols<D>(sO + r * (D + 4), cg, o[i]);
+        if (cg == 0) {
+            sM[r] = m[i];
+            sL[r] = l[i];
         }
     }
-
-    // merge the 32 lane states
-    float m_all = m;
+    cluster_sync();
+    const int rows = BR / share.parts, r0 = rows * share.rank;
+    for (int e = threadIdx.x; e < rows * (D / 4); e += kThreads) {
+        const int r = r0 + e / (D / 4), c4 = e % (D / 4);
+        if (r >= it.q_rows) continue;
+        // all loads of a CTA pair's states are in flight together (parts <= 8)
+        float mp[8], lp[8];
+        float4 y[8];
+        float m_all = -INFINITY;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xffffffffu, m_all, off));
-    const float f = (m == -INFINITY) ? 0.f : expf(m - m_all);
-    l *= f;
+        for (int p = 0; p < 8; ++p)
+            if (p < share.parts) {
+                mp[p] = peer_ld(peer_addr(sM + r, p));
+                lp[p] = peer_ld(peer_addr(sL + r, p));
+                y[p] = peer_ld4(peer_addr(sO + r * (D + 4) + 4 * c4, p));
+            }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
-    const float inv = 1.f / l;
-    float mine[D / 32];
+        for (int p = 0; p < 8; ++p)
+            if (p < share.parts) m_all = fmaxf(m_all, mp[p]);
+        float l_all = 0.f;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int d = 0; d < D; ++d) {
-        float a = acc[d] * f;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-        if ((d & 31) == lane) mine[d >> 5] = a * inv;
+        for (int p = 0; p < 8; ++p)
+            if (p < share.parts) {
+                const float w = mp[p] == m_all ? 1.f : expf(mp[p] - m_all);   // a share of no blocks has m = -inf
+                l_all = fmaf(lp[p], w, l_all);
+                acc.x = fmaf(y[p].x, w, acc.x);
+                acc.y = fmaf(y[p].y, w, acc.y);
+                acc.z = fmaf(y[p].z, w, acc.z);
+                acc.w = fmaf(y[p].w, w, acc.w);
+            }
+        const float inv = 1.f / l_all;
+        const int out_row = out_map ? out_map[it.q_start + r] : it.q_start + r;
+        *reinterpret_cast<float4 *>(out + base + (long long)out_row * stride_s + 4 * c4) =
+            make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+        if (lse && c4 == 0) lse[(long long)bh * S + out_row] = m_all + logf(l_all);
     }
-    const int out_row = out_map ? out_map[row] : row;  // optional fused exit scatter
-    float *orow = out + base + (long long)out_row * stride_s;
-    if (lse && lane == 0) lse[(long long)bh * S + out_row] = m_all + logf(l);
-#pragma unroll
-    for (int i = 0; i < D / 32; ++i) orow[i * 32 + lane] = mine[i];
+    cluster_sync();   // no CTA leaves while a peer may still read its shared memory
+}
+
+}  // namespace
+
+// Work list of the fp32 kernels: items of 64 rows, longest key lists first, all of more than two blocks
+// cut over clusters of up to 8 CTAs as long as that leaves no SM more than a few CTAs.  Prefix rows see the
+// whole sequence, and on the problems this path serves a handful of them would otherwise outlast everything
+// else (and a small problem would leave most SMs idle); every cut costs each CTA its start and a merge.  The
+// bounds are read off sweeps on the B200 (us; clusters of 1 / 2 / 4 / 8): 32 x 32 + 64 tokens, 8 heads of
+// 64, forward + backward (19 items) 340 / 205 / 190 / 244; 32 x 32 + 226, 4 heads of 64 (21) 411 / 253 / 207 /
+// 212; 16 x 16, 2 heads of 64, forward (5) 32 / 20 / 13 / 11; 25 x 34 + 333, 6 heads of 32 (19) 373 / 261 / 291 /
+// 278; 16 x 16 + 128, 16 heads of 128 (7) 235 / 166 / 187 / 236; 35 x 35 + 77, 13 heads of 128 (23) 343 / 350 /
+// 339 / 397.
+int attn_fp32_prepare(hilberta_plan_t *p) {
+    std::vector<WorkItem> items = build_work_items(p, BR, BC);
+    const int rc = check_work_items(items.data(), (int)items.size(), p->S, BR, BC);
+    if (rc != HILBERTA_OK) return rc;
+    auto blocks = [](const WorkItem &it) {
+        long long n = 0;
+        for (int s = 0; s < it.n_seg; ++s) n += it.seg_len[s];
+        return (n + BC - 1) / BC;   // the kernels read the ranges as one list
+    };
+    std::stable_sort(items.begin(), items.end(), [&](const WorkItem &a, const WorkItem &b) { return blocks(a) > blocks(b); });
+    const long long instances = (long long)items.size() * p->batch * p->heads;
+    const long long most = (long long)p->sm_count * (p->head_dim == 64 ? 9 : 6) / 2;
+    p->f32_cluster = 1;
+    while (p->f32_cluster < 8 && instances * p->f32_cluster * 2 <= most) p->f32_cluster *= 2;
+    p->n_f32_split = 0;
+    if (p->f32_cluster > 1)
+        while (p->n_f32_split < (int)items.size() && blocks(items[p->n_f32_split]) > 2) ++p->n_f32_split;
+    p->n_f32_work = (int)items.size();
+    cudaFree(p->d_f32_work);
+    p->d_f32_work = nullptr;
+    if (items.empty()) return HILBERTA_OK;
+    HB_CUDA(cudaMalloc(&p->d_f32_work, sizeof(WorkItem) * items.size()));
+    HB_CUDA(cudaMemcpy(p->d_f32_work, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice));
+    // the shared-memory opt-in is an attribute of the kernel on one device
+    static std::mutex attr_mutex;
+    static bool attr_done[64] = {};
+    std::lock_guard<std::mutex> lock(attr_mutex);
+    if (p->device < 0 || p->device >= 64) return HILBERTA_ERR_INVALID;
+    if (!attr_done[p->device]) {
+        HB_CUDA(cudaFuncSetAttribute(attn_fp32_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, fwd_smem<32>()));
+        HB_CUDA(cudaFuncSetAttribute(attn_fp32_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, fwd_smem<64>()));
+        HB_CUDA(cudaFuncSetAttribute(attn_fp32_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, fwd_smem<128>()));
+        const int rc_bwd = attn_fp32_bwd_opt_in();
+        if (rc_bwd != HILBERTA_OK) return rc_bwd;
+        attr_done[p->device] = true;
+    }
+    return HILBERTA_OK;
 }
 
 int launch_attn_fp32(const hilberta_plan_t *p, const void *q, const void *k, const void *v, void *out,
                      float *lse, const int *out_map, const int *in_map, cudaStream_t stream, int chunk) {
     const uintptr_t bits = (uintptr_t)q | (uintptr_t)k | (uintptr_t)v | (uintptr_t)out;
     if ((bits & 15) || ((p->stride_b | p->stride_h | p->stride_s) & 3)) return HILBERTA_ERR_INVALID;
-    int heads = p->heads;
-    if (chunk >= 0) {
-        // a slice of heads: same strides, shifted base pointers
-        if (lse) return HILBERTA_ERR_INVALID;
-        heads = p->chunk_heads;
-        const long long off = (long long)chunk * heads * p->stride_h;
-        q = (const float *)q + off;
-        k = (const float *)k + off;
-        v = (const float *)v + off;
-        out = (float *)out + off;
+    if (chunk >= 0) return HILBERTA_ERR_INVALID;   // fp32 bindings have no slices of heads
+    if (p->n_f32_work == 0) return HILBERTA_OK;
+#define HB_FP32_CASE(DD)                                                                                              \
+    case DD: {                                                                                                        \
+        const ClusterLaunch cfg(p, fwd_smem<DD>(), 1, stream);                                                        \
+        if (cfg.ctas > 0x7fffffffll) return HILBERTA_ERR_INVALID;                                                     \
+        HB_CUDA(cudaLaunchKernelEx(&cfg.config, attn_fp32_kernel<DD>, (const float *)q, (const float *)k,             \
+                                   (const float *)v, (float *)out, (long long)p->stride_b, (long long)p->stride_h,    \
+                                   (long long)p->stride_s, p->heads, p->batch * p->heads, p->S,                       \
+                                   (const WorkItem *)p->d_f32_work,                                                   \
+                                   p->n_f32_work, p->n_f32_split, p->f32_cluster, out_map, in_map, lse, p->scale));   \
+        break;                                                                                                        \
     }
-    dim3 grid((p->S + kRowsPerBlock - 1) / kRowsPerBlock, p->batch * heads);
-    dim3 block(kRowsPerBlock * 32);
-#define HB_FP32_CASE(DD)                                                                              \
-    case DD:                                                                                          \
-        attn_fp32_kernel<DD><<<grid, block, 0, stream>>>(                                             \
-            (const float *)q, (const float *)k, (const float *)v, (float *)out, p->stride_b,          \
-            p->stride_h, p->stride_s, heads, p->S, p->P, p->d_row_window, p->d_windows, out_map, in_map,   \
-            lse, p->scale);                                                                                \
-        break;
     switch (p->head_dim) {
         HB_FP32_CASE(32)
         HB_FP32_CASE(64)

@@ -1,27 +1,29 @@
-// fp32 backward for fp32 inputs: plain FMA arithmetic, the counterpart of attn_fp32.cu (the
+// fp32 backward for fp32 inputs on register-tiled FMA products, the counterpart of attn_fp32.cu (the
 // paper trains through its kernel, Sec. 4.1, without describing the backward pass; this is the
-// derivative of Algorithm 1's result).  One warp per resident row; the 32 lanes split the head
-// dimension, so every dot product is a warp reduction and every accumulator is D / 32 registers.
-//   mode 0: resident = query row i;  for the keys j it sees:  dq_i += dS_ij k_j
-//   mode 1: resident = key row j;    for the queries i that see it (the same ranges, the mask
+// derivative of Algorithm 1's result).  One launch holds both directions:
+//   mode 0: resident = 64 query rows;  over the keys they see:  dq_i += dS_ij k_j
+//   mode 1: resident = 64 key rows;    over the queries that see them (the same ranges, the mask
 //           being symmetric):  dk_j += dS_ij q_i,  dv_j += P_ij dO_i
-// with P_ij = exp(s q_i.k_j - lse_i), dS_ij = P_ij (dO_i.v_j - delta_i).  Not a performance target.
+// with P_ij = exp(s q_i.k_j - lse_i), dS_ij = P_ij (dO_i.v_j - delta_i).  Nothing is accumulated across
+// CTAs but through a cluster's shared memory in rank order, so results are bit-reproducible.
 #include <math.h>
 
-#include "common.cuh"
+#include "attn_fp32_tile.cuh"
 
 namespace hilberta {
 
+using namespace fp32t;
+
 namespace {
 
-constexpr int kRowsPerBlock = 4;
+constexpr int kDeltaRows = 4;
 
 template <int D>
-__global__ void __launch_bounds__(kRowsPerBlock * 32)
+__global__ void __launch_bounds__(kDeltaRows * 32)
 delta_fp32_kernel(const float *__restrict__ dout, const float *__restrict__ out, float *__restrict__ delta,
                   long long stride_b, long long stride_h, long long stride_s, int heads, int S) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row = blockIdx.x * kRowsPerBlock + warp;
+    const int row = blockIdx.x * kDeltaRows + warp;
     if (row >= S) return;
     const int bh = blockIdx.y;
     const long long off = (long long)(bh / heads) * stride_b + (long long)(bh % heads) * stride_h +
@@ -34,109 +36,198 @@ delta_fp32_kernel(const float *__restrict__ dout, const float *__restrict__ out,
     if (lane == 0) delta[(long long)bh * S + row] = acc;
 }
 
-template <int D, int MODE>
-__global__ void __launch_bounds__(kRowsPerBlock * 32)
-attn_fp32_bwd_kernel(const float *__restrict__ q, const float *__restrict__ k, const float *__restrict__ v,
-                     const float *__restrict__ dout, const float *__restrict__ lse, const float *__restrict__ delta,
-                     float *__restrict__ out_a, float *__restrict__ out_b, long long stride_b, long long stride_h,
-                     long long stride_s, int heads, int S, int P, const int *__restrict__ row_window,
-                     const Window *__restrict__ windows, float scale) {
-    constexpr int E = D / 32;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row = blockIdx.x * kRowsPerBlock + warp;
-    if (row >= S) return;
-    const int bh = blockIdx.y;
-    const long long base = (long long)(bh / heads) * stride_b + (long long)(bh % heads) * stride_h;
-    const float *r1 = (MODE == 0 ? q : k) + base + (long long)row * stride_s;
-    const float *r2 = (MODE == 0 ? dout : v) + base + (long long)row * stride_s;
-    const float *t1 = (MODE == 0 ? k : q) + base;      // streamed operand of the scores
-    const float *t2 = (MODE == 0 ? v : dout) + base;   // streamed operand of dP
-    float a1[E], a2[E], accA[E], accB[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        a1[e] = r1[lane + 32 * e];
-        a2[e] = r2[lane + 32 * e];
-        accA[e] = 0.f;
-        accB[e] = 0.f;
-    }
-    const float row_lse = lse[(long long)bh * S + row], row_delta = delta[(long long)bh * S + row];
+// pairs of streamed tiles in shared memory: two where two CTAs of that size fit an SM, one at head dim 128
+// (145 KB with two; at head dim 64 one pair and three CTAs measured equal, 0.5 % behind)
+__host__ __device__ constexpr int stages(int D) { return D == 128 ? 1 : 2; }
+template <int D>
+constexpr int bwd_smem() { return (2 * res_floats(D) + 2 * stages(D) * blk_floats(D) + BR * PS) * (int)sizeof(float); }
 
-    int seg_start[3], seg_len[3], n_seg;
-    const int w = row_window[row];
-    if (w < 0) {
-        n_seg = 1;
-        seg_start[0] = 0;
-        seg_len[0] = S;
-    } else {
-        const Window win = windows[w];
-        n_seg = 3;
-        seg_start[0] = 0;
-        seg_len[0] = P;
-        seg_start[1] = win.seg0_start;
-        seg_len[1] = win.seg0_len;
-        seg_start[2] = win.seg1_start;
-        seg_len[2] = win.seg1_len;
+// One mode for one CTA.  r1 / t1: resident and streamed operand of the scores, r2 / t2: of dP.
+template <int D, int MODE>
+__device__ __forceinline__ void bwd_tile(const float *r1, const float *r2, const float *t1, const float *t2,
+                                         const float *lse, const float *delta, float *out_a, float *out_b,
+                                         long long stride_s, const WorkItem &it, const Share &share, float scale) {
+    extern __shared__ float4 smem4[];
+    constexpr int C = D / 8;
+    float *sR1 = reinterpret_cast<float *>(smem4), *sR2 = sR1 + res_floats(D), *sT = sR2 + res_floats(D);
+    float *sP = sT + 2 * stages(D) * blk_floats(D);
+    const KeyList kl(it);
+    const int nb = (kl.total + BC - 1) / BC;
+    const int j0 = (int)((long long)nb * share.rank / share.parts), j1 = (int)((long long)nb * (share.rank + 1) / share.parts);
+    const int lane = threadIdx.x & 31, rg = lane >> 3, cg = lane & 7;
+    const int wrow = (threadIdx.x >> 5) * 16 + rg;
+
+    load_rows<D>(sR1, r1, stride_s, it.q_start, it.q_rows, nullptr);
+    load_rows<D>(sR2, r2, stride_s, it.q_start, it.q_rows, nullptr);
+    float row_lse[4], row_delta[4];
+    float a[4][C], b[4][C];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int r = wrow + 4 * i;
+        row_lse[i] = MODE == 0 && r < it.q_rows ? lse[it.q_start + r] : 0.f;
+        row_delta[i] = MODE == 0 && r < it.q_rows ? delta[it.q_start + r] : 0.f;
+#pragma unroll
+        for (int c = 0; c < C; ++c) a[i][c] = b[i][c] = 0.f;
     }
-    for (int s = 0; s < n_seg; ++s) {
-        const int end = seg_start[s] + seg_len[s];
-        for (int j = seg_start[s]; j < end; ++j) {
-            const float *x1 = t1 + (long long)j * stride_s, *x2 = t2 + (long long)j * stride_s;
-            float b1[E], b2[E];
-            float dot1 = 0.f, dot2 = 0.f;
+    const float one[4] = {1.f, 1.f, 1.f, 1.f};
+    auto load = [&](int j, float *dst) {
+        load_block<D>(dst, t1, stride_s, kl, j, nullptr);
+        load_block<D>(dst + blk_floats(D), t2, stride_s, kl, j, nullptr);
+    };
+    if (j0 < j1) load(j0, sT);
+    cp_commit();
+    for (int j = j0; j < j1; ++j) {
+        const float *sT1 = sT + ((j - j0) % stages(D)) * 2 * blk_floats(D), *sT2 = sT1 + blk_floats(D);
+        const int valid = kl.total - j * BC;   // >= 1
+        // the statistics belong to the QUERY of the pair: the streamed row in mode 1
+        float col_lse[4], col_delta[4];
+        if (MODE == 1) {
 #pragma unroll
-            for (int e = 0; e < E; ++e) {
-                b1[e] = __ldg(x1 + lane + 32 * e);
-                b2[e] = __ldg(x2 + lane + 32 * e);
-                dot1 = fmaf(a1[e], b1[e], dot1);
-                dot2 = fmaf(a2[e], b2[e], dot2);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                dot1 += __shfl_xor_sync(0xffffffffu, dot1, o);
-                dot2 += __shfl_xor_sync(0xffffffffu, dot2, o);
-            }
-            // the statistics belong to the QUERY of the pair
-            const float l = MODE == 0 ? row_lse : __ldg(lse + (long long)bh * S + j);
-            const float dl = MODE == 0 ? row_delta : __ldg(delta + (long long)bh * S + j);
-            const float p = expf(fmaf(dot1, scale, -l));
-            const float ds = p * (dot2 - dl);
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                accA[e] = fmaf(ds, b1[e], accA[e]);                   // dq += dS k   |  dk += dS q
-                if (MODE == 1) accB[e] = fmaf(p, b2[e], accB[e]);     //              |  dv += P dO
+            for (int jj = 0; jj < 4; ++jj) {
+                const int row = kl.row(8 * jj + cg < valid ? j * BC + 8 * jj + cg : 0);
+                col_lse[jj] = __ldg(lse + row);
+                col_delta[jj] = __ldg(delta + row);
             }
         }
-    }
-    float *oa = out_a + base + (long long)row * stride_s;
+        cp_wait<0>();
+        __syncthreads();   // this block's tiles are in, and every warp is done with the other pair
+        if (stages(D) == 2) {
+            if (j + 1 < j1) load(j + 1, sT + ((j + 1 - j0) % stages(D)) * 2 * blk_floats(D));
+            cp_commit();
+        }
+        float p[4][4];
+        dot_tile<D>(p, sR1 + wrow * (D + 4), sT1 + cg * (D + 4));
 #pragma unroll
-    for (int e = 0; e < E; ++e) oa[lane + 32 * e] = accA[e] * scale;
-    if (MODE == 1) {
-        float *ob = out_b + base + (long long)row * stride_s;
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int e = 0; e < E; ++e) ob[lane + 32 * e] = accB[e];
+            for (int jj = 0; jj < 4; ++jj)
+                p[i][jj] = 8 * jj + cg < valid ? expf(fmaf(p[i][jj], scale, -(MODE == 0 ? row_lse[i] : col_lse[jj]))) : 0.f;
+        float ds[4][4];
+        dot_tile<D>(ds, sR2 + wrow * (D + 4), sT2 + cg * (D + 4));
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int jj = 0; jj < 4; ++jj)   // beyond the list P is zero and the streamed rows and statistics are any
+                ds[i][jj] = 8 * jj + cg < valid ? p[i][jj] * (ds[i][jj] - (MODE == 0 ? row_delta[i] : col_delta[jj])) : 0.f;
+        if (MODE == 1) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int jj = 0; jj < 4; ++jj) sP[(wrow + 4 * i) * PS + 8 * jj + cg] = p[i][jj];
+            __syncwarp();
+            acc_tile<D>(b, one, sP + wrow * PS, sT2, cg);   // dv += P dO
+            __syncwarp();
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int jj = 0; jj < 4; ++jj) sP[(wrow + 4 * i) * PS + 8 * jj + cg] = ds[i][jj];
+        __syncwarp();
+        acc_tile<D>(a, one, sP + wrow * PS, sT1, cg);       // dq += dS k  |  dk += dS q
+        if (stages(D) == 1) {
+            __syncthreads();   // the streamed tiles are free
+            if (j + 1 < j1) load(j + 1, sT);
+            cp_commit();
+        } else {
+            __syncwarp();
+        }
     }
+    cp_wait<0>();
+    if (share.parts == 1) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = wrow + 4 * i;
+            if (r >= it.q_rows) continue;
+#pragma unroll
+            for (int c = 0; c < C; ++c) a[i][c] *= scale;
+            store_cols<D>(out_a + (long long)(it.q_start + r) * stride_s, cg, a[i]);
+            if (MODE == 1) store_cols<D>(out_b + (long long)(it.q_start + r) * stride_s, cg, b[i]);
+        }
+        return;
+    }
+    // sum of the cluster's shares, in rank order; rank c writes rows [64 c / parts, 64 (c + 1) / parts)
+    // (the resident tiles' space holds them)
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        store_cols<D>(sR1 + (wrow + 4 * i) * (D + 4), cg, a[i]);
+        if (MODE == 1) store_cols<D>(sR2 + (wrow + 4 * i) * (D + 4), cg, b[i]);
+    }
+    cluster_sync();
+    const int rows = BR / share.parts, r0 = rows * share.rank;
+    for (int e = threadIdx.x; e < (MODE + 1) * rows * (D / 4); e += kThreads) {
+        const bool second = e >= rows * (D / 4);
+        const int f = second ? e - rows * (D / 4) : e;
+        const int r = r0 + f / (D / 4), c4 = f % (D / 4);
+        if (r >= it.q_rows) continue;
+        const float *src = (second ? sR2 : sR1) + r * (D + 4) + 4 * c4;
+        float4 y[8];
+#pragma unroll
+        for (int p = 0; p < 8; ++p)
+            if (p < share.parts) y[p] = peer_ld4(peer_addr(src, p));
+        float4 acc = y[0];
+#pragma unroll
+        for (int p = 1; p < 8; ++p)
+            if (p < share.parts) {
+                acc.x += y[p].x;
+                acc.y += y[p].y;
+                acc.z += y[p].z;
+                acc.w += y[p].w;
+            }
+        const float f4 = second ? 1.f : scale;
+        *reinterpret_cast<float4 *>((second ? out_b : out_a) + (long long)(it.q_start + r) * stride_s + 4 * c4) =
+            make_float4(acc.x * f4, acc.y * f4, acc.z * f4, acc.w * f4);
+    }
+    cluster_sync();   // no CTA leaves while a peer may still read its shared memory
+}
+
+template <int D>
+__global__ void __launch_bounds__(kThreads, D == 128 ? 1 : 2)
+attn_fp32_bwd_kernel(const float *__restrict__ q, const float *__restrict__ k, const float *__restrict__ v,
+                     const float *__restrict__ dout, const float *__restrict__ lse, const float *__restrict__ delta,
+                     float *__restrict__ dq, float *__restrict__ dk, float *__restrict__ dv, long long stride_b,
+                     long long stride_h, long long stride_s, int heads, int bhs, int S, const WorkItem *__restrict__ work,
+                     int n_items, int n_split, int cluster, float scale) {
+    const Share share(n_items, n_split, cluster, 2 * bhs);
+    if (share.item < 0) return;
+    const WorkItem it = work[share.item];
+    const bool keys = share.column < bhs;   // the direction with more work per pair first
+    const int bh = keys ? share.column : share.column - bhs;
+    const long long base = (long long)(bh / heads) * stride_b + (long long)(bh % heads) * stride_h;
+    lse += (long long)bh * S;
+    delta += (long long)bh * S;
+    if (keys)
+        bwd_tile<D, 1>(k + base, v + base, q + base, dout + base, lse, delta, dk + base, dv + base, stride_s, it, share, scale);
+    else
+        bwd_tile<D, 0>(q + base, dout + base, k + base, v + base, lse, delta, dq + base, nullptr, stride_s, it, share, scale);
 }
 
 template <int D>
 int launch(const hilberta_plan_t *p, const float *dout, const float *q, const float *k, const float *v,
            const float *out, const float *lse, float *dq, float *dk, float *dv, float *delta, cudaStream_t stream) {
-    dim3 grid((p->S + kRowsPerBlock - 1) / kRowsPerBlock, p->batch * p->heads);
-    dim3 block(kRowsPerBlock * 32);
-    delta_fp32_kernel<D><<<grid, block, 0, stream>>>(dout, out, delta, p->stride_b, p->stride_h, p->stride_s, p->heads,
-                                                     p->S);
+    if (p->n_f32_work == 0) return HILBERTA_OK;
+    dim3 grid((p->S + kDeltaRows - 1) / kDeltaRows, p->batch * p->heads);
+    delta_fp32_kernel<D><<<grid, kDeltaRows * 32, 0, stream>>>(dout, out, delta, p->stride_b, p->stride_h, p->stride_s,
+                                                               p->heads, p->S);
     HB_LAUNCHED();
-    attn_fp32_bwd_kernel<D, 0><<<grid, block, 0, stream>>>(q, k, v, dout, lse, delta, dq, nullptr, p->stride_b,
-                                                           p->stride_h, p->stride_s, p->heads, p->S, p->P,
-                                                           p->d_row_window, p->d_windows, p->scale);
-    HB_LAUNCHED();
-    attn_fp32_bwd_kernel<D, 1><<<grid, block, 0, stream>>>(q, k, v, dout, lse, delta, dk, dv, p->stride_b,
-                                                           p->stride_h, p->stride_s, p->heads, p->S, p->P,
-                                                           p->d_row_window, p->d_windows, p->scale);
+    const ClusterLaunch cfg(p, bwd_smem<D>(), 2, stream);
+    if (cfg.ctas > 0x7fffffffll) return HILBERTA_ERR_INVALID;
+    HB_CUDA(cudaLaunchKernelEx(&cfg.config, attn_fp32_bwd_kernel<D>, q, k, v, dout, lse, (const float *)delta, dq, dk, dv,
+                               (long long)p->stride_b, (long long)p->stride_h, (long long)p->stride_s, p->heads,
+                               p->batch * p->heads, p->S,
+                               (const WorkItem *)p->d_f32_work, p->n_f32_work, p->n_f32_split, p->f32_cluster, p->scale));
     HB_LAUNCHED();
     return HILBERTA_OK;
 }
 
 }  // namespace
+
+int attn_fp32_bwd_opt_in() {
+    HB_CUDA(cudaFuncSetAttribute(attn_fp32_bwd_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, bwd_smem<32>()));
+    HB_CUDA(cudaFuncSetAttribute(attn_fp32_bwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, bwd_smem<64>()));
+    HB_CUDA(cudaFuncSetAttribute(attn_fp32_bwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, bwd_smem<128>()));
+    return HILBERTA_OK;
+}
 
 int launch_attn_fp32_bwd(const hilberta_plan_t *p, const void *dout, const void *q, const void *k, const void *v,
                          const void *out, const float *lse, void *dq, void *dk, void *dv, float *delta,

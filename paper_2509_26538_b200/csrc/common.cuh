@@ -116,6 +116,10 @@ struct hilberta_plan_s {
     int *d_bwd_cta_begin;
     int n_bwd_cta;
     float *d_delta;               // [batch * heads * S]
+    // fp32 bindings: items of 64 rows by descending key count; the first n_f32_split of them are cut over
+    // clusters of f32_cluster CTAs
+    hilberta::WorkItem *d_f32_work;
+    int n_f32_work, n_f32_split, f32_cluster;
     int *d_status;  // [4] error word + diagnostics written by bounded waits
     // workspace of hilberta_forward_host
     void *ws;
@@ -167,6 +171,8 @@ int launch_attn_bwd(const hilberta_plan_t *p, const void *dout, const void *q, c
 int launch_attn_fp32_bwd(const hilberta_plan_t *p, const void *dout, const void *q, const void *k, const void *v,
                          const void *out, const float *lse, void *dq, void *dk, void *dv, float *delta,
                          cudaStream_t stream);
+int attn_fp32_prepare(hilberta_plan_t *p);
+int attn_fp32_bwd_opt_in();   // shared-memory opt-in of the fp32 backward kernels on the current device
 int launch_timeout_probe(const hilberta_plan_t *p, cudaStream_t stream);
 // plan.cu: does a written tensor share a byte with another tensor of the bound layout?
 bool bound_tensors_overlap(const hilberta_plan_t *p, const void *out, size_t esz_out, const void *in, size_t esz_in);

@@ -301,6 +301,7 @@ static void free_plan(hilberta_plan_t *p) {
     cudaFree(p->d_bwd_units);
     cudaFree(p->d_bwd_cta_begin);
     cudaFree(p->d_delta);
+    cudaFree(p->d_f32_work);
     cudaFree(p->d_status);
     cudaFree(p->ws);
     delete p;
@@ -617,6 +618,8 @@ extern "C" int hilberta_plan_bind(hilberta_plan_t *p, int batch, int heads, int 
         cudaFree(p->d_delta);
         p->d_delta = nullptr;
         HB_CUDA(cudaMalloc(&p->d_delta, sizeof(float) * 2 * (size_t)batch * heads * p->S));
+        const int rc = attn_fp32_prepare(p);
+        if (rc != HILBERTA_OK) return rc;
     }
     p->bound = true;
     return HILBERTA_OK;
