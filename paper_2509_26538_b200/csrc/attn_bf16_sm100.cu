@@ -65,9 +65,16 @@ constexpr int SLAB_BYTES = BN * 128;     // one 64-column slab of 128 rows (128-
 // e4m3 (fp8 = true), HD = 128: rows of 128 bytes, one slab.
 __host__ __device__ constexpr int tile_bytes(int hd, bool fp8 = false) { return BN * hd * (fp8 ? 1 : 2); }
 constexpr int THREADS = 384;   // 8 softmax warps + producer + MMA issuer + 2 idle (register donors)
-__host__ __device__ constexpr int smem_bytes(int hd, bool fp8 = false, bool gather = false) {
-    return (QT + ring_slots(gather, hd, fp8)) * tile_bytes(hd, fp8) + (gather ? 0 : STAGE_BYTES) + 1024;
+// Tiles of one CTA.  A split unit's partial state (256 rows of head-dim fp32 sums and their statistics)
+// takes the space of the tiles once they are read, and a little more than that with e4m3 tiles.
+__host__ __device__ constexpr int tile_area(int hd, bool fp8, bool gather, bool split) {
+    const int tiles = (QT + ring_slots(gather, hd, fp8)) * tile_bytes(hd, fp8), part = ITEM_ROWS * (hd * 4 + 16);
+    return split && part > tiles ? part : tiles;
 }
+__host__ __device__ constexpr int smem_bytes(int hd, bool fp8 = false, bool gather = false, bool split = false) {
+    return tile_area(hd, fp8, gather, split) + (gather ? 0 : STAGE_BYTES) + 1024;
+}
+constexpr int SPLIT_UNIT = -2;   // WorkUnit::bh2 of a unit that the CTAs of a cluster share
 constexpr uint32_t TMEM_COLS = 512;
 constexpr float RESCALE_THRESHOLD = 8.0f;        // log2 units
 // e4m3 weights: the running maximum may lag by 2^4 and every weight carries a factor 2^4 (divided
@@ -97,7 +104,10 @@ enum Bar {
     P_READY = S_FULL + QT,        // [t * 2 + part]: P columns of the keys of that part written, 128 arrivals
     PV_DONE = P_READY + 2 * QT,
     KV_FULL = PV_DONE + QT, KV_EMPTY = KV_FULL + NSTAGE,
-    NUM_BARS = KV_EMPTY + NSTAGE
+    // split units: every MMA of this CTA's share has retired; [t]: tile t's partial states of the whole
+    // cluster are in shared memory (4 warps per CTA); they have been read (8 warps per CTA)
+    UNIT_MMA = KV_EMPTY + NSTAGE, PART_READY, PART_READ = PART_READY + QT,
+    NUM_BARS
 };
 
 struct Params {
@@ -189,12 +199,89 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, int sr
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
 
+// Rows [rank 128 / C, (rank + 1) 128 / C) of tile t from the C partial states of the cluster (sO, sStat:
+// this CTA's, at the same address in every CTA) into `out` and lse.  C lanes per row, each with every
+// C-th group of eight columns; eight 32-byte remote loads of a lane are in flight at a time.
+template <int C, int HD, bool FP8>
+__device__ __forceinline__ void merge_parts(const Params &prm, const WorkItem &wi, int t, int r, int rank, int b, int h,
+                                            int bh, uint32_t sO, uint32_t sStat) {
+    const int part = r % C, mrow = rank * (BM / C) + r / C;
+    float4 st[C];
+#pragma unroll
+    for (int p = 0; p < C; ++p) st[p] = ld_cluster_v4(cluster_map(sStat + mrow * 16, p));
+    constexpr int GROUPS = HD / 8 / C, BATCH = GROUPS < 8 / C ? GROUPS : 8 / C;
+    float4 x[BATCH][C][2];
+    auto load = [&](int g0) {
+#pragma unroll
+        for (int g = 0; g < BATCH; ++g)
+#pragma unroll
+            for (int p = 0; p < C; ++p)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int ch = ((g0 + g) * C + part) * 2 + e;
+                    x[g][p][e] = ld_cluster_v4(cluster_map(sO + mrow * (HD * 4) + (((ch & ~7) | ((ch ^ mrow) & 7)) << 4), p));
+                }
+    };
+    load(0);   // in flight together with the statistics
+    const bool in = t * BM + mrow < wi.q_rows;
+    int out_row = wi.q_start + t * BM + mrow;
+    if (prm.out_map && in) out_row = prm.out_map[out_row];
+    __nv_bfloat16 *orow = prm.out + (long long)b * prm.stride_b + (long long)h * prm.stride_h + (long long)out_row * prm.stride_s;
+    float m = st[0].x;
+#pragma unroll
+    for (int p = 1; p < C; ++p) m = fmaxf(m, st[p].x);
+    float l = 0.f, l_fix = 0.f, w[C];
+#pragma unroll
+    for (int p = 0; p < C; ++p) {
+        // weight 0: not even a NaN of that share counts (a share of nothing but -inf scores has no maximum)
+        w[p] = ex2(st[p].x - m);
+        l = w[p] != 0.f ? fmaf(st[p].y, w[p], l) : l;
+        l_fix = w[p] != 0.f ? fmaf(st[p].z, w[p], l_fix) : l_fix;
+    }
+    const float inv = 1.f / (l + l_fix);
+#pragma unroll
+    for (int g0 = 0; g0 < GROUPS; g0 += BATCH) {
+        if (g0 > 0) load(g0);
+#pragma unroll
+        for (int g = 0; g < BATCH; ++g) {
+            float4 a[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                a[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int p = 0; p < C; ++p) {
+                    if (w[p] == 0.f) continue;
+                    a[e].x = fmaf(x[g][p][e].x, w[p], a[e].x);
+                    a[e].y = fmaf(x[g][p][e].y, w[p], a[e].y);
+                    a[e].z = fmaf(x[g][p][e].z, w[p], a[e].z);
+                    a[e].w = fmaf(x[g][p][e].w, w[p], a[e].w);
+                }
+            }
+            if (in)
+                *reinterpret_cast<uint4 *>(orow + ((g0 + g) * C + part) * 8) =
+                    make_uint4(pack_bf16(a[0].x * inv, a[0].y * inv), pack_bf16(a[0].z * inv, a[0].w * inv),
+                               pack_bf16(a[1].x * inv, a[1].y * inv), pack_bf16(a[1].z * inv, a[1].w * inv));
+        }
+    }
+    if (prm.lse && in && part == 0)
+        prm.lse[(long long)bh * prm.S + out_row] = 0.6931471805599453f * (m - (FP8 ? P_SHIFT_FP8 : 0.f) + log2f(l));
+}
+
 // GATHER = false: Q / K / V tiles arrive by TMA from tensors in physical order.
 // GATHER = true : the tensors are in ORIGINAL order (the entry gather of Sec. 3.4 fused in): two loader
 // warps fetch every tile row through the permutation table with 16-byte cp.async copies and place it
 // where a 128-byte-swizzled TMA box would have put it, so everything downstream is unchanged.
 // FP8: q, k, v hold e4m3 bytes (HD = 128 only); the weights P are rounded to e4m3 as well; out stays bf16.
-template <bool GATHER, int HD, bool FP8 = false>
+// SPLIT: launched in clusters; units marked SPLIT_UNIT hold a share of an item's keys each (the same item
+// and head in every CTA of the cluster, first in the CTAs' lists) and are merged at their end through
+// distributed shared memory: every CTA leaves (m, l, O) of its share in the space of its tiles, and rank c
+// writes its rows c 128 / C ... of each query tile.  No workspace, so launches of one plan on several
+// streams stay independent; the order of the sum is that of the ranks, so results are reproducible.
+// Measured (B200): 3 heads at 2048^2, where nine prefix units of 132 blocks each had a CTA of their own,
+// 220 -> 73 us a launch; 8 heads at 512^2, fused gathers, 28.7 -> 18.1 us.  A cluster launch costs 1.2 us and
+// a merge 5 ... 7, which is why only plans that gain more are cut (choose_split) and the others launch the
+// instantiation without it.
+template <bool GATHER, int HD, bool FP8 = false, bool SPLIT = false>
 __global__ void __launch_bounds__(THREADS, 1)
 attn_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                  const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
@@ -221,7 +308,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t sQ = smem_u32(smem);
     const uint32_t sKV = sQ + QT * TILE_BYTES;
-    const uint32_t sStage = sKV + NS * TILE_BYTES;   // TMA kernels only: 4 KB per softmax warp
+    const uint32_t sStage = sQ + tile_area(HD, FP8, GATHER, SPLIT);   // TMA kernels only: 4 KB per softmax warp
     const int tid = threadIdx.x, warp = tid >> 5;
     const uint32_t bar0 = smem_u32(&bars[0]);
     auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
@@ -232,6 +319,8 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         {
             uint32_t count = 1;
             if (i >= P_READY && i < P_READY + 2 * QT) count = HB_WARP_ARRIVE ? 4 : 128;
+            if (SPLIT && i >= PART_READY && i < PART_READY + QT) count = 4 * cluster_cta_count();
+            if (SPLIT && i == PART_READ) count = 8 * cluster_cta_count();
             if (GATHER && (i == Q_FULL || (i >= KV_FULL && i < KV_FULL + NSTAGE))) count = GATHER_THREADS;
             mbar_init(bar(i), count);
         }
@@ -244,6 +333,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (SPLIT) cluster_sync_all();   // the peers' barriers are initialised
     const uint32_t tmem = tmem_slot;
     const int u_begin = prm.cta_begin[blockIdx.x], u_end = prm.cta_begin[blockIdx.x + 1];
     if (blockIdx.x == 0 && tid == 0) {
@@ -263,7 +353,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     if constexpr (GATHER) {
     if (warp == 10 || warp == 11) {
         // ------------------------------------------------- gathering loaders (entry permute fused in)
-        uint32_t kvc = 0, qc = 0;
+        uint32_t kvc = 0, qc = 0, sc = 0;
         bool ok = true;
         // The stage's barrier counts one arrival per loader thread; each arrival fires by itself
         // when that thread's copies into the stage have landed, so the loaders never wait for data.
@@ -376,6 +466,9 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                     publish(bar(KV_FULL + sv));
                 }
             }
+            // the partial states in the tiles' space have been read by the whole cluster
+            if (SPLIT && ok && unit.bh2 == SPLIT_UNIT)
+                ok = wait_or_abort(bar(PART_READ), sc++ & 1, &abort_flag, prm.status, 0x114);
         }
         // every copy lands before the CTA retires
         asm volatile("cp.async.wait_all;" ::: "memory");
@@ -387,7 +480,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             prefetch_tmap(&tmQ);
             prefetch_tmap(&tmK);
             prefetch_tmap(&tmV);
-            uint32_t kvc = 0, qc = 0;
+            uint32_t kvc = 0, qc = 0, sc = 0;
             bool ok = true;
             // one ring entry: the K or V tile at key row `row` of head (h, b)
             auto emit = [&](const CUtensorMap *tm, int row, int h, int b) {
@@ -442,6 +535,9 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                         }
                     }
                 }
+                // the partial states in the tiles' space have been read by the whole cluster
+                if (SPLIT && ok && unit.bh2 == SPLIT_UNIT)
+                    ok = wait_or_abort(bar(PART_READ), sc++ & 1, &abort_flag, prm.status, 0x103);
             }
             if (!ok) {
                 // let every copy already issued land before the CTA retires
@@ -573,6 +669,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                         if (j + 2 == n) mma_commit(bar(Q_EMPTY));
                     }
                 }
+                if (SPLIT && ok && unit.bh2 == SPLIT_UNIT) mma_commit(bar(UNIT_MMA));
             }
             // every MMA issued above has retired before TMEM is released
             mma_commit(bar(DRAIN));
@@ -595,6 +692,7 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         const uint32_t tO = tmem + lane_addr + 256 + t * HD;
         const float scale_log2 = prm.scale_log2;
         uint32_t cS = 0, cPV = 0;
+        uint32_t cSplit = 0, cPart = 0;   // split units so far: all, those with this tile present
         bool ok = true;
 #ifdef HB_STAMPS
         int st_b2 = 0, st_b1 = 0, st_items2 = 0, st_items1 = 0, st_prefix_blocks = 0;
@@ -613,7 +711,17 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             }
 #endif
             const bool dual = unit.bh2 >= 0;   // the item for two heads: tile slot 1 holds the same rows of head bh2
-            if (wi.q_rows <= t * BM && !dual) continue;  // this tile is absent from the item
+            const bool split = SPLIT && unit.bh2 == SPLIT_UNIT;
+            if (wi.q_rows <= t * BM && !dual) {   // this tile is absent from the item
+                if (split) {
+                    // has read nothing; in step with the other tile, so that no arrival runs a phase ahead
+                    ok = wait_or_abort(bar(PART_READY), cSplit++ & 1, &abort_flag, prm.status, 0x306);
+                    if (!ok) break;
+                    if ((uint32_t)(tid & 31) < cluster_cta_count())
+                        mbar_arrive_cluster(cluster_map(bar(PART_READ), tid & 31));
+                }
+                continue;
+            }
             const int bh = (dual && t) ? unit.bh2 : unit.bh;
             const int b = bh / prm.heads, h = bh % prm.heads;
             float m_ref = 0.f, l = 0.f;
@@ -752,6 +860,40 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             ok = wait_or_abort(bar(PV_DONE + t), (cPV - 1) & 1, &abort_flag, prm.status, 0x305 + t);
             if (!ok) break;
             tc_fence_after();
+            if (split) {
+                ok = wait_or_abort(bar(UNIT_MMA), cSplit++ & 1, &abort_flag, prm.status, 0x307);
+                if (!ok) break;
+                const uint32_t n_cta = cluster_cta_count();
+                const uint32_t sO = sQ + t * (BM * HD * 4), sStat = sQ + ITEM_ROWS * HD * 4 + t * (BM * 16);
+                // 16-byte chunk c of row r sits at chunk c ^ (r & 7) of its group of eight: conflict-free
+#pragma unroll
+                for (int c = 0; c < HD / 32; ++c) {
+                    uint32_t o[32];
+                    tmem_ld32(tO + c * 32, o);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) st_shared_v4(sO + r * (HD * 4) + ((c * 8 + (k ^ (r & 7))) << 4), o + 4 * k);
+                }
+                {
+                    const uint32_t w[4] = {__float_as_uint(m_ref), __float_as_uint(l), __float_as_uint(l_fix), 0u};
+                    st_shared_v4(sStat + r * 16, w);
+                }
+                tc_fence_before();
+                fence_proxy_async_smem();   // ... and the next unit's tiles land here through the async proxy
+                __syncwarp();
+                if ((uint32_t)(tid & 31) < n_cta) mbar_arrive_release_cluster(cluster_map(bar(PART_READY + t), tid & 31));
+                ok = wait_or_abort(bar(PART_READY + t), cPart++ & 1, &abort_flag, prm.status, 0x308 + t);
+                if (!ok) break;
+                cluster_acquire();
+                const int rank = (int)cluster_cta_rank();
+                if (n_cta == 2) merge_parts<2, HD, FP8>(prm, wi, t, r, rank, b, h, bh, sO, sStat);
+                else if (n_cta == 4) merge_parts<4, HD, FP8>(prm, wi, t, r, rank, b, h, bh, sO, sStat);
+                else merge_parts<8, HD, FP8>(prm, wi, t, r, rank, b, h, bh, sO, sStat);
+                __syncwarp();
+                // nothing to release: the loads above have returned
+                if ((uint32_t)(tid & 31) < n_cta) mbar_arrive_cluster(cluster_map(bar(PART_READ), tid & 31));
+                continue;
+            }
             const float inv = 1.f / (l + l_fix);
             const int row = dual ? r : t * BM + r;
             // each thread stores its own row, so writing it at its ORIGINAL position instead
@@ -855,6 +997,8 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     if (!GATHER && warp < 8 && (tid & 31) == 0) bulk_wait_group0();
     tc_fence_before();
     __syncthreads();
+    __syncwarp();
+    if (SPLIT) cluster_sync_all();   // peers signal this CTA's barriers until their last split unit is done
     if (blockIdx.x == 0 && tid == 0) {
         // elapsed SM cycles and nanoseconds of this CTA: the launch's effective SM clock
         unsigned long long ns;
@@ -960,6 +1104,58 @@ int launch_timeout_probe(const hilberta_plan_t *p, cudaStream_t stream) {
     return HILBERTA_OK;
 }
 
+namespace {
+
+template <bool GATHER, int HD, bool FP8, bool SPLIT>
+cudaError_t opt_in_one() {
+    return cudaFuncSetAttribute(attn_bf16_kernel<GATHER, HD, FP8, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                smem_bytes(HD, FP8, GATHER, SPLIT));
+}
+
+// Clusters of 2, 4 and 8 CTAs of this kernel that a device runs at once (one CTA per SM; GPCs with an odd
+// rest of SMs lose some); filled by attn_bf16_opt_in.
+int g_clusters[64][3] = {};
+const int *split_clusters(int device) { return g_clusters[device]; }
+
+// The shared-memory opt-in is an attribute of the kernel ON ONE DEVICE: set it once for every device a
+// plan is bound on (a failure is reported, not remembered).
+int attn_bf16_opt_in(int device) {
+    static std::mutex attr_mutex;
+    static bool attr_done[64] = {};
+    std::lock_guard<std::mutex> lock(attr_mutex);
+    if (device < 0 || device >= 64) return HILBERTA_ERR_INVALID;
+    if (attr_done[device]) return HILBERTA_OK;
+    HB_CUDA((opt_in_one<false, 128, false, false>()));
+    HB_CUDA((opt_in_one<true, 128, false, false>()));
+    HB_CUDA((opt_in_one<false, 64, false, false>()));
+    HB_CUDA((opt_in_one<true, 64, false, false>()));
+    HB_CUDA((opt_in_one<false, 128, true, false>()));
+    HB_CUDA((opt_in_one<true, 128, true, false>()));
+    HB_CUDA((opt_in_one<false, 128, false, true>()));
+    HB_CUDA((opt_in_one<true, 128, false, true>()));
+    HB_CUDA((opt_in_one<false, 64, false, true>()));
+    HB_CUDA((opt_in_one<true, 64, false, true>()));
+    HB_CUDA((opt_in_one<false, 128, true, true>()));
+    HB_CUDA((opt_in_one<true, 128, true, true>()));
+    for (int i = 0; i < 3; ++i) {
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = 2u << i;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cfg.gridDim = dim3(2u << i);
+        cfg.blockDim = dim3(THREADS);
+        cfg.dynamicSmemBytes = (size_t)smem_bytes(128, false, false, true);
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        HB_CUDA(cudaOccupancyMaxActiveClusters(&g_clusters[device][i], attn_bf16_kernel<false, 128, false, true>, &cfg));
+    }
+    attr_done[device] = true;
+    return HILBERTA_OK;
+}
+
+}  // namespace
+
 // Work list (items of two query tiles, key blocks of 128) and the static schedules.
 int attn_bf16_prepare(hilberta_plan_t *p) {
     // Cost of a unit in twentieths of a two-tile key block (about 140 SM cycles), from per-unit cycle
@@ -996,13 +1192,11 @@ int attn_bf16_prepare(hilberta_plan_t *p) {
     p->n_cta_chunk = 0;
     p->n_work = (int)items.size();
     p->n_cta = 0;
+    p->split_cluster = 1;
     if (items.empty()) return HILBERTA_OK;
-
-    HB_CUDA(cudaMalloc(&p->d_work, sizeof(WorkItem) * items.size()));
-    HB_CUDA(cudaMemcpy(p->d_work, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice));
-    int rc = upload_schedule(items, cost, p->batch * p->heads, p->sm_count, &p->d_units, &p->d_cta_begin, &p->n_cta,
-                             &cost_two_heads);
+    int rc = attn_bf16_opt_in(p->device);
     if (rc != HILBERTA_OK) return rc;
+
     // slice of heads for the pipelined host-buffer path: the largest divisor of `heads` not above heads / HB_HOST_SLICES (rounded up)
     p->chunk_heads = p->heads;
     for (int d = (p->heads + HB_HOST_SLICES - 1) / HB_HOST_SLICES; d >= 1; --d)
@@ -1010,27 +1204,23 @@ int attn_bf16_prepare(hilberta_plan_t *p) {
             p->chunk_heads = d;
             break;
         }
+    // How the longest items are cut over clusters is decided once, for the whole problem: a slice of heads
+    // then gives every row the same sums in the same order.
+    SplitChoice choice;
+    choose_split(items, cost, cost_two_heads, p->batch * p->heads, p->sm_count, split_clusters(p->device), BN, choice);
+    p->split_cluster = choice.cluster;
+    const int n_whole = (int)items.size();
+    for (const WorkItem &it : choice.shares) items.push_back(it);
+    HB_CUDA(cudaMalloc(&p->d_work, sizeof(WorkItem) * items.size()));
+    HB_CUDA(cudaMemcpy(p->d_work, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice));
+    items.resize(n_whole);
+    rc = upload_split_schedule(items, cost, cost_two_heads, p->batch * p->heads, p->sm_count, choice, &p->d_units, &p->d_cta_begin,
+                               &p->n_cta);
+    if (rc != HILBERTA_OK) return rc;
     if (p->chunk_heads < p->heads) {
-        rc = upload_schedule(items, cost, p->batch * p->chunk_heads, p->sm_count, &p->d_units_chunk, &p->d_cta_begin_chunk,
-                             &p->n_cta_chunk, &cost_two_heads);
+        rc = upload_split_schedule(items, cost, cost_two_heads, p->batch * p->chunk_heads, p->sm_count, choice, &p->d_units_chunk,
+                                   &p->d_cta_begin_chunk, &p->n_cta_chunk);
         if (rc != HILBERTA_OK) return rc;
-    }
-    {
-        // The shared-memory opt-in is an attribute of the kernel ON ONE DEVICE: set it once for every
-        // device a plan is bound on (a failure is reported, not remembered).
-        static std::mutex attr_mutex;
-        static bool attr_done[64] = {};
-        std::lock_guard<std::mutex> lock(attr_mutex);
-        if (p->device < 0 || p->device >= 64) return HILBERTA_ERR_INVALID;
-        if (!attr_done[p->device]) {
-            HB_CUDA(cudaFuncSetAttribute(attn_bf16_kernel<false, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(128)));
-            HB_CUDA(cudaFuncSetAttribute(attn_bf16_kernel<true, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(128, false, true)));
-            HB_CUDA(cudaFuncSetAttribute(attn_bf16_kernel<false, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(64)));
-            HB_CUDA(cudaFuncSetAttribute(attn_bf16_kernel<true, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(64, false, true)));
-            HB_CUDA(cudaFuncSetAttribute(attn_bf16_kernel<false, 128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(128, true)));
-            HB_CUDA(cudaFuncSetAttribute(attn_bf16_kernel<true, 128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(128, true, true)));
-            attr_done[p->device] = true;
-        }
     }
     {
         const int rc_solo = attn_bf16_solo_prepare(p);
@@ -1099,29 +1289,40 @@ int launch_attn_bf16(const hilberta_plan_t *p, const void *q, const void *k, con
     prm.out_align32 = (((uintptr_t)out & 31) == 0 && ((p->stride_b | p->stride_h | p->stride_s) & 15) == 0) ? 1 : 0;
     CUtensorMap mo = mq;   // a valid map in any case; read only with bit 1 set
     if (!in_map && !out_map && make_out_tensor_map(&mo, out, p, heads)) prm.out_align32 |= 2;
-    if (in_map) {
-        KernelParams<true> gprm;
-        static_cast<Params &>(gprm) = prm;
-        gprm.in_map = in_map;
-        gprm.gq = q;
-        gprm.gk = k;
-        gprm.gv = v;
-        if (fp8)
-            attn_bf16_kernel<true, 128, true><<<n_cta, THREADS, smem_bytes(128, true, true), stream>>>(mq, mk, mv, mo, gprm);
-        else if (p->head_dim == 128)
-            attn_bf16_kernel<true, 128><<<n_cta, THREADS, smem_bytes(128, false, true), stream>>>(mq, mk, mv, mo, gprm);
-        else
-            attn_bf16_kernel<true, 64><<<n_cta, THREADS, smem_bytes(64, false, true), stream>>>(mq, mk, mv, mo, gprm);
-    } else {
-        KernelParams<false> pprm;
-        static_cast<Params &>(pprm) = prm;
-        if (fp8)
-            attn_bf16_kernel<false, 128, true><<<n_cta, THREADS, smem_bytes(128, true), stream>>>(mq, mk, mv, mo, pprm);
-        else if (p->head_dim == 128)
-            attn_bf16_kernel<false, 128><<<n_cta, THREADS, smem_bytes(128), stream>>>(mq, mk, mv, mo, pprm);
-        else
-            attn_bf16_kernel<false, 64><<<n_cta, THREADS, smem_bytes(64), stream>>>(mq, mk, mv, mo, pprm);
-    }
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr{};
+    cfg.gridDim = dim3((unsigned)n_cta);
+    cfg.blockDim = dim3(THREADS);
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)p->split_cluster;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.numAttrs = p->split_cluster > 1 ? 1 : 0;
+    KernelParams<true> gprm;
+    static_cast<Params &>(gprm) = prm;
+    gprm.in_map = in_map;
+    gprm.gq = q;
+    gprm.gk = k;
+    gprm.gv = v;
+    KernelParams<false> pprm;
+    static_cast<Params &>(pprm) = prm;
+    auto launch = [&](auto split) {
+        constexpr bool SPLIT = decltype(split)::value;
+        auto go = [&](auto kernel, int smem, const auto &params) {
+            cfg.dynamicSmemBytes = (size_t)smem;
+            return cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, mo, params);
+        };
+        if (in_map) {
+            if (fp8) return go(attn_bf16_kernel<true, 128, true, SPLIT>, smem_bytes(128, true, true, SPLIT), gprm);
+            if (p->head_dim == 128) return go(attn_bf16_kernel<true, 128, false, SPLIT>, smem_bytes(128, false, true, SPLIT), gprm);
+            return go(attn_bf16_kernel<true, 64, false, SPLIT>, smem_bytes(64, false, true, SPLIT), gprm);
+        }
+        if (fp8) return go(attn_bf16_kernel<false, 128, true, SPLIT>, smem_bytes(128, true, false, SPLIT), pprm);
+        if (p->head_dim == 128) return go(attn_bf16_kernel<false, 128, false, SPLIT>, smem_bytes(128, false, false, SPLIT), pprm);
+        return go(attn_bf16_kernel<false, 64, false, SPLIT>, smem_bytes(64, false, false, SPLIT), pprm);
+    };
+    HB_CUDA(p->split_cluster > 1 ? launch(std::true_type{}) : launch(std::false_type{}));
     HB_LAUNCHED();
     return HILBERTA_OK;
 }

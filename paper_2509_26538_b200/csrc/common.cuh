@@ -52,7 +52,8 @@ struct WorkItem {
 // A work item applied to one (batch, head).  Units are assigned to CTAs on the
 // host (longest-processing-time-first) and stored grouped by CTA.  bh2 >= 0 (forward kernel
 // only, items of one query tile): the same item for a second (batch, head), which takes the
-// CTA's other query-tile slot with a K/V stream of its own.
+// CTA's other query-tile slot with a K/V stream of its own.  bh2 == -2 (forward kernel in clusters): a
+// share of an item's keys, the other shares being the same unit of the cluster's other CTAs.
 struct WorkUnit {
     int item;
     int bh;
@@ -92,6 +93,7 @@ struct hilberta_plan_s {
     // a second schedule over a slice of chunk_heads heads (all batches), for the host-buffer entry
     // point, which pipelines copies and launches slice by slice; chunk_heads == heads: no slicing
     int chunk_heads;
+    int split_cluster;            // CTAs per cluster of the forward launches (1: no clusters, no split units)
     hilberta::WorkUnit *d_units_chunk;
     int *d_cta_begin_chunk;
     int n_cta_chunk;
@@ -153,6 +155,24 @@ long long build_schedule(int n_items, const long long *cost, const long long *co
 int upload_schedule(const std::vector<WorkItem> &items, const std::vector<long long> &cost, int bh, int sm_count,
                     WorkUnit **d_units, int **d_cta_begin, int *n_cta_out,
                     const std::vector<long long> *cost_two_heads = nullptr);
+// How a schedule cuts its longest items (the first n_items of the list) over clusters of `cluster` CTAs;
+// shares: cluster entries per cut item, in rank order, appended to the uploaded work list.
+struct SplitChoice {
+    int cluster = 1, n_clusters = 0, n_items = 0;
+    bool pair_heads = true;
+    std::vector<WorkItem> shares;
+};
+// clusters: how many clusters of 2, 4 and 8 CTAs run at once.  items sorted by descending cost.
+void choose_split(const std::vector<WorkItem> &items, const std::vector<long long> &cost,
+                  const std::vector<long long> &cost_two_heads, int bh, int sm_count, const int *clusters, int block,
+                  SplitChoice &choice);
+// The schedule of such a choice (units null: none is written); returns the largest CTA load.
+long long build_split_schedule(const std::vector<WorkItem> &items, const std::vector<long long> &cost,
+                               const std::vector<long long> &cost_two_heads, int bh, int sm_count, const SplitChoice &choice,
+                               std::vector<WorkUnit> *units, std::vector<int> *cta_begin);
+int upload_split_schedule(const std::vector<WorkItem> &items, const std::vector<long long> &cost,
+                          const std::vector<long long> &cost_two_heads, int bh, int sm_count, const SplitChoice &choice,
+                          WorkUnit **d_units, int **d_cta_begin, int *n_cta_out);
 int attn_bf16_prepare(hilberta_plan_t *p);
 // attn_bf16_pair_sm100.cu: the forward kernel on pairs of SMs (bf16, head dim 128, inputs in physical order)
 int attn_bf16_pair_prepare(hilberta_plan_t *p);

@@ -149,6 +149,207 @@ int upload_schedule(const std::vector<WorkItem> &items, const std::vector<long l
     return HILBERTA_OK;
 }
 
+// ---------------------------------------------------------------------------
+// Items cut over clusters.  A prefix item's key list is the whole sequence; with few heads a handful of
+// them outlasts everything else (3 heads at 2048^2: 9 units of 132 blocks against 26 blocks per SM of
+// work in all).  Such items are cut into one share per CTA of a cluster.
+// ---------------------------------------------------------------------------
+
+// Cost of merging a share, in the cost model's twentieths of a key block (1.45 us): the partial sums' way
+// through shared memory and the waits for the cluster.  From one problem of five ten-block items on the
+// B200: 22.7 us uncut, 21.3 in shares of two and 20.8 in shares of four, i.e. 6 and 8 us a merge.
+static long long merge_cost(int cluster) { return cluster == 2 ? 85 : cluster == 4 ? 110 : 135; }
+
+// Greedy assignment to the least loaded of n machines: loads and machine numbers in one heap of 64-bit
+// keys (load, then number, smallest first).
+struct LeastLoaded {
+    std::vector<uint64_t> heap;
+    explicit LeastLoaded(const std::vector<long long> &load) {
+        for (size_t i = 0; i < load.size(); ++i) heap.push_back(((uint64_t)load[i] << 16) | i);
+        std::make_heap(heap.begin(), heap.end(), std::greater<uint64_t>());
+    }
+    // adds `cost` to the least loaded machine; returns (its new load, its number)
+    std::pair<long long, int> add(long long cost) {
+        const size_t n = heap.size();
+        const uint64_t top = heap[0] + ((uint64_t)cost << 16);
+        size_t i = 0;
+        for (;;) {   // sift the grown top down
+            size_t c = 2 * i + 1;
+            if (c >= n) break;
+            if (c + 1 < n && heap[c + 1] < heap[c]) ++c;
+            if (heap[c] >= top) break;
+            heap[i] = heap[c];
+            i = c;
+        }
+        heap[i] = top;
+        return std::make_pair((long long)(top >> 16), (int)(top & 0xffff));
+    }
+};
+
+// Every rank's list starts with the cut units of its cluster, in the same order; the other units go,
+// longest first, to the least loaded CTA.  units == nullptr: the largest load only.
+long long build_split_schedule(const std::vector<WorkItem> &items, const std::vector<long long> &cost,
+                               const std::vector<long long> &cost_two_heads, int bh, int sm_count, const SplitChoice &ch,
+                               std::vector<WorkUnit> *units, std::vector<int> *cta_begin) {
+    const int C = ch.cluster;
+    // runs of equal units: of item i, for two heads each or for one, from head `first` on
+    struct Run {
+        long long cost;
+        int item, first, count, step;
+    };
+    std::vector<Run> runs;
+    long long n_units = (long long)ch.n_items * bh * C;
+    for (int i = ch.n_items; i < (int)items.size(); ++i) {
+        const long long two = ch.pair_heads ? cost_two_heads[i] : 0;
+        int j = 0;
+        if (two > 0 && bh > 1) {
+            runs.push_back(Run{two, i, 0, bh / 2, 2});
+            j = bh / 2 * 2;
+        }
+        if (j < bh) runs.push_back(Run{cost[i], i, j, bh - j, 1});
+        n_units += bh / 2 * (j > 0 ? 1 : 0) + (bh - j);
+    }
+    std::stable_sort(runs.begin(), runs.end(), [](const Run &a, const Run &b) { return a.cost > b.cost; });
+    const int most = C > 1 ? ch.n_clusters * C : sm_count;
+    const int n_cta = C > 1 ? (int)std::min<long long>((n_units + C - 1) / C * C, most) : (int)std::min<long long>(n_units, most);
+    std::vector<int> cta_of;   // of every unit, in the order of assignment
+    std::vector<WorkUnit> order;
+    if (units) {
+        cta_of.reserve((size_t)n_units);
+        order.reserve((size_t)n_units);
+    }
+    long long makespan = 0;
+    std::vector<long long> load((size_t)n_cta, 0);
+    if (ch.n_items > 0) {
+        LeastLoaded clusters(std::vector<long long>((size_t)(n_cta / C), 0));
+        for (int i = 0; i < ch.n_items; ++i)
+            for (int j = 0; j < bh; ++j) {
+                const std::pair<long long, int> at = clusters.add((cost[i] + C - 1) / C + merge_cost(C));
+                makespan = std::max(makespan, at.first);
+                for (int r = 0; r < C; ++r) {
+                    load[(size_t)(at.second * C + r)] = at.first;
+                    if (units) {
+                        order.push_back(WorkUnit{(int)items.size() + i * C + r, j, -2});
+                        cta_of.push_back(at.second * C + r);
+                    }
+                }
+            }
+    }
+    LeastLoaded ctas(load);
+    for (const Run &run : runs)
+        for (int k = 0; k < run.count; ++k) {
+            const std::pair<long long, int> at = ctas.add(run.cost);
+            makespan = std::max(makespan, at.first);
+            if (units) {
+                const int j = run.first + k * run.step;
+                order.push_back(WorkUnit{run.item, j, run.step == 2 ? j + 1 : -1});
+                cta_of.push_back(at.second);
+            }
+        }
+    if (units) {
+        cta_begin->assign((size_t)n_cta + 1, 0);
+        for (int c : cta_of) ++(*cta_begin)[(size_t)c + 1];
+        for (int c = 0; c < n_cta; ++c) (*cta_begin)[(size_t)c + 1] += (*cta_begin)[(size_t)c];
+        std::vector<int> next(cta_begin->begin(), cta_begin->end() - 1);
+        units->resize(order.size());
+        for (size_t u = 0; u < order.size(); ++u) (*units)[(size_t)next[(size_t)cta_of[u]]++] = order[u];
+    }
+    return makespan;
+}
+
+// Blocks [lo, hi) of an item's key list as an item of its own (the same rows, part of the keys).
+static WorkItem share_of(const WorkItem &it, int lo, int hi, int block) {
+    WorkItem s = it;
+    s.n_seg = 0;
+    s.kv_blocks = hi - lo;
+    for (int g = 0, b0 = 0; g < it.n_seg; ++g) {
+        const int nb = (it.seg_len[g] + block - 1) / block;
+        const int a = std::max(lo - b0, 0), e = std::min(hi - b0, nb);
+        if (a < e) {
+            s.seg_start[s.n_seg] = it.seg_start[g] + a * block;
+            s.seg_len[s.n_seg] = std::min(it.seg_len[g], e * block) - a * block;
+            ++s.n_seg;
+        }
+        b0 += nb;
+    }
+    for (int g = s.n_seg; g < 3; ++g) s.seg_start[g] = s.seg_len[g] = 0;
+    return s;
+}
+
+void choose_split(const std::vector<WorkItem> &items, const std::vector<long long> &cost,
+                  const std::vector<long long> &cost_two_heads, int bh, int sm_count, const int *clusters, int block,
+                  SplitChoice &choice) {
+    choice = SplitChoice();
+    long long total = 0, n_units = 0;   // as scheduled without cuts
+    for (size_t i = 0; i < items.size(); ++i) {
+        const int pairs = cost_two_heads[i] > 0 ? bh / 2 : 0;
+        total += cost_two_heads[i] * pairs + cost[i] * (bh - 2 * pairs);
+        n_units += bh - pairs;
+    }
+    auto load_of = [&](const SplitChoice &c) {
+        return build_split_schedule(items, cost, cost_two_heads, bh, sm_count, c, nullptr, nullptr);
+    };
+    long long best = load_of(choice);
+    // within 3 % of a perfect balance nothing is to be gained
+    if (best * sm_count <= total + total / 32) return;
+    // (units per head instead of per two only matter where there are CTAs to take them)
+    const bool few = n_units < 2ll * sm_count;
+    if (few) {
+        SplitChoice c = choice;
+        c.pair_heads = false;   // idle CTAs: a unit per head is shorter than one for two
+        const long long m = load_of(c);
+        if (m < best) {
+            best = m;
+            choice = c;
+        }
+    }
+    for (int k = 0; k < 3; ++k) {
+        const int C = 2 << k;
+        if (clusters[k] < 1) continue;
+        SplitChoice c;
+        c.cluster = C;
+        c.n_clusters = clusters[k];
+        // cut the items of the longest, of the two longest, ... lengths; every share gets a block at least
+        int levels = 0;
+        for (int n = 1; n <= (int)items.size() && levels < (n_units > 16ll * sm_count ? 1 : 4); ++n) {
+            if (items[n - 1].kv_blocks < C) break;
+            if (n < (int)items.size() && items[n].kv_blocks == items[n - 1].kv_blocks) continue;
+            ++levels;
+            c.n_items = n;
+            for (int pair = 1; pair >= (few ? 0 : 1); --pair) {
+                c.pair_heads = pair != 0;
+                const long long m = load_of(c);
+                // clusters start together and merging is not free: only for a clear gain
+                if (m + m / 32 < best) {
+                    best = m;
+                    choice = c;
+                }
+            }
+        }
+    }
+    for (int i = 0; i < choice.n_items; ++i) {
+        const int n = items[i].kv_blocks;
+        for (int r = 0; r < choice.cluster; ++r)
+            choice.shares.push_back(share_of(items[i], (int)((long long)n * r / choice.cluster),
+                                             (int)((long long)n * (r + 1) / choice.cluster), block));
+    }
+}
+
+int upload_split_schedule(const std::vector<WorkItem> &items, const std::vector<long long> &cost,
+                          const std::vector<long long> &cost_two_heads, int bh, int sm_count, const SplitChoice &choice,
+                          WorkUnit **d_units, int **d_cta_begin, int *n_cta_out) {
+    if ((long long)items.size() * bh > (1ll << 30)) return HILBERTA_ERR_INVALID;
+    std::vector<WorkUnit> units;
+    std::vector<int> cta_begin;
+    build_split_schedule(items, cost, cost_two_heads, bh, sm_count, choice, &units, &cta_begin);
+    *n_cta_out = (int)cta_begin.size() - 1;
+    HB_CUDA(cudaMalloc(d_units, sizeof(WorkUnit) * units.size()));
+    HB_CUDA(cudaMemcpy(*d_units, units.data(), sizeof(WorkUnit) * units.size(), cudaMemcpyHostToDevice));
+    HB_CUDA(cudaMalloc(d_cta_begin, sizeof(int) * cta_begin.size()));
+    HB_CUDA(cudaMemcpy(*d_cta_begin, cta_begin.data(), sizeof(int) * cta_begin.size(), cudaMemcpyHostToDevice));
+    return HILBERTA_OK;
+}
+
 }  // namespace hilberta
 
 static_assert(sizeof(hilberta::WorkItem) == 10 * sizeof(int32_t), "hilberta_check_work_list takes ten ints per item");
