@@ -600,13 +600,7 @@ int make_tensor_map(CUtensorMap *m, const void *base, const hilberta_plan_t *p, 
 
 // Work list (items of 256 rows = one pair of CTAs) and the static schedule over pairs of SMs.
 // Returns OK and leaves p->n_pair == 0 if this shape is not served by the pair kernel.
-int attn_bf16_pair_prepare(hilberta_plan_t *p) {
-    cudaFree(p->d_work_pair);
-    cudaFree(p->d_units_pair);
-    cudaFree(p->d_pair_begin);
-    p->d_work_pair = nullptr;
-    p->d_units_pair = nullptr;
-    p->d_pair_begin = nullptr;
+int attn_bf16_pair_prepare(hilberta_plan_t *p, BindImage &image) {
     p->n_pair = 0;
     if (p->dtype != HILBERTA_BF16 || p->head_dim != HD) return HILBERTA_OK;
     {
@@ -646,9 +640,8 @@ int attn_bf16_pair_prepare(hilberta_plan_t *p) {
                      [&](const WorkItem &a, const WorkItem &b) { return cost_of(a) > cost_of(b); });
     std::vector<long long> cost;
     for (const WorkItem &it : items) cost.push_back(cost_of(it));
-    HB_CUDA(cudaMalloc(&p->d_work_pair, sizeof(WorkItem) * items.size()));
-    HB_CUDA(cudaMemcpy(p->d_work_pair, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice));
-    return upload_schedule(items, cost, p->batch * p->heads, max_pairs, &p->d_units_pair, &p->d_pair_begin, &p->n_pair);
+    image.add(items, &p->d_work_pair);
+    return add_schedule(image, cost, {}, p->batch * p->heads, max_pairs, SplitChoice(), &p->d_units_pair, &p->d_pair_begin, &p->n_pair);
 }
 
 int launch_attn_bf16_pair(const hilberta_plan_t *p, const void *q, const void *k, const void *v, void *out,

@@ -1157,7 +1157,7 @@ int attn_bf16_opt_in(int device) {
 }  // namespace
 
 // Work list (items of two query tiles, key blocks of 128) and the static schedules.
-int attn_bf16_prepare(hilberta_plan_t *p) {
+int attn_bf16_prepare(hilberta_plan_t *p, BindImage &image) {
     // Cost of a unit in twentieths of a two-tile key block (about 140 SM cycles), from per-unit cycle
     // counts of the kernel at 1024^2 and 2048^2: two tiles 2760 cycles per block + 5500; one tile --
     // nothing to overlap its softmax with the MMAs -- 2580 per block + 2600, i.e. hardly cheaper.
@@ -1179,16 +1179,6 @@ int attn_bf16_prepare(hilberta_plan_t *p) {
         // the second stream's tile loads.
         cost_two_heads.push_back(it.q_rows > BM ? 0 : (long long)it.kv_blocks * 21 + 40);
     }
-    cudaFree(p->d_work);
-    cudaFree(p->d_units);
-    cudaFree(p->d_cta_begin);
-    cudaFree(p->d_units_chunk);
-    cudaFree(p->d_cta_begin_chunk);
-    p->d_work = nullptr;
-    p->d_units = nullptr;
-    p->d_cta_begin = nullptr;
-    p->d_units_chunk = nullptr;
-    p->d_cta_begin_chunk = nullptr;
     p->n_cta_chunk = 0;
     p->n_work = (int)items.size();
     p->n_cta = 0;
@@ -1209,24 +1199,28 @@ int attn_bf16_prepare(hilberta_plan_t *p) {
     SplitChoice choice;
     choose_split(items, cost, cost_two_heads, p->batch * p->heads, p->sm_count, split_clusters(p->device), BN, choice);
     p->split_cluster = choice.cluster;
-    const int n_whole = (int)items.size();
     for (const WorkItem &it : choice.shares) items.push_back(it);
-    HB_CUDA(cudaMalloc(&p->d_work, sizeof(WorkItem) * items.size()));
-    HB_CUDA(cudaMemcpy(p->d_work, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice));
-    items.resize(n_whole);
-    rc = upload_split_schedule(items, cost, cost_two_heads, p->batch * p->heads, p->sm_count, choice, &p->d_units, &p->d_cta_begin,
-                               &p->n_cta);
+    image.add(items, &p->d_work);
+    rc = add_schedule(image, cost, cost_two_heads, p->batch * p->heads, p->sm_count, choice, &p->d_units,
+                            &p->d_cta_begin, &p->n_cta);
     if (rc != HILBERTA_OK) return rc;
     if (p->chunk_heads < p->heads) {
-        rc = upload_split_schedule(items, cost, cost_two_heads, p->batch * p->chunk_heads, p->sm_count, choice, &p->d_units_chunk,
-                                   &p->d_cta_begin_chunk, &p->n_cta_chunk);
+        rc = add_schedule(image, cost, cost_two_heads, p->batch * p->chunk_heads, p->sm_count, choice,
+                                &p->d_units_chunk, &p->d_cta_begin_chunk, &p->n_cta_chunk);
         if (rc != HILBERTA_OK) return rc;
     }
-    {
-        const int rc_solo = attn_bf16_solo_prepare(p);
-        if (rc_solo != HILBERTA_OK) return rc_solo;
-    }
-    return attn_bf16_pair_prepare(p);
+    // the alternative kernels' tables: only where they are selected
+    if (forward_kernel_choice() == 's') return attn_bf16_solo_prepare(p, image);
+    if (forward_kernel_choice() == 'p') return attn_bf16_pair_prepare(p, image);
+    return HILBERTA_OK;
+}
+
+char forward_kernel_choice() {
+    static const char choice = [] {
+        const char *e = getenv("HILBERTA_FORWARD_KERNEL");
+        return e && (e[0] == 'p' || e[0] == 's') ? e[0] : (char)0;
+    }();
+    return choice;
 }
 
 int launch_attn_bf16(const hilberta_plan_t *p, const void *q, const void *k, const void *v, void *out,
@@ -1235,18 +1229,10 @@ int launch_attn_bf16(const hilberta_plan_t *p, const void *q, const void *k, con
     // bf16 with head dim 128 and inputs in physical order can also run on pairs of SMs
     // (attn_bf16_pair_sm100.cu) or with one query tile per CTA (attn_bf16_solo_sm100.cu).  Those kernels
     // are correct but measure slower than this one, so they are opt-in: the environment variable
-    // HILBERTA_FORWARD_KERNEL=pair or =solo selects them (read once).
-    static const bool use_pair = [] {
-        const char *e = getenv("HILBERTA_FORWARD_KERNEL");
-        return e && e[0] == 'p';
-    }();
-    if (use_pair && !in_map && chunk < 0 && p->n_pair > 0)
+    // HILBERTA_FORWARD_KERNEL=pair or =solo selects them (read once, by the first bind).
+    if (forward_kernel_choice() == 'p' && !in_map && chunk < 0 && p->n_pair > 0)
         return launch_attn_bf16_pair(p, q, k, v, out, lse, out_map, stream);
-    static const bool use_solo = [] {
-        const char *e = getenv("HILBERTA_FORWARD_KERNEL");
-        return e && e[0] == 's';
-    }();
-    if (use_solo && !in_map && chunk < 0 && p->n_solo > 0)
+    if (forward_kernel_choice() == 's' && !in_map && chunk < 0 && p->n_solo > 0)
         return launch_attn_bf16_solo(p, q, k, v, out, lse, out_map, stream);
     int heads = p->heads, n_cta = p->n_cta;
     const WorkUnit *units = p->d_units;

@@ -568,13 +568,7 @@ int make_tensor_map(CUtensorMap *m, const void *base, const hilberta_plan_t *p, 
 
 // Work list (items of 128 rows) and the static schedule.
 // Returns OK and leaves p->n_solo == 0 if this shape is not served by this kernel.
-int attn_bf16_solo_prepare(hilberta_plan_t *p) {
-    cudaFree(p->d_work_solo);
-    cudaFree(p->d_units_solo);
-    cudaFree(p->d_solo_begin);
-    p->d_work_solo = nullptr;
-    p->d_units_solo = nullptr;
-    p->d_solo_begin = nullptr;
+int attn_bf16_solo_prepare(hilberta_plan_t *p, BindImage &image) {
     p->n_solo = 0;
     if (p->dtype != HILBERTA_BF16 || p->head_dim != HD) return HILBERTA_OK;
     {
@@ -597,9 +591,8 @@ int attn_bf16_solo_prepare(hilberta_plan_t *p) {
                      [&](const WorkItem &a, const WorkItem &b) { return cost_of(a) > cost_of(b); });
     std::vector<long long> cost;
     for (const WorkItem &it : items) cost.push_back(cost_of(it));
-    HB_CUDA(cudaMalloc(&p->d_work_solo, sizeof(WorkItem) * items.size()));
-    HB_CUDA(cudaMemcpy(p->d_work_solo, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice));
-    return upload_schedule(items, cost, p->batch * p->heads, p->sm_count, &p->d_units_solo, &p->d_solo_begin, &p->n_solo);
+    image.add(items, &p->d_work_solo);
+    return add_schedule(image, cost, {}, p->batch * p->heads, p->sm_count, SplitChoice(), &p->d_units_solo, &p->d_solo_begin, &p->n_solo);
 }
 
 int launch_attn_bf16_solo(const hilberta_plan_t *p, const void *q, const void *k, const void *v, void *out,

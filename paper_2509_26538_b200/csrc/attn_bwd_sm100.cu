@@ -582,8 +582,8 @@ delta_kernel(const __nv_bfloat16 *__restrict__ dout, const __nv_bfloat16 *__rest
 
 // Work list of the backward kernels: 128 resident rows per item, the rows they exchange
 // gradients with listed as up to three contiguous ranges and counted in blocks of 128.
-// Also allocates the per-row scratch: lse * log2 e for every row, then delta for every row.  Called from hilberta_plan_bind for bf16 bindings.
-int attn_bwd_prepare(hilberta_plan_t *p) {
+// Also asks for the per-row scratch: lse * log2 e for every row, then delta for every row.  Called from hilberta_plan_bind for bf16 bindings.
+int attn_bwd_prepare(hilberta_plan_t *p, BindImage &image) {
     std::vector<WorkItem> items = build_work_items(p, BM, BK);
     {
         const int rc_items = check_work_items(items.data(), (int)items.size(), p->S, BM, BK);
@@ -593,24 +593,15 @@ int attn_bwd_prepare(hilberta_plan_t *p) {
                      [](const WorkItem &a, const WorkItem &b) { return a.kv_blocks > b.kv_blocks; });
     std::vector<long long> cost;
     for (const WorkItem &it : items) cost.push_back((long long)it.kv_blocks + 3);
-    cudaFree(p->d_bwd_work);
-    cudaFree(p->d_bwd_units);
-    cudaFree(p->d_bwd_cta_begin);
-    cudaFree(p->d_delta);
-    p->d_bwd_work = nullptr;
-    p->d_bwd_units = nullptr;
-    p->d_bwd_cta_begin = nullptr;
-    p->d_delta = nullptr;
     p->n_bwd_work = (int)items.size();
     p->n_bwd_cta = 0;
     if (items.empty()) return HILBERTA_OK;
 
     const int bh = p->batch * p->heads;
-    HB_CUDA(cudaMalloc(&p->d_bwd_work, sizeof(WorkItem) * items.size()));
-    HB_CUDA(cudaMemcpy(p->d_bwd_work, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice));
-    const int rc = upload_schedule(items, cost, bh, p->sm_count, &p->d_bwd_units, &p->d_bwd_cta_begin, &p->n_bwd_cta);
+    image.add(items, &p->d_bwd_work);
+    const int rc = add_schedule(image, cost, {}, bh, p->sm_count, SplitChoice(), &p->d_bwd_units, &p->d_bwd_cta_begin, &p->n_bwd_cta);
     if (rc != HILBERTA_OK) return rc;
-    HB_CUDA(cudaMalloc(&p->d_delta, sizeof(float) * 2 * (size_t)bh * p->S));
+    image.add_scratch(2 * (size_t)bh * p->S, &p->d_delta);
     {
         // The shared-memory opt-in is an attribute of the kernel ON ONE DEVICE: set it once for every
         // device a plan is bound on (a failure is reported, not remembered).

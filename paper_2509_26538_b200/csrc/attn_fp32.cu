@@ -182,7 +182,7 @@ attn_fp32_kernel(const float *__restrict__ q, const float *__restrict__ k, const
 // 212; 16 x 16, 2 heads of 64, forward (5) 32 / 20 / 13 / 11; 25 x 34 + 333, 6 heads of 32 (19) 373 / 261 / 291 /
 // 278; 16 x 16 + 128, 16 heads of 128 (7) 235 / 166 / 187 / 236; 35 x 35 + 77, 13 heads of 128 (23) 343 / 350 /
 // 339 / 397.
-int attn_fp32_prepare(hilberta_plan_t *p) {
+int attn_fp32_prepare(hilberta_plan_t *p, BindImage &image) {
     std::vector<WorkItem> items = build_work_items(p, BR, BC);
     const int rc = check_work_items(items.data(), (int)items.size(), p->S, BR, BC);
     if (rc != HILBERTA_OK) return rc;
@@ -200,11 +200,10 @@ int attn_fp32_prepare(hilberta_plan_t *p) {
     if (p->f32_cluster > 1)
         while (p->n_f32_split < (int)items.size() && blocks(items[p->n_f32_split]) > 2) ++p->n_f32_split;
     p->n_f32_work = (int)items.size();
-    cudaFree(p->d_f32_work);
-    p->d_f32_work = nullptr;
     if (items.empty()) return HILBERTA_OK;
-    HB_CUDA(cudaMalloc(&p->d_f32_work, sizeof(WorkItem) * items.size()));
-    HB_CUDA(cudaMemcpy(p->d_f32_work, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice));
+    image.add(items, &p->d_f32_work);
+    // scratch of the backward pass (delta per row; sized like the bf16 path's)
+    image.add_scratch(2 * (size_t)p->batch * p->heads * p->S, &p->d_delta);
     // the shared-memory opt-in is an attribute of the kernel on one device
     static std::mutex attr_mutex;
     static bool attr_done[64] = {};

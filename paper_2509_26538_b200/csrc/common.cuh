@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <atomic>
 #include <vector>
@@ -60,6 +61,33 @@ struct WorkUnit {
     int bh2;
 };
 
+// Tables of a binding, gathered on the host: one allocation and one copy for all of them (every
+// cudaMalloc, cudaFree and pageable copy is tens of microseconds of a bind).  `where` receives the device
+// address; scratch lies behind the tables, uninitialised.
+struct BindImage {
+    std::vector<char> bytes;
+    size_t scratch = 0;
+    struct Place {
+        void **where;
+        size_t at;
+        bool in_scratch;
+    };
+    std::vector<Place> places;
+    static size_t up(size_t n) { return (n + 255) & ~(size_t)255; }
+    template <class T>
+    void add(const std::vector<T> &table, T **where) {
+        const size_t at = bytes.size(), n = sizeof(T) * table.size();
+        bytes.resize(up(at + n));
+        if (n) memcpy(bytes.data() + at, table.data(), n);
+        places.push_back(Place{(void **)where, at, false});
+    }
+    template <class T>
+    void add_scratch(size_t count, T **where) {
+        places.push_back(Place{(void **)where, scratch, true});
+        scratch = up(scratch + sizeof(T) * count);
+    }
+};
+
 }  // namespace hilberta
 
 struct hilberta_plan_s {
@@ -71,7 +99,9 @@ struct hilberta_plan_s {
     bool compact;           // tiles are equal groups over the non-shared tokens (Algorithm 1) instead of curve intervals
     int tile, offset, shared_region, n_text, n_shared, T, S, P;
     uint64_t nnz;
-    // device tables
+    // device tables: two allocations, made by the plan and by its binding; the pointers below point into them
+    void *d_plan, *d_bind;
+    size_t plan_bytes, bind_bytes;
     int *d_hil_d2t, *d_hil_t2d;      // [HW]
     int *d_c;                        // [NP + 1] real non-shared cells with padded Hilbert index below d
     int *d_phys2orig, *d_orig2phys;  // [S]
@@ -147,14 +177,6 @@ int launch_attn_bf16(const hilberta_plan_t *p, const void *q, const void *k, con
 std::vector<WorkItem> build_work_items(const hilberta_plan_t *p, int item_rows, int block);
 // HILBERTA_OK iff the list is safe to hand to a kernel (ranges inside [0, S), rows covered exactly once)
 int check_work_items(const WorkItem *items, int n, int S, int item_rows, int block);
-// the schedule on the host (see hilberta_schedule_units); returns the largest CTA load
-long long build_schedule(int n_items, const long long *cost, const long long *cost_two_heads, int bh, int sm_count,
-                         std::vector<WorkUnit> &units, std::vector<int> &cta_begin);
-// cost_two_heads: nullptr, or per item the cost of running it for TWO (batch, head) indices in one unit
-// (0: the item is not paired); such items are emitted as units of two consecutive indices.
-int upload_schedule(const std::vector<WorkItem> &items, const std::vector<long long> &cost, int bh, int sm_count,
-                    WorkUnit **d_units, int **d_cta_begin, int *n_cta_out,
-                    const std::vector<long long> *cost_two_heads = nullptr);
 // How a schedule cuts its longest items (the first n_items of the list) over clusters of `cluster` CTAs;
 // shares: cluster entries per cut item, in rank order, appended to the uploaded work list.
 struct SplitChoice {
@@ -167,23 +189,26 @@ void choose_split(const std::vector<WorkItem> &items, const std::vector<long lon
                   const std::vector<long long> &cost_two_heads, int bh, int sm_count, const int *clusters, int block,
                   SplitChoice &choice);
 // The schedule of such a choice (units null: none is written); returns the largest CTA load.
-long long build_split_schedule(const std::vector<WorkItem> &items, const std::vector<long long> &cost,
-                               const std::vector<long long> &cost_two_heads, int bh, int sm_count, const SplitChoice &choice,
-                               std::vector<WorkUnit> *units, std::vector<int> *cta_begin);
-int upload_split_schedule(const std::vector<WorkItem> &items, const std::vector<long long> &cost,
-                          const std::vector<long long> &cost_two_heads, int bh, int sm_count, const SplitChoice &choice,
-                          WorkUnit **d_units, int **d_cta_begin, int *n_cta_out);
-int attn_bf16_prepare(hilberta_plan_t *p);
+// cost_two_heads: empty, or per item the cost of running it for TWO (batch, head) indices in one unit
+// (0: the item is not paired); such items become units of two consecutive indices.
+long long build_schedule(const std::vector<long long> &cost, const std::vector<long long> &cost_two_heads, int bh, int sm_count,
+                         const SplitChoice &choice, std::vector<WorkUnit> *units, std::vector<int> *cta_begin);
+int add_schedule(BindImage &image, const std::vector<long long> &cost, const std::vector<long long> &cost_two_heads, int bh,
+                 int sm_count, const SplitChoice &choice, WorkUnit **d_units, int **d_cta_begin, int *n_cta_out);
+// The forward kernel that the environment variable HILBERTA_FORWARD_KERNEL selects, read once: 'p' (pairs
+// of SMs), 's' (one query tile per CTA) or 0 (the default kernel).
+char forward_kernel_choice();
+int attn_bf16_prepare(hilberta_plan_t *p, BindImage &image);
 // attn_bf16_pair_sm100.cu: the forward kernel on pairs of SMs (bf16, head dim 128, inputs in physical order)
-int attn_bf16_pair_prepare(hilberta_plan_t *p);
+int attn_bf16_pair_prepare(hilberta_plan_t *p, BindImage &image);
 int launch_attn_bf16_pair(const hilberta_plan_t *p, const void *q, const void *k, const void *v, void *out,
                           float *lse, const int *out_map, cudaStream_t stream);
 // attn_bf16_solo_sm100.cu: the forward kernel with one query tile per CTA and double-buffered scores
 // (bf16, head dim 128, inputs in physical order)
-int attn_bf16_solo_prepare(hilberta_plan_t *p);
+int attn_bf16_solo_prepare(hilberta_plan_t *p, BindImage &image);
 int launch_attn_bf16_solo(const hilberta_plan_t *p, const void *q, const void *k, const void *v, void *out,
                           float *lse, const int *out_map, cudaStream_t stream);
-int attn_bwd_prepare(hilberta_plan_t *p);
+int attn_bwd_prepare(hilberta_plan_t *p, BindImage &image);
 // dq, dk, dv (bf16, physical order, the bound strides) from dout, q, k, v, out and the forward's lse.
 int launch_attn_bwd(const hilberta_plan_t *p, const void *dout, const void *q, const void *k, const void *v,
                     const void *out, const float *lse, void *dq, void *dk, void *dv, float *delta,
@@ -191,7 +216,7 @@ int launch_attn_bwd(const hilberta_plan_t *p, const void *dout, const void *q, c
 int launch_attn_fp32_bwd(const hilberta_plan_t *p, const void *dout, const void *q, const void *k, const void *v,
                          const void *out, const float *lse, void *dq, void *dk, void *dv, float *delta,
                          cudaStream_t stream);
-int attn_fp32_prepare(hilberta_plan_t *p);
+int attn_fp32_prepare(hilberta_plan_t *p, BindImage &image);
 int attn_fp32_bwd_opt_in();   // shared-memory opt-in of the fp32 backward kernels on the current device
 int launch_timeout_probe(const hilberta_plan_t *p, cudaStream_t stream);
 // plan.cu: does a written tensor share a byte with another tensor of the bound layout?

@@ -2,6 +2,7 @@
 // kernels), plus the plan object's host-side life cycle and table export.
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 
 #include "common.cuh"
@@ -43,8 +44,8 @@ __device__ __forceinline__ int hilbert2d_index(int k, int row, int col) {
     return d;
 }
 
-__global__ void hilbert_lut_kernel(int k, int H, int W, int *__restrict__ cell_of_pd,
-                                   int *__restrict__ pd_of_cell, unsigned char *__restrict__ kind_by_pd,
+__global__ void hilbert_lut_kernel(int k, int H, int W, int *__restrict__ pd_of_cell,
+                                   unsigned char *__restrict__ kind_by_pd,
                                    int sh_r0, int sh_c0, int sh_side) {
     const int n = 1 << k;
     const int pc = blockIdx.x * blockDim.x + threadIdx.x;   // padded cell
@@ -54,11 +55,9 @@ __global__ void hilbert_lut_kernel(int k, int H, int W, int *__restrict__ cell_o
     if (row < H && col < W) {
         const int cell = row * W + col;
         pd_of_cell[cell] = d;
-        cell_of_pd[d] = cell;
         const bool sh = row >= sh_r0 && row < sh_r0 + sh_side && col >= sh_c0 && col < sh_c0 + sh_side;
         kind_by_pd[d] = sh ? CELL_SHARED : CELL_REAL;
     } else {
-        cell_of_pd[d] = -1;
         kind_by_pd[d] = CELL_PAD;
     }
 }
@@ -107,8 +106,8 @@ __device__ __forceinline__ int hilbert3d_index(int k, int f, int row, int col) {
     return d;
 }
 
-__global__ void hilbert3d_lut_kernel(int a, int b, int F, int H, int W, int *__restrict__ cell_of_pd,
-                                     int *__restrict__ pd_of_cell, unsigned char *__restrict__ kind_by_pd,
+__global__ void hilbert3d_lut_kernel(int a, int b, int F, int H, int W, int *__restrict__ pd_of_cell,
+                                     unsigned char *__restrict__ kind_by_pd,
                                      int sh_f0, int sh_r0, int sh_c0, int sh_side, int sh_frames) {
     const int side = a >= b ? a : b;         // log2 of the padded image side
     const int pc = blockIdx.x * blockDim.x + threadIdx.x;   // padded cell, frame-major
@@ -124,12 +123,10 @@ __global__ void hilbert3d_lut_kernel(int a, int b, int F, int H, int W, int *__r
     if (f < F && row < H && col < W) {
         const int cell = (f * H + row) * W + col;
         pd_of_cell[cell] = d;
-        cell_of_pd[d] = cell;
         const bool sh = f >= sh_f0 && f < sh_f0 + sh_frames && row >= sh_r0 && row < sh_r0 + sh_side &&
                         col >= sh_c0 && col < sh_c0 + sh_side;
         kind_by_pd[d] = sh ? CELL_SHARED : CELL_REAL;
     } else {
-        cell_of_pd[d] = -1;
         kind_by_pd[d] = CELL_PAD;
     }
 }
@@ -273,135 +270,174 @@ __global__ void window_compact_kernel(int R, int groups, int size, int offset, i
     win[w] = r;
 }
 
+// Device blocks of destroyed plans and replaced bindings, kept for the next ones: allocating and freeing a
+// plan's two blocks took 0.6 ms of the 1.2 ms of a plan, bind and destroy at 1024^2.  At most 16 blocks and
+// 64 MB; beyond that, and when an allocation fails, they go back to the device.  A block is put aside only after
+// the device has finished all work (which cudaFree would have waited for as well), so its next owner may be
+// on any stream.
+namespace {
+struct Block {
+    int device;
+    void *ptr;
+    size_t bytes;
+};
+std::mutex g_blocks_mutex;
+std::vector<Block> &g_blocks = *new std::vector<Block>();   // never destroyed: plans may go after the statics
+constexpr size_t kKeepBlocks = 16, kKeepBytes = 64u << 20;
+
+struct OnDevice {
+    int before = -1, device;
+    explicit OnDevice(int d) : device(d) {
+        cudaGetDevice(&before);
+        if (before != device) cudaSetDevice(device);
+    }
+    ~OnDevice() {
+        if (before != device && before >= 0) cudaSetDevice(before);
+    }
+};
+
+// bytes: wanted; on return the size of the block
+cudaError_t take_block(int device, void **ptr, size_t *bytes) {
+    *bytes = (*bytes + 65535) & ~(size_t)65535;
+    {
+        std::lock_guard<std::mutex> lock(g_blocks_mutex);
+        size_t best = g_blocks.size();
+        for (size_t i = 0; i < g_blocks.size(); ++i)
+            if (g_blocks[i].device == device && g_blocks[i].bytes >= *bytes && g_blocks[i].bytes <= 2 * *bytes + (1u << 20) &&
+                (best == g_blocks.size() || g_blocks[i].bytes < g_blocks[best].bytes))
+                best = i;
+        if (best < g_blocks.size()) {
+            *ptr = g_blocks[best].ptr;
+            *bytes = g_blocks[best].bytes;
+            g_blocks.erase(g_blocks.begin() + (long)best);
+            return cudaSuccess;
+        }
+    }
+    const OnDevice on(device);
+    cudaError_t e = cudaMalloc(ptr, *bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();   // not the caller's business if the second try succeeds
+        {
+            std::lock_guard<std::mutex> lock(g_blocks_mutex);
+            for (const Block &b : g_blocks) cudaFree(b.ptr);
+            g_blocks.clear();
+        }
+        e = cudaMalloc(ptr, *bytes);
+    }
+    return e;
+}
+
+void give_block(int device, void *ptr, size_t bytes) {
+    if (!ptr) return;
+    const OnDevice on(device);
+    const bool idle = cudaDeviceSynchronize() == cudaSuccess;
+    if (idle) {
+        std::lock_guard<std::mutex> lock(g_blocks_mutex);
+        size_t held = bytes;
+        for (const Block &b : g_blocks) held += b.bytes;
+        if (held <= kKeepBytes && g_blocks.size() < kKeepBlocks) {
+            g_blocks.push_back(Block{device, ptr, bytes});
+            return;
+        }
+    }
+    cudaFree(ptr);
+}
+}  // namespace
+
 static void free_plan(hilberta_plan_t *p) {
     if (!p) return;
-    cudaFree(p->d_hil_d2t);
-    cudaFree(p->d_hil_t2d);
-    cudaFree(p->d_c);
-    cudaFree(p->d_phys2orig);
-    cudaFree(p->d_orig2phys);
-    cudaFree(p->d_row_window);
-    cudaFree(p->d_windows);
-    cudaFree(p->d_work);
-    cudaFree(p->d_units);
-    cudaFree(p->d_cta_begin);
-    cudaFree(p->d_units_chunk);
-    cudaFree(p->d_work_pair);
-    cudaFree(p->d_units_pair);
-    cudaFree(p->d_pair_begin);
-    cudaFree(p->d_work_solo);
-    cudaFree(p->d_units_solo);
-    cudaFree(p->d_solo_begin);
-    cudaFree(p->d_cta_begin_chunk);
+    give_block(p->device, p->d_plan, p->plan_bytes);
+    give_block(p->device, p->d_bind, p->bind_bytes);
     for (cudaEvent_t e : p->ev_in) cudaEventDestroy(e);
     for (cudaEvent_t e : p->ev_done) cudaEventDestroy(e);
     if (p->s_in) cudaStreamDestroy(p->s_in);
     if (p->s_out) cudaStreamDestroy(p->s_out);
-    cudaFree(p->d_bwd_work);
-    cudaFree(p->d_bwd_units);
-    cudaFree(p->d_bwd_cta_begin);
-    cudaFree(p->d_delta);
-    cudaFree(p->d_f32_work);
-    cudaFree(p->d_status);
     cudaFree(p->ws);
     delete p;
 }
 
+// All tables in one allocation: each cudaMalloc and cudaFree is tens of microseconds.  The windows and the
+// kinds of the cells lie side by side and come back to the host in one copy, which also waits for the
+// kernels.
 static int build_plan(hilberta_plan_t *p) {
     const int HW = p->HW, S = p->S, NP = p->NP;
-    unsigned char *d_kind = nullptr;
-    int *d_cell_of_pd = nullptr, *d_pd_of_cell = nullptr, *d_c_real = nullptr;
-    HB_CUDA(cudaMalloc(&p->d_hil_d2t, sizeof(int) * HW));
-    HB_CUDA(cudaMalloc(&p->d_hil_t2d, sizeof(int) * HW));
-    HB_CUDA(cudaMalloc(&p->d_c, sizeof(int) * (NP + 1)));
-    HB_CUDA(cudaMalloc(&p->d_phys2orig, sizeof(int) * S));
-    HB_CUDA(cudaMalloc(&p->d_orig2phys, sizeof(int) * S));
-    HB_CUDA(cudaMalloc(&p->d_row_window, sizeof(int) * S));
-    HB_CUDA(cudaMalloc(&p->d_windows, sizeof(Window) * p->T));
-    HB_CUDA(cudaMalloc(&p->d_status, sizeof(int) * 4096));
-    HB_CUDA(cudaMemset(p->d_status, 0, sizeof(int) * 4096));
+    size_t bytes = 0;
+    auto place = [&](size_t n) {
+        const size_t at = bytes;
+        bytes = (bytes + n + 255) & ~(size_t)255;
+        return at;
+    };
+    const size_t windows = sizeof(Window) * p->T;
+    const size_t o_d2t = place(sizeof(int) * HW), o_t2d = place(sizeof(int) * HW), o_c = place(sizeof(int) * (NP + 1));
+    const size_t o_p2o = place(sizeof(int) * S), o_o2p = place(sizeof(int) * S), o_rw = place(sizeof(int) * S);
+    const size_t o_status = place(sizeof(int) * 4096), o_win = place(windows + (size_t)NP), o_kind = o_win + windows;
+    const size_t o_pd = place(sizeof(int) * HW), o_real = place(sizeof(int) * (NP + 1));   // needed here only
+    p->plan_bytes = bytes;
+    HB_CUDA(take_block(p->device, &p->d_plan, &p->plan_bytes));
+    char *base = (char *)p->d_plan;
+    p->d_hil_d2t = (int *)(base + o_d2t);
+    p->d_hil_t2d = (int *)(base + o_t2d);
+    p->d_c = (int *)(base + o_c);
+    p->d_phys2orig = (int *)(base + o_p2o);
+    p->d_orig2phys = (int *)(base + o_o2p);
+    p->d_row_window = (int *)(base + o_rw);
+    p->d_status = (int *)(base + o_status);
+    p->d_windows = (Window *)(base + o_win);
+    unsigned char *d_kind = (unsigned char *)(base + o_kind);
+    int *d_pd_of_cell = (int *)(base + o_pd), *d_c_real = (int *)(base + o_real);
+    HB_CUDA(cudaMemsetAsync(p->d_status, 0, sizeof(int) * 4096, 0));
 
     const int sh_r0 = p->H / 2 - p->shared_region / 2;
     const int sh_c0 = p->W / 2 - p->shared_region / 2;
-    int rc = HILBERTA_OK;
-    do {
-        cudaError_t e = cudaMalloc(&d_kind, NP);
-        if (e == cudaSuccess) e = cudaMalloc(&d_cell_of_pd, sizeof(int) * NP);
-        if (e == cudaSuccess) e = cudaMalloc(&d_pd_of_cell, sizeof(int) * HW);
-        if (e == cudaSuccess) e = cudaMalloc(&d_c_real, sizeof(int) * (NP + 1));
-        if (e != cudaSuccess) {
-            g_last_cuda_error = (int)e;
-            rc = HILBERTA_ERR_CUDA;
-            break;
+    if (p->frames > 1)
+        hilbert3d_lut_kernel<<<(NP + 255) / 256, 256>>>(p->ka_log2, p->kb_log2, p->frames, p->H, p->W, d_pd_of_cell, d_kind,
+                                                        p->frames / 2 - p->shared_frames / 2, sh_r0, sh_c0,
+                                                        p->shared_region, p->shared_frames);
+    else
+        hilbert_lut_kernel<<<(NP + 255) / 256, 256>>>(p->k_log2, p->H, p->W, d_pd_of_cell, d_kind, sh_r0, sh_c0,
+                                                      p->shared_region);
+    g_launches.fetch_add(1);
+    cell_scan_kernel<<<1, 1024>>>(d_kind, NP, p->d_c, d_c_real);
+    g_launches.fetch_add(1);
+    layout_kernel<<<(S + 255) / 256, 256>>>(HW, NP, p->n_text, p->P, p->tile, p->offset, p->compact ? S - p->P : 0,
+                                            d_pd_of_cell, p->d_c, d_c_real, d_kind, p->d_hil_d2t, p->d_hil_t2d,
+                                            p->d_phys2orig, p->d_orig2phys, p->d_row_window);
+    g_launches.fetch_add(1);
+    if (p->compact)
+        window_compact_kernel<<<(p->T + 127) / 128, 128>>>(S - p->P, p->T, p->tile, p->offset, p->P, p->d_windows);
+    else
+        window_kernel<<<(p->T + 127) / 128, 128>>>(NP, p->T, p->tile, p->offset, p->P, p->d_c, p->d_windows);
+    g_launches.fetch_add(1);
+    HB_CUDA(cudaGetLastError());
+    // host mirrors of the small tables
+    std::vector<char> back(windows + (size_t)NP);
+    HB_CUDA(cudaMemcpy(back.data(), p->d_windows, back.size(), cudaMemcpyDeviceToHost));
+    p->h_windows.resize(p->T);
+    memcpy(p->h_windows.data(), back.data(), windows);
+    const unsigned char *h_kind = (const unsigned char *)back.data() + windows;
+    int n_sh = 0;
+    for (int d = 0; d < NP; ++d) {
+        if (h_kind[d] != CELL_SHARED) continue;
+        ++n_sh;
+        size_t n = p->h_shared_runs.size();
+        if (n && p->h_shared_runs[n - 2] + p->h_shared_runs[n - 1] == d) {
+            p->h_shared_runs[n - 1] += 1;
+        } else {
+            p->h_shared_runs.push_back(d);
+            p->h_shared_runs.push_back(1);
         }
-        if (p->frames > 1)
-            hilbert3d_lut_kernel<<<(NP + 255) / 256, 256>>>(p->ka_log2, p->kb_log2, p->frames, p->H, p->W, d_cell_of_pd,
-                                                            d_pd_of_cell, d_kind, p->frames / 2 - p->shared_frames / 2,
-                                                            sh_r0, sh_c0, p->shared_region, p->shared_frames);
-        else
-            hilbert_lut_kernel<<<(NP + 255) / 256, 256>>>(p->k_log2, p->H, p->W, d_cell_of_pd, d_pd_of_cell, d_kind,
-                                                          sh_r0, sh_c0, p->shared_region);
-        g_launches.fetch_add(1);
-        cell_scan_kernel<<<1, 1024>>>(d_kind, NP, p->d_c, d_c_real);
-        g_launches.fetch_add(1);
-        layout_kernel<<<(S + 255) / 256, 256>>>(HW, NP, p->n_text, p->P, p->tile, p->offset,
-                                                p->compact ? S - p->P : 0, d_pd_of_cell, p->d_c,
-                                                d_c_real, d_kind, p->d_hil_d2t, p->d_hil_t2d, p->d_phys2orig,
-                                                p->d_orig2phys, p->d_row_window);
-        g_launches.fetch_add(1);
-        if (p->compact)
-            window_compact_kernel<<<(p->T + 127) / 128, 128>>>(S - p->P, p->T, p->tile, p->offset, p->P, p->d_windows);
-        else
-            window_kernel<<<(p->T + 127) / 128, 128>>>(NP, p->T, p->tile, p->offset, p->P, p->d_c, p->d_windows);
-        g_launches.fetch_add(1);
-        e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaDeviceSynchronize();
-        if (e != cudaSuccess) {
-            g_last_cuda_error = (int)e;
-            rc = HILBERTA_ERR_CUDA;
-            break;
-        }
-        // host mirrors of the small tables
-        p->h_windows.resize(p->T);
-        std::vector<unsigned char> h_kind(NP);
-        e = cudaMemcpy(p->h_windows.data(), p->d_windows, sizeof(Window) * p->T, cudaMemcpyDeviceToHost);
-        if (e == cudaSuccess) e = cudaMemcpy(h_kind.data(), d_kind, NP, cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) {
-            g_last_cuda_error = (int)e;
-            rc = HILBERTA_ERR_CUDA;
-            break;
-        }
-        int n_sh = 0;
-        for (int d = 0; d < NP; ++d) {
-            if (h_kind[d] != CELL_SHARED) continue;
-            ++n_sh;
-            size_t n = p->h_shared_runs.size();
-            if (n && p->h_shared_runs[n - 2] + p->h_shared_runs[n - 1] == d) {
-                p->h_shared_runs[n - 1] += 1;
-            } else {
-                p->h_shared_runs.push_back(d);
-                p->h_shared_runs.push_back(1);
-            }
-        }
-        if (n_sh != p->n_shared) {
-            rc = HILBERTA_ERR_INVALID;  // cannot happen for validated arguments
-            break;
-        }
-        // kept pairs: prefix rows see everything; other rows see the prefix and
-        // the non-shared members of their own slid tile
-        const uint64_t Pq = (uint64_t)p->P, Sq = (uint64_t)S;
-        uint64_t nnz = Pq * Sq;
-        for (const Window &w : p->h_windows) {
-            const uint64_t r = (uint64_t)w.seg0_len + (uint64_t)w.seg1_len;
-            nnz += r * (Pq + r);
-        }
-        p->nnz = nnz;
-    } while (0);
-    cudaFree(d_kind);
-    cudaFree(d_cell_of_pd);
-    cudaFree(d_pd_of_cell);
-    cudaFree(d_c_real);
-    return rc;
+    }
+    if (n_sh != p->n_shared) return HILBERTA_ERR_INVALID;  // cannot happen for validated arguments
+    // kept pairs: prefix rows see everything; other rows see the prefix and
+    // the non-shared members of their own slid tile
+    const uint64_t Pq = (uint64_t)p->P, Sq = (uint64_t)S;
+    uint64_t nnz = Pq * Sq;
+    for (const Window &w : p->h_windows) {
+        const uint64_t r = (uint64_t)w.seg0_len + (uint64_t)w.seg1_len;
+        nnz += r * (Pq + r);
+    }
+    p->nnz = nnz;
+    return HILBERTA_OK;
 }
 
 }  // namespace hilberta
@@ -456,14 +492,15 @@ static int make_plan(int frames, int H, int W, int tile, int groups, int layer_o
 
     int dev = 0;
     HB_CUDA(cudaGetDevice(&dev));
-    cudaDeviceProp prop;
-    HB_CUDA(cudaGetDeviceProperties(&prop, dev));
-    if (prop.major != 10) return HILBERTA_ERR_ARCH;
+    int major = 0, sm_count = 0;   // two attributes: the whole property struct takes milliseconds to fill
+    HB_CUDA(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
+    HB_CUDA(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev));
+    if (major != 10) return HILBERTA_ERR_ARCH;
 
     hilberta_plan_t *p = new (std::nothrow) hilberta_plan_t();
     if (!p) return HILBERTA_ERR_NOMEM;
     p->device = dev;
-    p->sm_count = prop.multiProcessorCount;
+    p->sm_count = sm_count;
     p->frames = frames;
     p->shared_frames = frames > 1 ? shared_frames : 0;
     p->H = H;
@@ -602,25 +639,26 @@ extern "C" int hilberta_plan_bind(hilberta_plan_t *p, int batch, int heads, int 
     p->stride_h = stride_h;
     p->stride_s = stride_s;
     p->scale = scale > 0.f ? scale : 1.0f / sqrtf((float)head_dim);
-    if (dtype == HILBERTA_BF16) {
-        int rc = attn_bf16_prepare(p);
-        if (rc != HILBERTA_OK) return rc;
-        rc = attn_bwd_prepare(p);
-        if (rc != HILBERTA_OK) return rc;
-    }
-    if (dtype == HILBERTA_FP8_E4M3) {
-        // forward only: the bf16 kernel's work list and schedule, no backward tables
-        int rc = attn_bf16_prepare(p);
-        if (rc != HILBERTA_OK) return rc;
-    }
+    give_block(p->device, p->d_bind, p->bind_bytes);   // waits for launches that still read the old tables
+    p->d_bind = nullptr;
+    BindImage image;
+    int rc = HILBERTA_OK;
     if (dtype == HILBERTA_FP32) {
-        // scratch of the backward pass (delta per row; sized like the bf16 path's)
-        cudaFree(p->d_delta);
-        p->d_delta = nullptr;
-        HB_CUDA(cudaMalloc(&p->d_delta, sizeof(float) * 2 * (size_t)batch * heads * p->S));
-        const int rc = attn_fp32_prepare(p);
-        if (rc != HILBERTA_OK) return rc;
+        rc = attn_fp32_prepare(p, image);
+    } else {
+        rc = attn_bf16_prepare(p, image);
+        // e4m3 bindings are forward only: no backward tables
+        if (rc == HILBERTA_OK && dtype == HILBERTA_BF16) rc = attn_bwd_prepare(p, image);
     }
+    if (rc != HILBERTA_OK) return rc;
+    const size_t total = image.bytes.size() + image.scratch;
+    if (total) {
+        p->bind_bytes = total;
+        HB_CUDA(take_block(p->device, &p->d_bind, &p->bind_bytes));
+        HB_CUDA(cudaMemcpy(p->d_bind, image.bytes.data(), image.bytes.size(), cudaMemcpyHostToDevice));
+    }
+    for (const BindImage::Place &at : image.places)
+        *at.where = (char *)p->d_bind + at.at + (at.in_scratch ? image.bytes.size() : 0);
     p->bound = true;
     return HILBERTA_OK;
 }
@@ -635,11 +673,10 @@ static bool layouts_overlap(uint64_t a, uint64_t b, int batch, int heads, int S,
                             int64_t row_bytes) {
     if (batch < 1 || heads < 1 || S < 1 || row_bytes < 1) return false;
     const int64_t d = (int64_t)(b - a);
-    if (ss <= 0) {
-        // no usable token stride: compare the address ranges
-        const int64_t ext = (batch - 1) * llabs(sb) + (heads - 1) * llabs(sh) + (int64_t)(S - 1) * llabs(ss) + row_bytes;
-        return d < ext && -d < ext;
-    }
+    // disjoint address ranges, the usual case, need no search (18 x 47 steps in a backward call of 24 heads)
+    const int64_t ext = (batch - 1) * llabs(sb) + (heads - 1) * llabs(sh) + (int64_t)(S - 1) * llabs(ss) + row_bytes;
+    if (d >= ext || -d >= ext) return false;
+    if (ss <= 0) return true;   // no usable token stride: the address ranges decide
     for (int dx = -(batch - 1); dx <= batch - 1; ++dx)
         for (int dy = -(heads - 1); dy <= heads - 1; ++dy) {
             const int64_t rem = d - dx * sb - dy * sh;

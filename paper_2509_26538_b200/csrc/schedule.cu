@@ -8,7 +8,6 @@
 // the host, longest units first onto the least-loaded CTA, and stored grouped by CTA.
 #include <algorithm>
 #include <functional>
-#include <queue>
 #include <utility>
 
 #include "common.cuh"
@@ -86,69 +85,6 @@ int check_work_items(const WorkItem *items, int n, int S, int item_rows, int blo
     return next == S ? HILBERTA_OK : HILBERTA_ERR_INVALID;
 }
 
-// The static schedule on the host: every (item, batch * head) unit -- items with a two-head cost as
-// units of two consecutive indices -- goes, longest first, to the CTA with the smallest load so far.
-// units: grouped by CTA; cta_begin: n_cta + 1 offsets.  Returns the largest CTA load.
-long long build_schedule(int n_items, const long long *cost, const long long *cost_two_heads, int bh, int sm_count,
-                         std::vector<WorkUnit> &units, std::vector<int> &cta_begin) {
-    struct Costed {
-        WorkUnit unit;
-        long long cost;
-    };
-    std::vector<Costed> all;
-    all.reserve((size_t)n_items * (size_t)bh);
-    for (int i = 0; i < n_items; ++i) {
-        const long long two = cost_two_heads ? cost_two_heads[i] : 0;
-        int j = 0;
-        if (two > 0)
-            for (; j + 1 < bh; j += 2) all.push_back(Costed{WorkUnit{i, j, j + 1}, two});
-        for (; j < bh; ++j) all.push_back(Costed{WorkUnit{i, j, -1}, cost[i]});
-    }
-    // paired units may cost more than the single units of an earlier item, hence the sort (stable:
-    // equal costs keep the order of the items and of the heads)
-    std::stable_sort(all.begin(), all.end(), [](const Costed &a, const Costed &b) { return a.cost > b.cost; });
-    const long long n_units = (long long)all.size();
-    const int n_cta = (int)std::min<long long>(n_units, sm_count);
-    std::vector<std::vector<WorkUnit>> bins((size_t)std::max(n_cta, 0));
-    typedef std::pair<long long, int> Load;  // (load, cta)
-    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> heap;
-    for (int c = 0; c < n_cta; ++c) heap.push(Load(0, c));
-    long long makespan = 0;
-    for (const Costed &cu : all) {
-        Load top = heap.top();
-        heap.pop();
-        bins[top.second].push_back(cu.unit);
-        heap.push(Load(top.first + cu.cost, top.second));
-        makespan = std::max(makespan, top.first + cu.cost);
-    }
-    units.clear();
-    units.reserve((size_t)n_units);
-    cta_begin.assign((size_t)n_cta + 1, 0);
-    for (int c = 0; c < n_cta; ++c) {
-        cta_begin[c] = (int)units.size();
-        units.insert(units.end(), bins[c].begin(), bins[c].end());
-    }
-    cta_begin[n_cta] = (int)units.size();
-    return makespan;
-}
-
-// items must be sorted by descending cost.  On success *d_units holds the units grouped by CTA and
-// *d_cta_begin the n_cta + 1 offsets (both device memory, owned by the caller).
-int upload_schedule(const std::vector<WorkItem> &items, const std::vector<long long> &cost, int bh, int sm_count,
-                    WorkUnit **d_units, int **d_cta_begin, int *n_cta_out, const std::vector<long long> *cost_two_heads) {
-    if ((long long)items.size() * bh > (1ll << 30)) return HILBERTA_ERR_INVALID;
-    std::vector<WorkUnit> units;
-    std::vector<int> cta_begin;
-    build_schedule((int)items.size(), cost.data(), cost_two_heads ? cost_two_heads->data() : nullptr, bh, sm_count, units,
-                   cta_begin);
-    *n_cta_out = (int)cta_begin.size() - 1;
-    HB_CUDA(cudaMalloc(d_units, sizeof(WorkUnit) * units.size()));
-    HB_CUDA(cudaMemcpy(*d_units, units.data(), sizeof(WorkUnit) * units.size(), cudaMemcpyHostToDevice));
-    HB_CUDA(cudaMalloc(d_cta_begin, sizeof(int) * cta_begin.size()));
-    HB_CUDA(cudaMemcpy(*d_cta_begin, cta_begin.data(), sizeof(int) * cta_begin.size(), cudaMemcpyHostToDevice));
-    return HILBERTA_OK;
-}
-
 // ---------------------------------------------------------------------------
 // Items cut over clusters.  A prefix item's key list is the whole sequence; with few heads a handful of
 // them outlasts everything else (3 heads at 2048^2: 9 units of 132 blocks against 26 blocks per SM of
@@ -160,38 +96,39 @@ int upload_schedule(const std::vector<WorkItem> &items, const std::vector<long l
 // B200: 22.7 us uncut, 21.3 in shares of two and 20.8 in shares of four, i.e. 6 and 8 us a merge.
 static long long merge_cost(int cluster) { return cluster == 2 ? 85 : cluster == 4 ? 110 : 135; }
 
-// Greedy assignment to the least loaded of n machines: loads and machine numbers in one heap of 64-bit
-// keys (load, then number, smallest first).
+// Greedy assignment to the least loaded of n machines (of equally loaded ones the lowest number).
 struct LeastLoaded {
-    std::vector<uint64_t> heap;
+    typedef std::pair<long long, int> Load;   // (load, machine)
+    std::vector<Load> heap;
     explicit LeastLoaded(const std::vector<long long> &load) {
-        for (size_t i = 0; i < load.size(); ++i) heap.push_back(((uint64_t)load[i] << 16) | i);
-        std::make_heap(heap.begin(), heap.end(), std::greater<uint64_t>());
+        for (size_t i = 0; i < load.size(); ++i) heap.push_back(Load(load[i], (int)i));
+        std::make_heap(heap.begin(), heap.end(), std::greater<Load>());
     }
-    // adds `cost` to the least loaded machine; returns (its new load, its number)
-    std::pair<long long, int> add(long long cost) {
+    // adds `cost` to the least loaded machine; returns its new load and its number
+    Load add(long long cost) {
         const size_t n = heap.size();
-        const uint64_t top = heap[0] + ((uint64_t)cost << 16);
+        const Load top(heap[0].first + cost, heap[0].second);
         size_t i = 0;
         for (;;) {   // sift the grown top down
             size_t c = 2 * i + 1;
             if (c >= n) break;
             if (c + 1 < n && heap[c + 1] < heap[c]) ++c;
-            if (heap[c] >= top) break;
+            if (!(heap[c] < top)) break;
             heap[i] = heap[c];
             i = c;
         }
         heap[i] = top;
-        return std::make_pair((long long)(top >> 16), (int)(top & 0xffff));
+        return top;
     }
 };
 
-// Every rank's list starts with the cut units of its cluster, in the same order; the other units go,
-// longest first, to the least loaded CTA.  units == nullptr: the largest load only.
-long long build_split_schedule(const std::vector<WorkItem> &items, const std::vector<long long> &cost,
-                               const std::vector<long long> &cost_two_heads, int bh, int sm_count, const SplitChoice &ch,
-                               std::vector<WorkUnit> *units, std::vector<int> *cta_begin) {
-    const int C = ch.cluster;
+// The static schedule on the host: every (item, batch * head) unit -- items with a two-head cost as units of
+// two consecutive indices -- goes, longest first, to the CTA with the smallest load so far.  With cut items
+// every rank's list starts with the cut units of its cluster, in the same order.  units: grouped by CTA;
+// cta_begin: n_cta + 1 offsets; both null: only the largest CTA load is wanted, which is returned.
+long long build_schedule(const std::vector<long long> &cost, const std::vector<long long> &cost_two_heads, int bh, int sm_count,
+                         const SplitChoice &ch, std::vector<WorkUnit> *units, std::vector<int> *cta_begin) {
+    const int C = ch.cluster, n_items = (int)cost.size();
     // runs of equal units: of item i, for two heads each or for one, from head `first` on
     struct Run {
         long long cost;
@@ -199,8 +136,8 @@ long long build_split_schedule(const std::vector<WorkItem> &items, const std::ve
     };
     std::vector<Run> runs;
     long long n_units = (long long)ch.n_items * bh * C;
-    for (int i = ch.n_items; i < (int)items.size(); ++i) {
-        const long long two = ch.pair_heads ? cost_two_heads[i] : 0;
+    for (int i = ch.n_items; i < n_items; ++i) {
+        const long long two = ch.pair_heads && !cost_two_heads.empty() ? cost_two_heads[i] : 0;
         int j = 0;
         if (two > 0 && bh > 1) {
             runs.push_back(Run{two, i, 0, bh / 2, 2});
@@ -224,12 +161,12 @@ long long build_split_schedule(const std::vector<WorkItem> &items, const std::ve
         LeastLoaded clusters(std::vector<long long>((size_t)(n_cta / C), 0));
         for (int i = 0; i < ch.n_items; ++i)
             for (int j = 0; j < bh; ++j) {
-                const std::pair<long long, int> at = clusters.add((cost[i] + C - 1) / C + merge_cost(C));
+                const LeastLoaded::Load at = clusters.add((cost[i] + C - 1) / C + merge_cost(C));
                 makespan = std::max(makespan, at.first);
                 for (int r = 0; r < C; ++r) {
                     load[(size_t)(at.second * C + r)] = at.first;
                     if (units) {
-                        order.push_back(WorkUnit{(int)items.size() + i * C + r, j, -2});
+                        order.push_back(WorkUnit{n_items + i * C + r, j, -2});
                         cta_of.push_back(at.second * C + r);
                     }
                 }
@@ -238,7 +175,7 @@ long long build_split_schedule(const std::vector<WorkItem> &items, const std::ve
     LeastLoaded ctas(load);
     for (const Run &run : runs)
         for (int k = 0; k < run.count; ++k) {
-            const std::pair<long long, int> at = ctas.add(run.cost);
+            const LeastLoaded::Load at = ctas.add(run.cost);
             makespan = std::max(makespan, at.first);
             if (units) {
                 const int j = run.first + k * run.step;
@@ -287,7 +224,7 @@ void choose_split(const std::vector<WorkItem> &items, const std::vector<long lon
         n_units += bh - pairs;
     }
     auto load_of = [&](const SplitChoice &c) {
-        return build_split_schedule(items, cost, cost_two_heads, bh, sm_count, c, nullptr, nullptr);
+        return build_schedule(cost, cost_two_heads, bh, sm_count, c, nullptr, nullptr);
     };
     long long best = load_of(choice);
     // within 3 % of a perfect balance nothing is to be gained
@@ -311,11 +248,17 @@ void choose_split(const std::vector<WorkItem> &items, const std::vector<long lon
         c.n_clusters = clusters[k];
         // cut the items of the longest, of the two longest, ... lengths; every share gets a block at least
         int levels = 0;
+        long long rest = total, cut = 0;   // of the uncut units; of all shares
         for (int n = 1; n <= (int)items.size() && levels < (n_units > 16ll * sm_count ? 1 : 4); ++n) {
             if (items[n - 1].kv_blocks < C) break;
+            const int pairs = cost_two_heads[n - 1] > 0 ? bh / 2 : 0;
+            rest -= cost_two_heads[n - 1] * pairs + cost[n - 1] * (bh - 2 * pairs);
+            cut += ((cost[n - 1] + C - 1) / C + merge_cost(C)) * C * bh;
             if (n < (int)items.size() && items[n].kv_blocks == items[n - 1].kv_blocks) continue;
             ++levels;
             c.n_items = n;
+            // not even in perfect balance
+            if (!few && (rest + cut) / ((long long)c.n_clusters * C) >= best) continue;
             for (int pair = 1; pair >= (few ? 0 : 1); --pair) {
                 c.pair_heads = pair != 0;
                 const long long m = load_of(c);
@@ -335,18 +278,16 @@ void choose_split(const std::vector<WorkItem> &items, const std::vector<long lon
     }
 }
 
-int upload_split_schedule(const std::vector<WorkItem> &items, const std::vector<long long> &cost,
-                          const std::vector<long long> &cost_two_heads, int bh, int sm_count, const SplitChoice &choice,
-                          WorkUnit **d_units, int **d_cta_begin, int *n_cta_out) {
-    if ((long long)items.size() * bh > (1ll << 30)) return HILBERTA_ERR_INVALID;
+// Adds the units grouped by CTA and the n_cta + 1 offsets to the image.
+int add_schedule(BindImage &image, const std::vector<long long> &cost, const std::vector<long long> &cost_two_heads, int bh,
+                 int sm_count, const SplitChoice &choice, WorkUnit **d_units, int **d_cta_begin, int *n_cta_out) {
+    if ((long long)cost.size() * bh > (1ll << 30)) return HILBERTA_ERR_INVALID;
     std::vector<WorkUnit> units;
     std::vector<int> cta_begin;
-    build_split_schedule(items, cost, cost_two_heads, bh, sm_count, choice, &units, &cta_begin);
+    build_schedule(cost, cost_two_heads, bh, sm_count, choice, &units, &cta_begin);
     *n_cta_out = (int)cta_begin.size() - 1;
-    HB_CUDA(cudaMalloc(d_units, sizeof(WorkUnit) * units.size()));
-    HB_CUDA(cudaMemcpy(*d_units, units.data(), sizeof(WorkUnit) * units.size(), cudaMemcpyHostToDevice));
-    HB_CUDA(cudaMalloc(d_cta_begin, sizeof(int) * cta_begin.size()));
-    HB_CUDA(cudaMemcpy(*d_cta_begin, cta_begin.data(), sizeof(int) * cta_begin.size(), cudaMemcpyHostToDevice));
+    image.add(units, d_units);
+    image.add(cta_begin, d_cta_begin);
     return HILBERTA_OK;
 }
 
@@ -368,7 +309,7 @@ extern "C" int hilberta_schedule_units(int n_items, const int64_t *cost, const i
     if (cost_two_heads) c2.assign(cost_two_heads, cost_two_heads + n_items);
     std::vector<hilberta::WorkUnit> u;
     std::vector<int> cb;
-    const long long m = hilberta::build_schedule(n_items, c1.data(), cost_two_heads ? c2.data() : nullptr, bh, n_cta, u, cb);
+    const long long m = hilberta::build_schedule(c1, c2, bh, n_cta, hilberta::SplitChoice(), &u, &cb);
     for (size_t i = 0; i < u.size(); ++i) {
         units[3 * i] = u[i].item;
         units[3 * i + 1] = u[i].bh;

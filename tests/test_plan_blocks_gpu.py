@@ -1,0 +1,51 @@
+"""Plans that come and go: tables built in a block that another plan or binding has left behind are the
+plan's own, rebinding included, from several threads at once."""
+import threading
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import hilberta_oracle as orc
+from paper_2509_26538_b200 import binding as hb
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [(16, 16, 64, 5, 2, 7), (32, 24, 256, 100, 4, 0), (8, 8, 16, 3, 0, 33), (48, 48, 512, 7, 8, 300)]
+
+
+def test_blocks_are_reused_from_several_threads():
+    ref = {s: orc.plan_arrays(*s) for s in SHAPES}
+    bad = []
+
+    def work(k):
+        torch.cuda.set_device(0)
+        stream = torch.cuda.Stream()
+        for i in range(12):
+            s = SHAPES[(i + k) % len(SHAPES)]
+            plan = hb.Plan(*s)
+            S = plan.S
+            g = torch.Generator(device="cuda")
+            g.manual_seed(i)
+            with torch.cuda.stream(stream):
+                q, kk, v = (torch.randn((1, 2, S, 64), generator=g, device="cuda") for _ in range(3))
+                b = [t.to(torch.bfloat16) for t in (q, kk, v)]
+                plan.bind_like(b[0])
+                one = plan.forward(*b, torch.empty_like(b[0]))
+                plan.bind_like(q)              # another binding takes the first one's place
+                two = plan.forward(q, kk, v, torch.empty_like(q))
+                stream.synchronize()
+                # bf16 operands and weights: 2^-9 each, N(0, 1) values
+                if not (torch.isfinite(two).all() and (one.float() - two).norm() <= 1e-2 * two.norm()):
+                    bad.append((k, i, "forward"))
+            for what, key in ((hb.EXPORT_PHYS2ORIG, "phys2orig"), (hb.EXPORT_WINDOWS, "windows")):
+                if not np.array_equal(plan.export(what), ref[s][key]):
+                    bad.append((k, i, key))
+            plan.destroy()
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(3)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad, bad
