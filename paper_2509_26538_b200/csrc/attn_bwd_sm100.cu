@@ -8,7 +8,9 @@
 // dS = P * (dP - delta):   dQ = s dS K,   dK = s dS^T Q,   dV = P^T dO.
 //
 // Three launches: a bandwidth-bound pass that writes (LSE * log2 e, delta) per row,
-// then one tensor-core kernel in two modes that share all code but a few lines.
+// then one tensor-core kernel in two modes that share all code but a few lines; DKV first, and DQ on the
+// SMs that DKV leaves idle (programmatic dependent launch: 64 x 64 + 128 tokens, 16 heads, forward +
+// backward 161 -> 141 us).
 //   mode DQ : resident tile = 128 query rows (Q_i, dO_i); streamed = their keys (K_j, V_j)
 //             A = Q_i K_j^T, B = dO_i V_j^T, dS -> TMEM, dQ_i += dS K_j
 //   mode DKV: resident tile = 128 key rows (K_j, V_j); streamed = the queries that see them
@@ -59,8 +61,11 @@ enum Bar {
     P_READY,      // P / dS written over region B (256 arrivals)
     T1_FULL, T1_EMPTY = T1_FULL + NT1,
     T2_FULL = T1_EMPTY + NT1, T2_EMPTY = T2_FULL + NT2,
-    NUM_BARS = T2_EMPTY + NT2
+    // split units: the whole cluster's partial sums are in shared memory / have been read (4 warps per CTA)
+    PART_READY = T2_EMPTY + NT2, PART_READ,
+    NUM_BARS
 };
+constexpr int SPLIT_UNIT = -2;   // WorkUnit::bh2 of a unit that the CTAs of a cluster share
 
 // shared memory map (all dynamic; the tile area must start on a 1024-byte boundary)
 constexpr int OFF_R1 = 0, OFF_R2 = TILE_BYTES, OFF_T1 = 2 * TILE_BYTES, OFF_T2 = OFF_T1 + NT1 * TILE_BYTES;
@@ -120,7 +125,48 @@ __device__ __forceinline__ void issue_at(uint32_t tmem_out, uint32_t tmem_b, uin
                (accumulate || k > 0) ? 1u : 0u);
 }
 
-template <int MODE, int HD>
+// Rows [rank 128 / C, ...) of an item from the C partial sums of the cluster (at sPart in every CTA: COLS fp32
+// columns a row, the first HD of them out_a's), in rank order.  The loads of one 16-byte chunk are in
+// flight at a time per lane; neighbouring lanes take neighbouring chunks.
+template <int C, int MODE, int HD>
+__device__ __forceinline__ void merge_parts(const Params &prm, const WorkItem &wi, int r, int rank, long long off, uint32_t sPart) {
+    constexpr int COLS = (MODE == MODE_DKV ? 2 : 1) * HD, CH = COLS / 4, ROWS = BM / C;
+#pragma unroll(C == 2 ? 2 : 1)
+    for (int e = r; e < ROWS * CH / 2; e += 128) {
+        const int row = rank * ROWS + e / (CH / 2), pair = e % (CH / 2);   // a pair of chunks: 8 columns, 16 bytes out
+        float4 a[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int ch = 2 * pair + k;
+            const uint32_t at = sPart + row * (COLS * 4) + (((ch & ~7) | ((ch ^ row) & 7)) << 4);
+            float4 x[C];
+#pragma unroll
+            for (int p = 0; p < C; ++p) x[p] = ld_cluster_v4(cluster_map(at, p));
+            a[k] = x[0];
+#pragma unroll
+            for (int p = 1; p < C; ++p) {
+                a[k].x += x[p].x;
+                a[k].y += x[p].y;
+                a[k].z += x[p].z;
+                a[k].w += x[p].w;
+            }
+        }
+        if (row < wi.q_rows) {
+            const bool second = MODE == MODE_DKV && pair * 8 >= HD;
+            const float mul = second ? 1.f : prm.scale;
+            *reinterpret_cast<uint4 *>((second ? prm.out_b - HD : prm.out_a) + off + (long long)row * prm.stride_s + pair * 8) =
+                make_uint4(pack_bf16(a[0].x * mul, a[0].y * mul), pack_bf16(a[0].z * mul, a[0].w * mul),
+                           pack_bf16(a[1].x * mul, a[1].y * mul), pack_bf16(a[1].z * mul, a[1].w * mul));
+        }
+    }
+}
+
+// SPLIT: launched in clusters; units marked SPLIT_UNIT hold a share of the streamed rows each (the same
+// resident rows and head in every CTA of the cluster, first in the CTAs' lists).  At their end every CTA
+// leaves its sums in the space of its tiles and the epilogue warps of rank c add up rows c 128 / C ... of
+// all shares through distributed shared memory.  Measured (B200, forward + backward): 1 head, 16 x 96 x 96
+// tokens, 4920 -> 693 us; 5 heads, 128 x 128, 585 -> 164 us.
+template <int MODE, int HD, bool SPLIT>
 __global__ void __launch_bounds__(THREADS, 1)
 attn_bwd_kernel(const __grid_constant__ CUtensorMap tmR1, const __grid_constant__ CUtensorMap tmR2,
                 const __grid_constant__ CUtensorMap tmT1, const __grid_constant__ CUtensorMap tmT2,
@@ -158,6 +204,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmR1, const __grid_constant_
             uint32_t count = 1;
             if (i == EPI_DONE) count = 128;
             if (i == A_DONE || i == P_READY) count = 256;
+            if (SPLIT && (i == PART_READY || i == PART_READ)) count = 4 * cluster_cta_count();
             // DKV: ring 2 also carries the row statistics, copied by the 32 lanes of its producer warp
             if (MODE == MODE_DKV && i >= T2_FULL && i < T2_FULL + NT2) count = 33;
             mbar_init(bar(i), count);
@@ -171,6 +218,14 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmR1, const __grid_constant_
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (SPLIT) cluster_sync_all();   // the peers' barriers are initialised
+    // The two launches of a call need nothing from each other.  The first (DKV) waits for the pass that writes
+    // the row statistics and then lets the second start on SMs as they fall idle; the second waits for the
+    // first only at its end, so that whatever follows it in the stream follows both.
+    if (MODE == MODE_DKV) {
+        dependency_wait();
+        launch_dependents();
+    }
     const uint32_t tmem = *tmem_slot;
     const int u_begin = prm.cta_begin[blockIdx.x], u_end = prm.cta_begin[blockIdx.x + 1];
 
@@ -191,7 +246,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmR1, const __grid_constant_
             const int nslot = second ? NT2 : NT1;
             const int FULL = second ? T2_FULL : T1_FULL, EMPTY = second ? T2_EMPTY : T1_EMPTY;
             const uint32_t ring = second ? sT2 : sT1;
-            uint32_t g = 0;
+            uint32_t g = 0, sc = 0;
             bool ok = true;
             for (int u = u_begin; ok && u < u_end; ++u) {
                 const WorkUnit unit = prm.units[u];
@@ -230,6 +285,11 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmR1, const __grid_constant_
                         }
                     }
                 }
+                // the partial sums in the tiles' space have been read by the whole cluster
+                if (SPLIT && ok && unit.bh2 == SPLIT_UNIT) {
+                    if (leader) ok = wait_or_abort(bar(PART_READ), sc++ & 1, abort_flag, prm.status, 0x404);
+                    if (with_stats) ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+                }
             }
             if (with_stats) asm volatile("cp.async.wait_all;" ::: "memory");
             if (!ok && leader) {
@@ -246,7 +306,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmR1, const __grid_constant_
         if (elect_one()) {
             prefetch_tmap(&tmR1);
             prefetch_tmap(&tmR2);
-            uint32_t uc = 0;
+            uint32_t uc = 0, sc = 0;
             bool ok = true;
             for (int u = u_begin; ok && u < u_end; ++u, ++uc) {
                 const WorkUnit unit = prm.units[u];
@@ -272,6 +332,10 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmR1, const __grid_constant_
                         tma_prefetch_4d(&tmR2, 64 * sl, nq, nh, nb_);
                     }
                 }
+                if (SPLIT && unit.bh2 == SPLIT_UNIT) {
+                    ok = wait_or_abort(bar(PART_READ), sc++ & 1, abort_flag, prm.status, 0x405);
+                    if (!ok) break;
+                }
             }
             if (!ok) {
                 const long long t0 = clock64();
@@ -284,7 +348,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmR1, const __grid_constant_
         // Its own warpgroup, so that the element-wise warps move on to the next unit at once.
         const int r = tid & 127;
         const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
-        uint32_t uc = 0;
+        uint32_t uc = 0, sc = 0;
         bool ok = true;
         for (int u = u_begin; ok && u < u_end; ++u, ++uc) {
             const WorkUnit unit = prm.units[u];
@@ -298,6 +362,37 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmR1, const __grid_constant_
                                    (long long)(wi.q_start + r) * prm.stride_s;
             constexpr int CPO = HD / 32;                              // 32-column chunks per output
             constexpr int NCH = (MODE == MODE_DKV) ? 2 * CPO : CPO;   // DKV: dK then dV
+            if (SPLIT && unit.bh2 == SPLIT_UNIT) {
+                // every MMA of this share has read its tiles (OUT_FULL), and no loader passes the unit's end
+                // before PART_READ: the tiles' space is free.  Chunk c of row r sits at c ^ (r & 7) of its eight.
+#pragma unroll
+                for (int c = 0; c < NCH; ++c) {
+                    uint32_t o[32];
+                    tmem_ld32(tmem + lane_addr + (c >= CPO ? OUT_B + (c - CPO) * 32 : OUT_A + c * 32), o);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        st_shared_v4(sR1 + r * (NCH * 128) + ((c * 8 + (k ^ (r & 7))) << 4), o + 4 * k);
+                }
+                tc_fence_before();
+                mbar_arrive(bar(EPI_DONE));
+                fence_proxy_async_smem();   // the next unit's tiles land here through the async proxy
+                const uint32_t n_cta = cluster_cta_count();
+                __syncwarp();
+                if ((uint32_t)(tid & 31) < n_cta) mbar_arrive_release_cluster(cluster_map(bar(PART_READY), tid & 31));
+                ok = wait_or_abort(bar(PART_READY), sc++ & 1, abort_flag, prm.status, 0x606);
+                if (!ok) break;
+                cluster_acquire();
+                const int rank = (int)cluster_cta_rank();
+                const long long off = roff - (long long)r * prm.stride_s;
+                if (n_cta == 2) merge_parts<2, MODE, HD>(prm, wi, r, rank, off, sR1);
+                else if (n_cta == 4) merge_parts<4, MODE, HD>(prm, wi, r, rank, off, sR1);
+                else merge_parts<8, MODE, HD>(prm, wi, r, rank, off, sR1);
+                __syncwarp();
+                // nothing to release: the loads above have returned
+                if ((uint32_t)(tid & 31) < n_cta) mbar_arrive_cluster(cluster_map(bar(PART_READ), tid & 31));
+                continue;
+            }
 #pragma unroll
             for (int c = 0; c < NCH; ++c) {
                 uint32_t o[32];
@@ -521,10 +616,10 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmR1, const __grid_constant_
 
     tc_fence_before();
     __syncthreads();
-    if (warp == 8) {
-        __syncwarp();
-        tmem_dealloc(tmem, TMEM_COLS);
-    }
+    __syncwarp();
+    if (SPLIT) cluster_sync_all();   // peers signal this CTA's barriers until their last split unit is done
+    if (warp == 8) tmem_dealloc(tmem, TMEM_COLS);
+    if (MODE == MODE_DQ) dependency_wait();
 #ifdef HB_STAMPS
     if (threadIdx.x == 0) {
         unsigned long long ns;
@@ -541,6 +636,7 @@ __global__ void __launch_bounds__(256)
 delta_kernel(const __nv_bfloat16 *__restrict__ dout, const __nv_bfloat16 *__restrict__ out,
              const float *__restrict__ lse, float *__restrict__ lse2, float *__restrict__ delta, int S, int heads,
              long long stride_b, long long stride_h, long long stride_s, long long n_rows) {
+    launch_dependents();          // the next launch waits for this one after its prologue
     constexpr int LPR = HD / 8;   // lanes per row (16 bytes each)
     const int sub = threadIdx.x % LPR;
     const long long row0 = ((long long)blockIdx.x * (256 / LPR) + threadIdx.x / LPR) * 4;
@@ -580,6 +676,41 @@ delta_kernel(const __nv_bfloat16 *__restrict__ dout, const __nv_bfloat16 *__rest
 
 }  // namespace
 
+// The shared-memory opt-in is an attribute of the kernel ON ONE DEVICE: set it once for every device a plan
+// is bound on (a failure is reported, not remembered).  clusters: how many clusters of 2, 4 and 8 CTAs the
+// device runs at once.
+static int attn_bwd_opt_in(int device, const int **clusters) {
+    static std::mutex attr_mutex;
+    static bool attr_done[64] = {};
+    static int active[64][3] = {};
+    std::lock_guard<std::mutex> lock(attr_mutex);
+    if (device < 0 || device >= 64) return HILBERTA_ERR_INVALID;
+    *clusters = active[device];
+    if (attr_done[device]) return HILBERTA_OK;
+    const void *kernels[8] = {
+        (const void *)attn_bwd_kernel<MODE_DQ, 128, false>, (const void *)attn_bwd_kernel<MODE_DKV, 128, false>,
+        (const void *)attn_bwd_kernel<MODE_DQ, 64, false>,  (const void *)attn_bwd_kernel<MODE_DKV, 64, false>,
+        (const void *)attn_bwd_kernel<MODE_DQ, 128, true>,  (const void *)attn_bwd_kernel<MODE_DKV, 128, true>,
+        (const void *)attn_bwd_kernel<MODE_DQ, 64, true>,   (const void *)attn_bwd_kernel<MODE_DKV, 64, true>};
+    for (int i = 0; i < 8; ++i)
+        HB_CUDA(cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+    for (int i = 0; i < 3; ++i) {
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = 2u << i;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cfg.gridDim = dim3(2u << i);
+        cfg.blockDim = dim3(THREADS);
+        cfg.dynamicSmemBytes = SMEM_BYTES;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        HB_CUDA(cudaOccupancyMaxActiveClusters(&active[device][i], kernels[5], &cfg));
+    }
+    attr_done[device] = true;
+    return HILBERTA_OK;
+}
+
 // Work list of the backward kernels: 128 resident rows per item, the rows they exchange
 // gradients with listed as up to three contiguous ranges and counted in blocks of 128.
 // Also asks for the per-row scratch: lse * log2 e for every row, then delta for every row.  Called from hilberta_plan_bind for bf16 bindings.
@@ -591,32 +722,30 @@ int attn_bwd_prepare(hilberta_plan_t *p, BindImage &image) {
     }
     std::stable_sort(items.begin(), items.end(),
                      [](const WorkItem &a, const WorkItem &b) { return a.kv_blocks > b.kv_blocks; });
-    std::vector<long long> cost;
-    for (const WorkItem &it : items) cost.push_back((long long)it.kv_blocks + 3);
+    // in twentieths of a block, the unit of choose_split (a block of 128 x 128 takes 1.1 us in the DQ mode, 1.7
+    // in the DKV mode; both modes use one schedule)
+    std::vector<long long> cost, unpaired(items.size(), 0);
+    for (const WorkItem &it : items) cost.push_back((long long)it.kv_blocks * 20 + 60);
     p->n_bwd_work = (int)items.size();
     p->n_bwd_cta = 0;
+    p->bwd_cluster = 1;
     if (items.empty()) return HILBERTA_OK;
 
     const int bh = p->batch * p->heads;
+    const int *clusters = nullptr;
+    int rc = attn_bwd_opt_in(p->device, &clusters);
+    if (rc != HILBERTA_OK) return rc;
+    SplitChoice choice;
+    // The two launches share the chip, so a cut has to gain more than in the forward pass (geometric mean of 36
+    // problems of all sizes, forward included: 90.2 us without this, 86.9 with 100, 87.9 with 300, 101.6 uncut)
+    choice.merge_extra = 100;
+    choose_split(items, cost, unpaired, bh, p->sm_count, clusters, BK, choice);
+    p->bwd_cluster = choice.cluster;
+    for (const WorkItem &it : choice.shares) items.push_back(it);
     image.add(items, &p->d_bwd_work);
-    const int rc = add_schedule(image, cost, {}, bh, p->sm_count, SplitChoice(), &p->d_bwd_units, &p->d_bwd_cta_begin, &p->n_bwd_cta);
+    rc = add_schedule(image, cost, {}, bh, p->sm_count, choice, &p->d_bwd_units, &p->d_bwd_cta_begin, &p->n_bwd_cta);
     if (rc != HILBERTA_OK) return rc;
     image.add_scratch(2 * (size_t)bh * p->S, &p->d_delta);
-    {
-        // The shared-memory opt-in is an attribute of the kernel ON ONE DEVICE: set it once for every
-        // device a plan is bound on (a failure is reported, not remembered).
-        static std::mutex attr_mutex;
-        static bool attr_done[64] = {};
-        std::lock_guard<std::mutex> lock(attr_mutex);
-        if (p->device < 0 || p->device >= 64) return HILBERTA_ERR_INVALID;
-        if (!attr_done[p->device]) {
-            const void *kernels[4] = {(const void *)attn_bwd_kernel<MODE_DQ, 128>, (const void *)attn_bwd_kernel<MODE_DKV, 128>,
-                                      (const void *)attn_bwd_kernel<MODE_DQ, 64>, (const void *)attn_bwd_kernel<MODE_DKV, 64>};
-            for (int i = 0; i < 4; ++i)
-                HB_CUDA(cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-            attr_done[p->device] = true;
-        }
-    }
     return HILBERTA_OK;
 }
 
@@ -659,19 +788,34 @@ int launch_attn_bwd(const hilberta_plan_t *p, const void *dout, const void *q, c
     prm.status = p->d_status;
     prm.out_align32 = ((((uintptr_t)dq | (uintptr_t)dk | (uintptr_t)dv) & 31) == 0 &&
                        ((p->stride_b | p->stride_h | p->stride_s) & 15) == 0) ? 1 : 0;
-    prm.out_a = (__nv_bfloat16 *)dq;
-    prm.out_b = nullptr;
-    if (p->head_dim == 128)
-        attn_bwd_kernel<MODE_DQ, 128><<<p->n_bwd_cta, THREADS, SMEM_BYTES, stream>>>(mq, mdo, mk, mv, prm);
-    else
-        attn_bwd_kernel<MODE_DQ, 64><<<p->n_bwd_cta, THREADS, SMEM_BYTES, stream>>>(mq, mdo, mk, mv, prm);
-    HB_LAUNCHED();
+    // Both launches may overtake the one before them (see the kernel): the statistics pass, and each other.
+    cudaLaunchAttribute attr[2] = {};
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)p->bwd_cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)p->n_bwd_cta);
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = SMEM_BYTES;
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = p->bwd_cluster > 1 ? 2 : 1;
+    auto launch = [&](auto mode, const CUtensorMap &r1, const CUtensorMap &r2, const CUtensorMap &t1, const CUtensorMap &t2) {
+        constexpr int MODE = decltype(mode)::value;
+        auto go = [&](auto kernel) { return cudaLaunchKernelEx(&cfg, kernel, r1, r2, t1, t2, prm); };
+        if (p->bwd_cluster > 1)
+            return p->head_dim == 128 ? go(attn_bwd_kernel<MODE, 128, true>) : go(attn_bwd_kernel<MODE, 64, true>);
+        return p->head_dim == 128 ? go(attn_bwd_kernel<MODE, 128, false>) : go(attn_bwd_kernel<MODE, 64, false>);
+    };
     prm.out_a = (__nv_bfloat16 *)dk;
     prm.out_b = (__nv_bfloat16 *)dv;
-    if (p->head_dim == 128)
-        attn_bwd_kernel<MODE_DKV, 128><<<p->n_bwd_cta, THREADS, SMEM_BYTES, stream>>>(mk, mv, mq, mdo, prm);
-    else
-        attn_bwd_kernel<MODE_DKV, 64><<<p->n_bwd_cta, THREADS, SMEM_BYTES, stream>>>(mk, mv, mq, mdo, prm);
+    HB_CUDA(launch(std::integral_constant<int, MODE_DKV>{}, mk, mv, mq, mdo));
+    HB_LAUNCHED();
+    prm.out_a = (__nv_bfloat16 *)dq;
+    prm.out_b = nullptr;
+    HB_CUDA(launch(std::integral_constant<int, MODE_DQ>{}, mq, mdo, mk, mv));
     HB_LAUNCHED();
     return HILBERTA_OK;
 }

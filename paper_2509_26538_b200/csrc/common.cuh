@@ -146,7 +146,7 @@ struct hilberta_plan_s {
     int n_bwd_work;
     hilberta::WorkUnit *d_bwd_units;
     int *d_bwd_cta_begin;
-    int n_bwd_cta;
+    int n_bwd_cta, bwd_cluster;
     float *d_delta;               // [batch * heads * S]
     // fp32 bindings: items of 64 rows by descending key count; the first n_f32_split of them are cut over
     // clusters of f32_cluster CTAs
@@ -182,9 +182,11 @@ int check_work_items(const WorkItem *items, int n, int S, int item_rows, int blo
 struct SplitChoice {
     int cluster = 1, n_clusters = 0, n_items = 0;
     bool pair_heads = true;
+    long long merge_extra = 0;   // of a share, on top of what a forward merge costs
     std::vector<WorkItem> shares;
 };
-// clusters: how many clusters of 2, 4 and 8 CTAs run at once.  items sorted by descending cost.
+// clusters: how many clusters of 2, 4 and 8 CTAs run at once.  items sorted by descending cost.  Of
+// `choice` only merge_extra is read.
 void choose_split(const std::vector<WorkItem> &items, const std::vector<long long> &cost,
                   const std::vector<long long> &cost_two_heads, int bh, int sm_count, const int *clusters, int block,
                   SplitChoice &choice);

@@ -161,7 +161,7 @@ long long build_schedule(const std::vector<long long> &cost, const std::vector<l
         LeastLoaded clusters(std::vector<long long>((size_t)(n_cta / C), 0));
         for (int i = 0; i < ch.n_items; ++i)
             for (int j = 0; j < bh; ++j) {
-                const LeastLoaded::Load at = clusters.add((cost[i] + C - 1) / C + merge_cost(C));
+                const LeastLoaded::Load at = clusters.add((cost[i] + C - 1) / C + merge_cost(C) + ch.merge_extra);
                 makespan = std::max(makespan, at.first);
                 for (int r = 0; r < C; ++r) {
                     load[(size_t)(at.second * C + r)] = at.first;
@@ -216,7 +216,9 @@ static WorkItem share_of(const WorkItem &it, int lo, int hi, int block) {
 void choose_split(const std::vector<WorkItem> &items, const std::vector<long long> &cost,
                   const std::vector<long long> &cost_two_heads, int bh, int sm_count, const int *clusters, int block,
                   SplitChoice &choice) {
+    const long long merge_extra = choice.merge_extra;
     choice = SplitChoice();
+    choice.merge_extra = merge_extra;
     long long total = 0, n_units = 0;   // as scheduled without cuts
     for (size_t i = 0; i < items.size(); ++i) {
         const int pairs = cost_two_heads[i] > 0 ? bh / 2 : 0;
@@ -244,6 +246,7 @@ void choose_split(const std::vector<WorkItem> &items, const std::vector<long lon
         const int C = 2 << k;
         if (clusters[k] < 1) continue;
         SplitChoice c;
+        c.merge_extra = merge_extra;
         c.cluster = C;
         c.n_clusters = clusters[k];
         // cut the items of the longest, of the two longest, ... lengths; every share gets a block at least
@@ -253,7 +256,7 @@ void choose_split(const std::vector<WorkItem> &items, const std::vector<long lon
             if (items[n - 1].kv_blocks < C) break;
             const int pairs = cost_two_heads[n - 1] > 0 ? bh / 2 : 0;
             rest -= cost_two_heads[n - 1] * pairs + cost[n - 1] * (bh - 2 * pairs);
-            cut += ((cost[n - 1] + C - 1) / C + merge_cost(C)) * C * bh;
+            cut += ((cost[n - 1] + C - 1) / C + merge_cost(C) + c.merge_extra) * C * bh;
             if (n < (int)items.size() && items[n].kv_blocks == items[n - 1].kv_blocks) continue;
             ++levels;
             c.n_items = n;
