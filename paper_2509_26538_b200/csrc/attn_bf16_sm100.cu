@@ -336,6 +336,8 @@ attn_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     if (SPLIT) cluster_sync_all();   // the peers' barriers are initialised
     const uint32_t tmem = tmem_slot;
     const int u_begin = prm.cta_begin[blockIdx.x], u_end = prm.cta_begin[blockIdx.x + 1];
+    allow_next();
+    wait_for_previous();
     if (blockIdx.x == 0 && tid == 0) {
         // start stamps of the launch's first CTA (kept in shared memory: no register lives across the kernel)
         unsigned long long ns;
@@ -1275,16 +1277,6 @@ int launch_attn_bf16(const hilberta_plan_t *p, const void *q, const void *k, con
     prm.out_align32 = (((uintptr_t)out & 31) == 0 && ((p->stride_b | p->stride_h | p->stride_s) & 15) == 0) ? 1 : 0;
     CUtensorMap mo = mq;   // a valid map in any case; read only with bit 1 set
     if (!in_map && !out_map && make_out_tensor_map(&mo, out, p, heads)) prm.out_align32 |= 2;
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute attr{};
-    cfg.gridDim = dim3((unsigned)n_cta);
-    cfg.blockDim = dim3(THREADS);
-    cfg.stream = stream;
-    cfg.attrs = &attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = (unsigned)p->split_cluster;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cfg.numAttrs = p->split_cluster > 1 ? 1 : 0;
     KernelParams<true> gprm;
     static_cast<Params &>(gprm) = prm;
     gprm.in_map = in_map;
@@ -1296,8 +1288,8 @@ int launch_attn_bf16(const hilberta_plan_t *p, const void *q, const void *k, con
     auto launch = [&](auto split) {
         constexpr bool SPLIT = decltype(split)::value;
         auto go = [&](auto kernel, int smem, const auto &params) {
-            cfg.dynamicSmemBytes = (size_t)smem;
-            return cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, mo, params);
+            return launch_overlapping(kernel, (unsigned)n_cta, THREADS, (size_t)smem, (unsigned)p->split_cluster, stream, true, mq, mk, mv,
+                                      mo, params);
         };
         if (in_map) {
             if (fp8) return go(attn_bf16_kernel<true, 128, true, SPLIT>, smem_bytes(128, true, true, SPLIT), gprm);

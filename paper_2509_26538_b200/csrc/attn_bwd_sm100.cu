@@ -222,10 +222,8 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmR1, const __grid_constant_
     // The two launches of a call need nothing from each other.  The first (DKV) waits for the pass that writes
     // the row statistics and then lets the second start on SMs as they fall idle; the second waits for the
     // first only at its end, so that whatever follows it in the stream follows both.
-    if (MODE == MODE_DKV) {
-        dependency_wait();
-        launch_dependents();
-    }
+    if (MODE == MODE_DKV) wait_for_previous();
+    allow_next();
     const uint32_t tmem = *tmem_slot;
     const int u_begin = prm.cta_begin[blockIdx.x], u_end = prm.cta_begin[blockIdx.x + 1];
 
@@ -619,7 +617,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmR1, const __grid_constant_
     __syncwarp();
     if (SPLIT) cluster_sync_all();   // peers signal this CTA's barriers until their last split unit is done
     if (warp == 8) tmem_dealloc(tmem, TMEM_COLS);
-    if (MODE == MODE_DQ) dependency_wait();
+    if (MODE == MODE_DQ) wait_for_previous();
 #ifdef HB_STAMPS
     if (threadIdx.x == 0) {
         unsigned long long ns;
@@ -636,7 +634,6 @@ __global__ void __launch_bounds__(256)
 delta_kernel(const __nv_bfloat16 *__restrict__ dout, const __nv_bfloat16 *__restrict__ out,
              const float *__restrict__ lse, float *__restrict__ lse2, float *__restrict__ delta, int S, int heads,
              long long stride_b, long long stride_h, long long stride_s, long long n_rows) {
-    launch_dependents();          // the next launch waits for this one after its prologue
     constexpr int LPR = HD / 8;   // lanes per row (16 bytes each)
     const int sub = threadIdx.x % LPR;
     const long long row0 = ((long long)blockIdx.x * (256 / LPR) + threadIdx.x / LPR) * 4;
@@ -646,6 +643,10 @@ delta_kernel(const __nv_bfloat16 *__restrict__ dout, const __nv_bfloat16 *__rest
     for (int i = 0; i < 4; ++i) {
         const long long row = row0 + i;
         in[i] = row < n_rows;
+        if (i == 0) {
+            allow_next();
+            wait_for_previous();
+        }
         if (in[i]) {
             const long long bh = row / S;
             const long long off = (bh / heads) * stride_b + (bh % heads) * stride_h + (row % S) * stride_s + sub * 8;
@@ -763,14 +764,10 @@ int launch_attn_bwd(const hilberta_plan_t *p, const void *dout, const void *q, c
     if ((rc = make_tensor_map(&mv, v, p, BK)) != HILBERTA_OK) return rc;
     if ((rc = make_tensor_map(&mdo, dout, p, BK)) != HILBERTA_OK) return rc;
     const long long n_rows = (long long)p->batch * p->heads * p->S;
-    if (p->head_dim == 128)
-        delta_kernel<128><<<(unsigned)((n_rows + 63) / 64), 256, 0, stream>>>(
-            (const __nv_bfloat16 *)dout, (const __nv_bfloat16 *)out, lse, delta, delta + n_rows, p->S, p->heads,
-            p->stride_b, p->stride_h, p->stride_s, n_rows);
-    else
-        delta_kernel<64><<<(unsigned)((n_rows + 127) / 128), 256, 0, stream>>>(
-            (const __nv_bfloat16 *)dout, (const __nv_bfloat16 *)out, lse, delta, delta + n_rows, p->S, p->heads,
-            p->stride_b, p->stride_h, p->stride_s, n_rows);
+    HB_CUDA(launch_overlapping(p->head_dim == 128 ? delta_kernel<128> : delta_kernel<64>,
+                               (unsigned)((n_rows + (p->head_dim == 128 ? 63 : 127)) / (p->head_dim == 128 ? 64 : 128)), 256, 0, 1,
+                               stream, true, (const __nv_bfloat16 *)dout, (const __nv_bfloat16 *)out, lse, delta, delta + n_rows,
+                               p->S, p->heads, p->stride_b, p->stride_h, p->stride_s, n_rows));
     HB_LAUNCHED();
     Params prm;
     prm.work = p->d_bwd_work;
@@ -788,23 +785,12 @@ int launch_attn_bwd(const hilberta_plan_t *p, const void *dout, const void *q, c
     prm.status = p->d_status;
     prm.out_align32 = ((((uintptr_t)dq | (uintptr_t)dk | (uintptr_t)dv) & 31) == 0 &&
                        ((p->stride_b | p->stride_h | p->stride_s) & 15) == 0) ? 1 : 0;
-    // Both launches may overtake the one before them (see the kernel): the statistics pass, and each other.
-    cudaLaunchAttribute attr[2] = {};
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned)p->bwd_cluster;
-    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)p->n_bwd_cta);
-    cfg.blockDim = dim3(THREADS);
-    cfg.dynamicSmemBytes = SMEM_BYTES;
-    cfg.stream = stream;
-    cfg.attrs = attr;
-    cfg.numAttrs = p->bwd_cluster > 1 ? 2 : 1;
     auto launch = [&](auto mode, const CUtensorMap &r1, const CUtensorMap &r2, const CUtensorMap &t1, const CUtensorMap &t2) {
         constexpr int MODE = decltype(mode)::value;
-        auto go = [&](auto kernel) { return cudaLaunchKernelEx(&cfg, kernel, r1, r2, t1, t2, prm); };
+        auto go = [&](auto kernel) {
+            return launch_overlapping(kernel, (unsigned)p->n_bwd_cta, THREADS, SMEM_BYTES, (unsigned)p->bwd_cluster, stream, true, r1, r2,
+                                      t1, t2, prm);
+        };
         if (p->bwd_cluster > 1)
             return p->head_dim == 128 ? go(attn_bwd_kernel<MODE, 128, true>) : go(attn_bwd_kernel<MODE, 64, true>);
         return p->head_dim == 128 ? go(attn_bwd_kernel<MODE, 128, false>) : go(attn_bwd_kernel<MODE, 64, false>);

@@ -42,6 +42,8 @@ attn_fp32_kernel(const float *__restrict__ q, const float *__restrict__ k, const
     const int lane = threadIdx.x & 31, rg = lane >> 3, cg = lane & 7;
     const int wrow = (threadIdx.x >> 5) * 16 + rg;   // this lane's rows: wrow + 2 i
 
+    allow_next();
+    wait_for_previous();
     // in_map: q, k, v are in original order and physical row p lives at row in_map[p]
     load_rows<D>(sQ, q + base, stride_s, it.q_start, it.q_rows, in_map);
     if (j0 < j1) {
@@ -226,17 +228,15 @@ int launch_attn_fp32(const hilberta_plan_t *p, const void *q, const void *k, con
     if ((bits & 15) || ((p->stride_b | p->stride_h | p->stride_s) & 3)) return HILBERTA_ERR_INVALID;
     if (chunk >= 0) return HILBERTA_ERR_INVALID;   // fp32 bindings have no slices of heads
     if (p->n_f32_work == 0) return HILBERTA_OK;
+    const long long ctas = grid_of(p, 1);
+    if (ctas > 0x7fffffffll) return HILBERTA_ERR_INVALID;
 #define HB_FP32_CASE(DD)                                                                                              \
-    case DD: {                                                                                                        \
-        const ClusterLaunch cfg(p, fwd_smem<DD>(), 1, stream);                                                        \
-        if (cfg.ctas > 0x7fffffffll) return HILBERTA_ERR_INVALID;                                                     \
-        HB_CUDA(cudaLaunchKernelEx(&cfg.config, attn_fp32_kernel<DD>, (const float *)q, (const float *)k,             \
-                                   (const float *)v, (float *)out, (long long)p->stride_b, (long long)p->stride_h,    \
-                                   (long long)p->stride_s, p->heads, p->batch * p->heads, p->S,                       \
-                                   (const WorkItem *)p->d_f32_work,                                                   \
+    case DD:                                                                                                          \
+        HB_CUDA(launch_overlapping(attn_fp32_kernel<DD>, (unsigned)ctas, kThreads, fwd_smem<DD>(), (unsigned)p->f32_cluster, stream, true, \
+                                   (const float *)q, (const float *)k, (const float *)v, (float *)out, p->stride_b,   \
+                                   p->stride_h, p->stride_s, p->heads, p->batch * p->heads, p->S, p->d_f32_work,      \
                                    p->n_f32_work, p->n_f32_split, p->f32_cluster, out_map, in_map, lse, p->scale));   \
-        break;                                                                                                        \
-    }
+        break;
     switch (p->head_dim) {
         HB_FP32_CASE(32)
         HB_FP32_CASE(64)

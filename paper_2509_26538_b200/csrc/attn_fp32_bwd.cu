@@ -21,11 +21,13 @@ constexpr int kDeltaRows = 4;
 template <int D>
 __global__ void __launch_bounds__(kDeltaRows * 32)
 delta_fp32_kernel(const float *__restrict__ dout, const float *__restrict__ out, float *__restrict__ delta,
-                  long long stride_b, long long stride_h, long long stride_s, int heads, int S) {
+                  long long stride_b, long long stride_h, long long stride_s, int heads, int S, long long rows) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row = blockIdx.x * kDeltaRows + warp;
-    if (row >= S) return;
-    const int bh = blockIdx.y;
+    const long long at = (long long)blockIdx.x * kDeltaRows + warp;   // (batch * head, row)
+    allow_next();
+    wait_for_previous();
+    if (at >= rows) return;
+    const int bh = (int)(at / S), row = (int)(at % S);
     const long long off = (long long)(bh / heads) * stride_b + (long long)(bh % heads) * stride_h +
                           (long long)row * stride_s;
     float acc = 0.f;
@@ -33,7 +35,7 @@ delta_fp32_kernel(const float *__restrict__ dout, const float *__restrict__ out,
     for (int e = 0; e < D / 32; ++e) acc = fmaf(dout[off + lane + 32 * e], out[off + lane + 32 * e], acc);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) delta[(long long)bh * S + row] = acc;
+    if (lane == 0) delta[at] = acc;
 }
 
 // pairs of streamed tiles in shared memory: two where two CTAs of that size fit an SM, one at head dim 128
@@ -191,6 +193,8 @@ attn_fp32_bwd_kernel(const float *__restrict__ q, const float *__restrict__ k, c
     const Share share(n_items, n_split, cluster, 2 * bhs);
     if (share.item < 0) return;
     const WorkItem it = work[share.item];
+    allow_next();
+    wait_for_previous();
     const bool keys = share.column < bhs;   // the direction with more work per pair first
     const int bh = keys ? share.column : share.column - bhs;
     const long long base = (long long)(bh / heads) * stride_b + (long long)(bh % heads) * stride_h;
@@ -206,16 +210,16 @@ template <int D>
 int launch(const hilberta_plan_t *p, const float *dout, const float *q, const float *k, const float *v,
            const float *out, const float *lse, float *dq, float *dk, float *dv, float *delta, cudaStream_t stream) {
     if (p->n_f32_work == 0) return HILBERTA_OK;
-    dim3 grid((p->S + kDeltaRows - 1) / kDeltaRows, p->batch * p->heads);
-    delta_fp32_kernel<D><<<grid, kDeltaRows * 32, 0, stream>>>(dout, out, delta, p->stride_b, p->stride_h, p->stride_s,
-                                                               p->heads, p->S);
+    const long long rows = (long long)p->batch * p->heads * p->S;
+    HB_CUDA(launch_overlapping(delta_fp32_kernel<D>, (unsigned)((rows + kDeltaRows - 1) / kDeltaRows), kDeltaRows * 32, 0, 1, stream, true, dout,
+                               out, delta, p->stride_b, p->stride_h, p->stride_s, p->heads, p->S, rows));
     HB_LAUNCHED();
-    const ClusterLaunch cfg(p, bwd_smem<D>(), 2, stream);
-    if (cfg.ctas > 0x7fffffffll) return HILBERTA_ERR_INVALID;
-    HB_CUDA(cudaLaunchKernelEx(&cfg.config, attn_fp32_bwd_kernel<D>, q, k, v, dout, lse, (const float *)delta, dq, dk, dv,
-                               (long long)p->stride_b, (long long)p->stride_h, (long long)p->stride_s, p->heads,
-                               p->batch * p->heads, p->S,
-                               (const WorkItem *)p->d_f32_work, p->n_f32_work, p->n_f32_split, p->f32_cluster, p->scale));
+    const long long ctas = grid_of(p, 2);
+    if (ctas > 0x7fffffffll || (rows + kDeltaRows - 1) / kDeltaRows > 0x7fffffffll) return HILBERTA_ERR_INVALID;
+    HB_CUDA(launch_overlapping(attn_fp32_bwd_kernel<D>, (unsigned)ctas, kThreads, bwd_smem<D>(), (unsigned)p->f32_cluster, stream, true, q, k, v,
+                               dout, lse, delta, dq, dk, dv, p->stride_b, p->stride_h, p->stride_s, p->heads,
+                               p->batch * p->heads, p->S, p->d_f32_work, p->n_f32_work, p->n_f32_split, p->f32_cluster,
+                               p->scale));
     HB_LAUNCHED();
     return HILBERTA_OK;
 }

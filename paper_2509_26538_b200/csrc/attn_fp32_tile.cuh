@@ -214,28 +214,12 @@ __device__ __forceinline__ void load_block(float *tile, const float *base, long 
     }
 }
 
-// Launch over a plan's fp32 work list: `directions` instances per (batch, head) and item, whole clusters.
-struct ClusterLaunch {
-    cudaLaunchConfig_t config;
-    cudaLaunchAttribute attr;
-    long long ctas;
-    ClusterLaunch(const hilberta_plan_t *p, int smem, int directions, cudaStream_t stream) : config{}, attr{} {
-        const long long c = p->f32_cluster, columns = (long long)p->batch * p->heads * directions;
-        const long long single = (p->n_f32_work - p->n_f32_split) * columns;
-        ctas = p->n_f32_split * columns * c + (single + c - 1) / c * c;
-        config.gridDim = dim3((unsigned)ctas);
-        config.blockDim = dim3(kThreads);
-        config.dynamicSmemBytes = (size_t)smem;
-        config.stream = stream;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = (unsigned)c;
-        attr.val.clusterDim.y = 1;
-        attr.val.clusterDim.z = 1;
-        config.attrs = &attr;
-        config.numAttrs = c > 1 ? 1 : 0;
-    }
-    ClusterLaunch(const ClusterLaunch &) = delete;   // config points into the object
-};
+// CTAs of a launch over a plan's fp32 work list: `directions` instances per (batch, head) and item, whole clusters.
+inline long long grid_of(const hilberta_plan_t *p, int directions) {
+    const long long c = p->f32_cluster, columns = (long long)p->batch * p->heads * directions;
+    const long long single = (p->n_f32_work - p->n_f32_split) * columns;
+    return p->n_f32_split * columns * c + (single + c - 1) / c * c;
+}
 
 }  // namespace fp32t
 }  // namespace hilberta

@@ -160,6 +160,35 @@ struct hilberta_plan_s {
 };
 
 namespace hilberta {
+
+// Programmatic dependent launch: the library's kernels allow the next one in the stream to be set up while
+// they drain (allow_next: once every CTA has said so), and each reads and writes nothing that an earlier
+// kernel could still touch before wait_for_previous has returned -- until then only its plan's tables, which
+// no kernel writes after the plan and its binding are made.  Every kernel waits, so its end implies the end
+// of all before it.  Saves the launch latency and the prologue between kernels, 1 ... 2 us each (one fused
+// launch after another, 512^2 and 8 heads: 18.7 -> 16.6 us).  overlap = false: an ordinary launch.
+__device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... Params, class... Args>
+cudaError_t launch_overlapping(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, unsigned cluster,
+                               cudaStream_t stream, bool overlap, const Args &...args) {
+    cudaLaunchAttribute attr[2] = {};
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t config{};
+    config.gridDim = dim3(grid);
+    config.blockDim = dim3(block);
+    config.dynamicSmemBytes = smem;
+    config.stream = stream;
+    config.attrs = attr;
+    config.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&config, kernel, Params(args)...);
+}
+
 // out_map: nullptr = write rows in physical order; else out_map[p] is the row of `out`
 // that physical row p goes to (the exit gather fused into the epilogue).
 // lse: nullptr, or [batch * heads, S] fp32 receiving log-sum-exp of the scaled logits

@@ -656,6 +656,7 @@ extern "C" int hilberta_plan_bind(hilberta_plan_t *p, int batch, int heads, int 
         p->bind_bytes = total;
         HB_CUDA(take_block(p->device, &p->d_bind, &p->bind_bytes));
         HB_CUDA(cudaMemcpy(p->d_bind, image.bytes.data(), image.bytes.size(), cudaMemcpyHostToDevice));
+        HB_CUDA(cudaStreamSynchronize(0));   // a copy from pageable memory returns when it is staged, not when it is done
     }
     for (const BindImage::Place &at : image.places)
         *at.where = (char *)p->d_bind + at.at + (at.in_scratch ? image.bytes.size() : 0);

@@ -231,10 +231,6 @@ __device__ __forceinline__ float4 ld_cluster_v4(uint32_t a) {
     asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(a) : "memory");
     return x;
 }
-// Programmatic dependent launch: the next launch in the stream (if it asks for it) may start once every CTA
-// has said so; wait: until the launch this one may have overtaken is complete and its writes are visible.
-__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // TMA tile load into this CTA's shared memory whose bytes are counted on a barrier of the pair's
 // leader CTA (cluster address).
 __device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap *m, uint32_t cluster_bar, int c0,
