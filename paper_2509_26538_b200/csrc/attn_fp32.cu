@@ -3,7 +3,7 @@
 // plus the rows' slid tile, or the whole sequence for prefix rows) and walks it in blocks of 32 keys; the
 // next block's K and V tiles arrive (cp.async) while this block is worked on, and a block costs one barrier.
 // Bound: the FMA pipes and, next to them, shared memory.  Measured (B200): 32 x 32 + 64 tokens, 8 heads of 64,
-// forward + backward 1500 -> 190 us (16 TFLOP/s useful; one warp per query row with a key per lane before,
+// forward + backward 1500 -> 179 us (17 TFLOP/s useful; one warp per query row with a key per lane before,
 // every lane reading whole rows of its own); 16 x 16 tokens, 2 heads of 64, 26 -> 10 us a call.
 #include <math.h>
 
@@ -232,7 +232,7 @@ int launch_attn_fp32(const hilberta_plan_t *p, const void *q, const void *k, con
     if (ctas > 0x7fffffffll) return HILBERTA_ERR_INVALID;
 #define HB_FP32_CASE(DD)                                                                                              \
     case DD:                                                                                                          \
-        HB_CUDA(launch_overlapping(attn_fp32_kernel<DD>, (unsigned)ctas, kThreads, fwd_smem<DD>(), (unsigned)p->f32_cluster, stream, true, \
+        HB_CUDA(launch_overlapping(attn_fp32_kernel<DD>, (unsigned)ctas, kThreads, fwd_smem<DD>(), (unsigned)p->f32_cluster, stream, may_overlap(p, ctas), \
                                    (const float *)q, (const float *)k, (const float *)v, (float *)out, p->stride_b,   \
                                    p->stride_h, p->stride_s, p->heads, p->batch * p->heads, p->S, p->d_f32_work,      \
                                    p->n_f32_work, p->n_f32_split, p->f32_cluster, out_map, in_map, lse, p->scale));   \

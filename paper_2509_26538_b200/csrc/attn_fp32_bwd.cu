@@ -6,6 +6,8 @@
 //           being symmetric):  dk_j += dS_ij q_i,  dv_j += P_ij dO_i
 // with P_ij = exp(s q_i.k_j - lse_i), dS_ij = P_ij (dO_i.v_j - delta_i).  Nothing is accumulated across
 // CTAs but through a cluster's shared memory in rank order, so results are bit-reproducible.
+// One pair of streamed tiles and three CTAs an SM (168 registers, 63 KB): their warps cover the waits for one
+// another's tiles; two pairs and two CTAs took 193 instead of 186 us (32 x 32 + 64 tokens, 8 heads of 64, both passes).
 #include <math.h>
 
 #include "attn_fp32_tile.cuh"
@@ -38,11 +40,8 @@ delta_fp32_kernel(const float *__restrict__ dout, const float *__restrict__ out,
     if (lane == 0) delta[at] = acc;
 }
 
-// pairs of streamed tiles in shared memory: two where two CTAs of that size fit an SM, one at head dim 128
-// (145 KB with two; at head dim 64 one pair and three CTAs measured equal, 0.5 % behind)
-__host__ __device__ constexpr int stages(int D) { return D == 128 ? 1 : 2; }
 template <int D>
-constexpr int bwd_smem() { return (2 * res_floats(D) + 2 * stages(D) * blk_floats(D) + BR * PS) * (int)sizeof(float); }
+constexpr int bwd_smem() { return (2 * res_floats(D) + 2 * blk_floats(D) + BR * PS) * (int)sizeof(float); }
 
 // One mode for one CTA.  r1 / t1: resident and streamed operand of the scores, r2 / t2: of dP.
 template <int D, int MODE>
@@ -52,7 +51,7 @@ __device__ __forceinline__ void bwd_tile(const float *r1, const float *r2, const
     extern __shared__ float4 smem4[];
     constexpr int C = D / 8;
     float *sR1 = reinterpret_cast<float *>(smem4), *sR2 = sR1 + res_floats(D), *sT = sR2 + res_floats(D);
-    float *sP = sT + 2 * stages(D) * blk_floats(D);
+    float *sP = sT + 2 * blk_floats(D);
     const KeyList kl(it);
     const int nb = (kl.total + BC - 1) / BC;
     const int j0 = (int)((long long)nb * share.rank / share.parts), j1 = (int)((long long)nb * (share.rank + 1) / share.parts);
@@ -72,14 +71,14 @@ __device__ __forceinline__ void bwd_tile(const float *r1, const float *r2, const
         for (int c = 0; c < C; ++c) a[i][c] = b[i][c] = 0.f;
     }
     const float one[4] = {1.f, 1.f, 1.f, 1.f};
-    auto load = [&](int j, float *dst) {
-        load_block<D>(dst, t1, stride_s, kl, j, nullptr);
-        load_block<D>(dst + blk_floats(D), t2, stride_s, kl, j, nullptr);
+    const float *sT1 = sT, *sT2 = sT + blk_floats(D);
+    auto load = [&](int j) {
+        load_block<D>(sT, t1, stride_s, kl, j, nullptr);
+        load_block<D>(sT + blk_floats(D), t2, stride_s, kl, j, nullptr);
     };
-    if (j0 < j1) load(j0, sT);
-    cp_commit();
+    if (j0 < j1) load(j0);
+    cp_commit();   // also where this share has no block: the resident tiles' space holds the sums at the end
     for (int j = j0; j < j1; ++j) {
-        const float *sT1 = sT + ((j - j0) % stages(D)) * 2 * blk_floats(D), *sT2 = sT1 + blk_floats(D);
         const int valid = kl.total - j * BC;   // >= 1
         // the statistics belong to the QUERY of the pair: the streamed row in mode 1
         float col_lse[4], col_delta[4];
@@ -92,11 +91,7 @@ __device__ __forceinline__ void bwd_tile(const float *r1, const float *r2, const
             }
         }
         cp_wait<0>();
-        __syncthreads();   // this block's tiles are in, and every warp is done with the other pair
-        if (stages(D) == 2) {
-            if (j + 1 < j1) load(j + 1, sT + ((j + 1 - j0) % stages(D)) * 2 * blk_floats(D));
-            cp_commit();
-        }
+        __syncthreads();   // this block's tiles are in
         float p[4][4];
         dot_tile<D>(p, sR1 + wrow * (D + 4), sT1 + cg * (D + 4));
 #pragma unroll
@@ -126,13 +121,9 @@ __device__ __forceinline__ void bwd_tile(const float *r1, const float *r2, const
             for (int jj = 0; jj < 4; ++jj) sP[(wrow + 4 * i) * PS + 8 * jj + cg] = ds[i][jj];
         __syncwarp();
         acc_tile<D>(a, one, sP + wrow * PS, sT1, cg);       // dq += dS k  |  dk += dS q
-        if (stages(D) == 1) {
-            __syncthreads();   // the streamed tiles are free
-            if (j + 1 < j1) load(j + 1, sT);
-            cp_commit();
-        } else {
-            __syncwarp();
-        }
+        __syncthreads();   // ... and free again; the other CTAs of the SM work while the next ones come
+        if (j + 1 < j1) load(j + 1);
+        cp_commit();
     }
     cp_wait<0>();
     if (share.parts == 1) {
@@ -184,7 +175,7 @@ __device__ __forceinline__ void bwd_tile(const float *r1, const float *r2, const
 }
 
 template <int D>
-__global__ void __launch_bounds__(kThreads, D == 128 ? 1 : 2)
+__global__ void __launch_bounds__(kThreads, D == 128 ? 2 : 3)
 attn_fp32_bwd_kernel(const float *__restrict__ q, const float *__restrict__ k, const float *__restrict__ v,
                      const float *__restrict__ dout, const float *__restrict__ lse, const float *__restrict__ delta,
                      float *__restrict__ dq, float *__restrict__ dk, float *__restrict__ dv, long long stride_b,
@@ -216,7 +207,7 @@ int launch(const hilberta_plan_t *p, const float *dout, const float *q, const fl
     HB_LAUNCHED();
     const long long ctas = grid_of(p, 2);
     if (ctas > 0x7fffffffll || (rows + kDeltaRows - 1) / kDeltaRows > 0x7fffffffll) return HILBERTA_ERR_INVALID;
-    HB_CUDA(launch_overlapping(attn_fp32_bwd_kernel<D>, (unsigned)ctas, kThreads, bwd_smem<D>(), (unsigned)p->f32_cluster, stream, true, q, k, v,
+    HB_CUDA(launch_overlapping(attn_fp32_bwd_kernel<D>, (unsigned)ctas, kThreads, bwd_smem<D>(), (unsigned)p->f32_cluster, stream, may_overlap(p, ctas), q, k, v,
                                dout, lse, delta, dq, dk, dv, p->stride_b, p->stride_h, p->stride_s, p->heads,
                                p->batch * p->heads, p->S, p->d_f32_work, p->n_f32_work, p->n_f32_split, p->f32_cluster,
                                p->scale));

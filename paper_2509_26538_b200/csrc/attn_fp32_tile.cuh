@@ -221,5 +221,10 @@ inline long long grid_of(const hilberta_plan_t *p, int directions) {
     return p->n_f32_split * columns * c + (single + c - 1) / c * c;
 }
 
+// Several CTAs of these kernels share an SM.  One that is set up while the kernel before it still runs goes
+// where there is room and not where the load is even: four layers of 25 x 34 + 333 tokens, 6 heads of 32 (228
+// CTAs), 318 us overlapping against 262 in turn; 112 CTAs of head dim 128 68 against 62; 80 CTAs 46 against 49.
+inline bool may_overlap(const hilberta_plan_t *p, long long ctas) { return 5 * ctas <= 3 * p->sm_count; }
+
 }  // namespace fp32t
 }  // namespace hilberta
