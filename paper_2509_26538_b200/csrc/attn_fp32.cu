@@ -52,6 +52,7 @@ attn_fp32_kernel(const float *__restrict__ q, const float *__restrict__ k, const
     }
     cp_commit();
 
+    const bool busy = (int)(threadIdx.x >> 5) * 16 < it.q_rows;   // a warp without rows only helps with the loads
     float m[4], l[4], o[4][C];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -70,6 +71,7 @@ attn_fp32_kernel(const float *__restrict__ q, const float *__restrict__ k, const
             load_block<D>(nK + blk_floats(D), v + base, stride_s, kl, j + 1, in_map);
         }
         cp_commit();
+        if (!busy) continue;
         float x[4][4];
         dot_tile<D>(x, sQ + wrow * (D + 4), sK + cg * (D + 4));
         const int valid = kl.total - j * BC;   // >= 1

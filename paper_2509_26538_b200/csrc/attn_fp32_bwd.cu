@@ -71,6 +71,7 @@ __device__ __forceinline__ void bwd_tile(const float *r1, const float *r2, const
         for (int c = 0; c < C; ++c) a[i][c] = b[i][c] = 0.f;
     }
     const float one[4] = {1.f, 1.f, 1.f, 1.f};
+    const bool busy = (int)(threadIdx.x >> 5) * 16 < it.q_rows;   // a warp without rows only helps with the loads
     const float *sT1 = sT, *sT2 = sT + blk_floats(D);
     auto load = [&](int j) {
         load_block<D>(sT, t1, stride_s, kl, j, nullptr);
@@ -92,35 +93,37 @@ __device__ __forceinline__ void bwd_tile(const float *r1, const float *r2, const
         }
         cp_wait<0>();
         __syncthreads();   // this block's tiles are in
-        float p[4][4];
-        dot_tile<D>(p, sR1 + wrow * (D + 4), sT1 + cg * (D + 4));
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj)
-                p[i][jj] = 8 * jj + cg < valid ? expf(fmaf(p[i][jj], scale, -(MODE == 0 ? row_lse[i] : col_lse[jj]))) : 0.f;
-        float ds[4][4];
-        dot_tile<D>(ds, sR2 + wrow * (D + 4), sT2 + cg * (D + 4));
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj)   // beyond the list P is zero and the streamed rows and statistics are any
-                ds[i][jj] = 8 * jj + cg < valid ? p[i][jj] * (ds[i][jj] - (MODE == 0 ? row_delta[i] : col_delta[jj])) : 0.f;
-        if (MODE == 1) {
+        if (busy) {
+            float p[4][4];
+            dot_tile<D>(p, sR1 + wrow * (D + 4), sT1 + cg * (D + 4));
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int jj = 0; jj < 4; ++jj) sP[(wrow + 4 * i) * PS + 8 * jj + cg] = p[i][jj];
+                for (int jj = 0; jj < 4; ++jj)
+                    p[i][jj] = 8 * jj + cg < valid ? expf(fmaf(p[i][jj], scale, -(MODE == 0 ? row_lse[i] : col_lse[jj]))) : 0.f;
+            float ds[4][4];
+            dot_tile<D>(ds, sR2 + wrow * (D + 4), sT2 + cg * (D + 4));
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int jj = 0; jj < 4; ++jj)   // beyond the list P is zero and the streamed rows and statistics are any
+                    ds[i][jj] = 8 * jj + cg < valid ? p[i][jj] * (ds[i][jj] - (MODE == 0 ? row_delta[i] : col_delta[jj])) : 0.f;
+            if (MODE == 1) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int jj = 0; jj < 4; ++jj) sP[(wrow + 4 * i) * PS + 8 * jj + cg] = p[i][jj];
+                __syncwarp();
+                acc_tile<D>(b, one, sP + wrow * PS, sT2, cg);   // dv += P dO
+                __syncwarp();
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int jj = 0; jj < 4; ++jj) sP[(wrow + 4 * i) * PS + 8 * jj + cg] = ds[i][jj];
             __syncwarp();
-            acc_tile<D>(b, one, sP + wrow * PS, sT2, cg);   // dv += P dO
-            __syncwarp();
+            acc_tile<D>(a, one, sP + wrow * PS, sT1, cg);       // dq += dS k  |  dk += dS q
         }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj) sP[(wrow + 4 * i) * PS + 8 * jj + cg] = ds[i][jj];
-        __syncwarp();
-        acc_tile<D>(a, one, sP + wrow * PS, sT1, cg);       // dq += dS k  |  dk += dS q
         __syncthreads();   // ... and free again; the other CTAs of the SM work while the next ones come
         if (j + 1 < j1) load(j + 1);
         cp_commit();
