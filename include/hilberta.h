@@ -175,7 +175,9 @@ int hilberta_plan_export(const hilberta_plan_t *plan, int what, void *host_buf, 
  *   scale          softmax scale s; <= 0 selects 1/sqrt(head_dim).
  *
  * Builds the kernel's work list (device memory) and may allocate and synchronise.
- * Rebinding replaces the previous binding. */
+ * Rebinding replaces the previous binding.  Long key lists may be cut over clusters
+ * of thread blocks, chosen from the shape alone, so the bits of a result depend on
+ * batch and heads but not on the stream, the entry point or the call. */
 int hilberta_plan_bind(hilberta_plan_t *plan, int batch, int heads, int head_dim, int dtype,
                        int64_t stride_b, int64_t stride_h, int64_t stride_s, float scale);
 
