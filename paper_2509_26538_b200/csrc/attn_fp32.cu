@@ -181,11 +181,10 @@ attn_fp32_kernel(const float *__restrict__ q, const float *__restrict__ k, const
 // cut over clusters of up to 8 CTAs as long as that leaves no SM more than a few CTAs.  Prefix rows see the
 // whole sequence, and on the problems this path serves a handful of them would otherwise outlast everything
 // else (and a small problem would leave most SMs idle); every cut costs each CTA its start and a merge.  The
-// bounds are read off sweeps on the B200 (us; clusters of 1 / 2 / 4 / 8): 32 x 32 + 64 tokens, 8 heads of
-// 64, forward + backward (19 items) 340 / 205 / 190 / 244; 32 x 32 + 226, 4 heads of 64 (21) 411 / 253 / 207 /
-// 212; 16 x 16, 2 heads of 64, forward (5) 32 / 20 / 13 / 11; 25 x 34 + 333, 6 heads of 32 (19) 373 / 261 / 291 /
-// 278; 16 x 16 + 128, 16 heads of 128 (7) 235 / 166 / 187 / 236; 35 x 35 + 77, 13 heads of 128 (23) 343 / 350 /
-// 339 / 397.
+// bound (CTAs per SM up to which cuts double) is the best of 1.5, 2, 3, 4.5, 6 and 8 over 42 problems on the
+// B200; geometric means in us, forward: head dim 64 65.8 / 61.2 / 55.4 / 54.6 / 55.8 / 56.7, 128 128 / 128 / 118 /
+// 104 / 103 / 102, 32 37.6 / 35.0 / 33.7 / 36.9 / 37.1 / 37.0; forward + backward: 64 219 / 177 / 167 / 160 / 168 /
+// 180, 128 242 / 208 / 204 / 191 / 207 / 223, 32 134 / 125 / 120 / 133 / 133 / 137.
 int attn_fp32_prepare(hilberta_plan_t *p, BindImage &image) {
     std::vector<WorkItem> items = build_work_items(p, BR, BC);
     const int rc = check_work_items(items.data(), (int)items.size(), p->S, BR, BC);
@@ -197,7 +196,7 @@ int attn_fp32_prepare(hilberta_plan_t *p, BindImage &image) {
     };
     std::stable_sort(items.begin(), items.end(), [&](const WorkItem &a, const WorkItem &b) { return blocks(a) > blocks(b); });
     const long long instances = (long long)items.size() * p->batch * p->heads;
-    const long long most = (long long)p->sm_count * (p->head_dim == 64 ? 9 : 6) / 2;
+    const long long most = (long long)p->sm_count * (p->head_dim == 32 ? 6 : 9) / 2;
     p->f32_cluster = 1;
     while (p->f32_cluster < 8 && instances * p->f32_cluster * 2 <= most) p->f32_cluster *= 2;
     p->n_f32_split = 0;
