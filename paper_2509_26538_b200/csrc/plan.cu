@@ -4,6 +4,7 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <utility>
 
 #include "common.cuh"
 
@@ -272,17 +273,22 @@ __global__ void window_compact_kernel(int R, int groups, int size, int offset, i
 
 // Device blocks of destroyed plans and replaced bindings, kept for the next ones: allocating and freeing a
 // plan's two blocks took 0.6 ms of the 1.2 ms of a plan, bind and destroy at 1024^2.  At most 16 blocks and
-// 64 MB; beyond that, and when an allocation fails, they go back to the device.  A block is put aside only after
-// the device has finished all work (which cudaFree would have waited for as well), so its next owner may be
-// on any stream.
+// 64 MB; beyond that, and when an allocation fails, they go back to the device.  Launches may still read a block
+// when it is put aside; it is handed out only after a wait for all of them, so its next owner may be on any
+// stream.
 namespace {
 struct Block {
     int device;
     void *ptr;
     size_t bytes;
+    uint64_t given;   // how many blocks had been put aside before it
+    bool idle;        // the device has finished the work of that time
 };
 std::mutex g_blocks_mutex;
 std::vector<Block> &g_blocks = *new std::vector<Block>();   // never destroyed: plans may go after the statics
+uint64_t g_blocks_given = 0;
+constexpr int kMaxDevices = 64;
+void *g_marker[kMaxDevices] = {};
 constexpr size_t kKeepBlocks = 16, kKeepBytes = 64u << 20;
 
 struct OnDevice {
@@ -296,9 +302,30 @@ struct OnDevice {
     }
 };
 
+// Waits for all work that the device (the current one) has been given: by freeing an allocation, which waits
+// for every stream, and not by cudaDeviceSynchronize, which ends a stream capture that another thread, or
+// a relaxed one, has begun.  The small allocation that always stays keeps the memory behind it mapped: without
+// it the pair of calls takes 600 us, with it plan, bind and destroy at 1024^2 take 227 us together (208 with
+// cudaDeviceSynchronize).
+bool wait_for_device(int device) {
+    void *marker = nullptr;
+    bool ok = device >= 0 && device < kMaxDevices && cudaMalloc(&marker, 256) == cudaSuccess;
+    if (ok) {
+        std::lock_guard<std::mutex> lock(g_blocks_mutex);
+        std::swap(g_marker[device], marker);
+    }
+    if (ok && !marker) ok = cudaMalloc(&marker, 256) == cudaSuccess;   // the first one stays
+    ok = ok && cudaFree(marker) == cudaSuccess;
+    if (!ok) cudaGetLastError();   // not the caller's business: it takes another block
+    return ok;
+}
+
 // bytes: wanted; on return the size of the block
 cudaError_t take_block(int device, void **ptr, size_t *bytes) {
+    const OnDevice on(device);
     *bytes = (*bytes + 65535) & ~(size_t)65535;
+    Block found{};
+    uint64_t given = 0;
     {
         std::lock_guard<std::mutex> lock(g_blocks_mutex);
         size_t best = g_blocks.size();
@@ -307,13 +334,22 @@ cudaError_t take_block(int device, void **ptr, size_t *bytes) {
                 (best == g_blocks.size() || g_blocks[i].bytes < g_blocks[best].bytes))
                 best = i;
         if (best < g_blocks.size()) {
-            *ptr = g_blocks[best].ptr;
-            *bytes = g_blocks[best].bytes;
+            found = g_blocks[best];
             g_blocks.erase(g_blocks.begin() + (long)best);
-            return cudaSuccess;
         }
+        given = g_blocks_given;
     }
-    const OnDevice on(device);
+    if (found.ptr && !found.idle) {
+        found.idle = wait_for_device(device);
+        std::lock_guard<std::mutex> lock(g_blocks_mutex);
+        for (Block &b : g_blocks) b.idle = b.idle || (found.idle && b.device == device && b.given < given);
+    }
+    if (found.ptr && found.idle) {
+        *ptr = found.ptr;
+        *bytes = found.bytes;
+        return cudaSuccess;
+    }
+    if (found.ptr) cudaFree(found.ptr);
     cudaError_t e = cudaMalloc(ptr, *bytes);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();   // not the caller's business if the second try succeeds
@@ -329,17 +365,16 @@ cudaError_t take_block(int device, void **ptr, size_t *bytes) {
 
 void give_block(int device, void *ptr, size_t bytes) {
     if (!ptr) return;
-    const OnDevice on(device);
-    const bool idle = cudaDeviceSynchronize() == cudaSuccess;
-    if (idle) {
+    {
         std::lock_guard<std::mutex> lock(g_blocks_mutex);
         size_t held = bytes;
         for (const Block &b : g_blocks) held += b.bytes;
         if (held <= kKeepBytes && g_blocks.size() < kKeepBlocks) {
-            g_blocks.push_back(Block{device, ptr, bytes});
+            g_blocks.push_back(Block{device, ptr, bytes, g_blocks_given++, false});
             return;
         }
     }
+    const OnDevice on(device);
     cudaFree(ptr);
 }
 }  // namespace
@@ -639,7 +674,7 @@ extern "C" int hilberta_plan_bind(hilberta_plan_t *p, int batch, int heads, int 
     p->stride_h = stride_h;
     p->stride_s = stride_s;
     p->scale = scale > 0.f ? scale : 1.0f / sqrtf((float)head_dim);
-    give_block(p->device, p->d_bind, p->bind_bytes);   // waits for launches that still read the old tables
+    give_block(p->device, p->d_bind, p->bind_bytes);   // launches may still read the old tables
     p->d_bind = nullptr;
     BindImage image;
     int rc = HILBERTA_OK;
