@@ -144,8 +144,16 @@ int hilberta_plan_groups(int H, int W, int groups, int layer_offset, int shared_
 int hilberta_plan_video(int frames, int H, int W, int tile, int layer_offset, int shared_region,
                         int shared_frames, int n_text, hilberta_plan_t **out);
 
-/* Free a plan and every device table it owns.  NULL is accepted. */
+/* Free a plan.  NULL is accepted.  Launches of the plan that are still under way keep their tables.  Its device
+ * memory is kept for the plans and bindings that follow (they wait for those launches before they use it): at
+ * most 16 blocks and 64 MB for each device, the newest ones, a reused block being up to twice and 1 MB larger
+ * than what was asked for.  The call waits for the device only where an older block has to go for it. */
 int hilberta_plan_destroy(hilberta_plan_t *plan);
+
+/* Give back to the devices all memory that destroyed plans and replaced bindings have left behind (the library
+ * does so by itself when one of its own allocations fails).  Returns the bytes.  Waits for the work under way
+ * on those devices; not to be called while a stream capture forbids freeing memory. */
+size_t hilberta_trim(void);
 
 /* Copy one canonical table of the plan to HOST memory (for parity checks and
  * callers that want the permutation).  `what` is a HILBERTA_EXPORT_* selector.

@@ -23,7 +23,8 @@ BF16, FP32, FP8_E4M3 = 0, 1, 2
 
 # every symbol include/hilberta.h declares
 SYMBOLS = (
-    "hilberta_plan", "hilberta_plan_groups", "hilberta_plan_video", "hilberta_plan_destroy", "hilberta_plan_export",
+    "hilberta_plan", "hilberta_plan_groups", "hilberta_plan_video", "hilberta_plan_destroy", "hilberta_trim",
+    "hilberta_plan_export",
     "hilberta_plan_bind",
     "hilberta_forward", "hilberta_forward_unpermute", "hilberta_forward_fused", "hilberta_forward_lse",
     "hilberta_backward",
@@ -66,6 +67,8 @@ def lib():
     L.hilberta_plan_video.restype = i32
     L.hilberta_plan_destroy.argtypes = [vp]
     L.hilberta_plan_destroy.restype = i32
+    L.hilberta_trim.argtypes = []
+    L.hilberta_trim.restype = sz
     L.hilberta_plan_export.argtypes = [vp, i32, vp, sz, ctypes.POINTER(sz)]
     L.hilberta_plan_export.restype = i32
     L.hilberta_plan_bind.argtypes = [vp, i32, i32, i32, i32, i64, i64, i64, f32]
@@ -327,6 +330,11 @@ def hilberta_permute(src, dst, plan: Plan, stream=None):
 
 def hilberta_unpermute(src, dst, plan: Plan, stream=None):
     return plan.unpermute(src, dst, stream)
+
+
+def trim() -> int:
+    """Give back the device memory that destroyed plans and replaced bindings have left behind; returns the bytes."""
+    return int(lib().hilberta_trim())
 
 
 def launch_count() -> int:

@@ -273,9 +273,9 @@ __global__ void window_compact_kernel(int R, int groups, int size, int offset, i
 
 // Device blocks of destroyed plans and replaced bindings, kept for the next ones: allocating and freeing a
 // plan's two blocks took 0.6 ms of the 1.2 ms of a plan, bind and destroy at 1024^2.  At most 16 blocks and
-// 64 MB; beyond that, and when an allocation fails, they go back to the device.  Launches may still read a block
-// when it is put aside; it is handed out only after a wait for all of them, so its next owner may be on any
-// stream.
+// 64 MB a device, the newest ones; all of them go back to their devices when an allocation fails and with
+// hilberta_trim.  Launches may still read a block when it is put aside; it is handed out only after a wait for
+// all of them, so its next owner may be on any stream.
 namespace {
 struct Block {
     int device;
@@ -320,6 +320,35 @@ bool wait_for_device(int device) {
     return ok;
 }
 
+// Bytes given back to the devices.  A block that cannot be freed now (a capture is under way) is kept.
+size_t free_blocks(const std::vector<Block> &blocks) {
+    size_t bytes = 0;
+    for (const Block &b : blocks) {
+        if (cudaFree(b.ptr) == cudaSuccess) {
+            bytes += b.bytes;
+            continue;
+        }
+        cudaGetLastError();
+        std::lock_guard<std::mutex> lock(g_blocks_mutex);
+        g_blocks.push_back(b);
+    }
+    return bytes;
+}
+
+size_t free_kept() {
+    std::vector<Block> out;
+    {
+        std::lock_guard<std::mutex> lock(g_blocks_mutex);
+        out.swap(g_blocks);
+        for (int d = 0; d < kMaxDevices; ++d)
+            if (g_marker[d]) {
+                out.push_back(Block{d, g_marker[d], 256, 0, false});
+                g_marker[d] = nullptr;
+            }
+    }
+    return free_blocks(out);
+}
+
 // bytes: wanted; on return the size of the block
 cudaError_t take_block(int device, void **ptr, size_t *bytes) {
     const OnDevice on(device);
@@ -349,15 +378,11 @@ cudaError_t take_block(int device, void **ptr, size_t *bytes) {
         *bytes = found.bytes;
         return cudaSuccess;
     }
-    if (found.ptr) cudaFree(found.ptr);
+    if (found.ptr) free_blocks({found});
     cudaError_t e = cudaMalloc(ptr, *bytes);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();   // not the caller's business if the second try succeeds
-        {
-            std::lock_guard<std::mutex> lock(g_blocks_mutex);
-            for (const Block &b : g_blocks) cudaFree(b.ptr);
-            g_blocks.clear();
-        }
+        free_kept();
         e = cudaMalloc(ptr, *bytes);
     }
     return e;
@@ -365,17 +390,28 @@ cudaError_t take_block(int device, void **ptr, size_t *bytes) {
 
 void give_block(int device, void *ptr, size_t bytes) {
     if (!ptr) return;
+    std::vector<Block> out;
     {
         std::lock_guard<std::mutex> lock(g_blocks_mutex);
-        size_t held = bytes;
-        for (const Block &b : g_blocks) held += b.bytes;
-        if (held <= kKeepBytes && g_blocks.size() < kKeepBlocks) {
-            g_blocks.push_back(Block{device, ptr, bytes, g_blocks_given++, false});
-            return;
+        size_t held = bytes, n = 1;
+        for (const Block &b : g_blocks)
+            if (b.device == device) {
+                held += b.bytes;
+                ++n;
+            }
+        g_blocks.push_back(Block{device, ptr, bytes, g_blocks_given++, false});
+        for (size_t i = 0; (held > kKeepBytes || n > kKeepBlocks) && i < g_blocks.size();) {   // the oldest first
+            if (g_blocks[i].device != device) {
+                ++i;
+                continue;
+            }
+            held -= g_blocks[i].bytes;
+            --n;
+            out.push_back(g_blocks[i]);
+            g_blocks.erase(g_blocks.begin() + (long)i);
         }
     }
-    const OnDevice on(device);
-    cudaFree(ptr);
+    free_blocks(out);
 }
 }  // namespace
 
@@ -598,6 +634,8 @@ extern "C" int hilberta_plan_destroy(hilberta_plan_t *plan) {
     free_plan(plan);
     return HILBERTA_OK;
 }
+
+extern "C" size_t hilberta_trim(void) { return free_kept(); }
 
 extern "C" int hilberta_plan_export(const hilberta_plan_t *p, int what, void *host_buf, size_t bytes,
                                     size_t *needed) {

@@ -49,3 +49,28 @@ def test_blocks_are_reused_from_several_threads():
     for t in threads:
         t.join()
     assert not bad, bad
+
+
+def test_kept_memory_is_bounded_recent_and_given_back():
+    hb.trim()
+    assert hb.trim() == 0
+    small = [hb.Plan(16, 16, 64, o, 2, 7) for o in range(40)]
+    for p in small:
+        p.destroy()
+    held = hb.trim()
+    assert 0 < held <= 16 * 65536 * 2
+    # many small blocks do not keep a larger one out
+    small = [hb.Plan(16, 16, 64, o, 2, 7) for o in range(40)]
+    for p in small:
+        p.destroy()
+    large = hb.Plan(64, 64, 256, 0, 0, 0)
+    large.bind(1, 64, 64, hb.FP32)          # two floats per row: 2 MB
+    large.destroy()
+    assert hb.trim() >= 64 * 4096 * 2 * 4
+    # nor do many large ones add up
+    plans = [hb.Plan(128, 128, 1024, o, 0, 0) for o in range(8)]
+    for p in plans:
+        p.bind(2, 48, 64, hb.FP32)          # 12 MB each
+    for p in plans:
+        p.destroy()
+    assert 48 << 20 <= hb.trim() <= 64 << 20
