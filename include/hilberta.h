@@ -331,8 +331,8 @@ int hilberta_forward_fused(const void *q, const void *k, const void *v, void *ou
  * gathers fused in and copies the result to `out` (HOST pointer, ORIGINAL order).
  * The heads are processed in up to eight slices whose copies (two internal copy
  * streams, one per direction) and launches (`stream`) overlap.
- * Uses a device workspace that the first call on a plan allocates (and
- * hilberta_plan_destroy frees).  Requires a dense binding (strides 0).  The
+ * Uses a device workspace that the first call on a plan allocates, or finds among
+ * what destroyed plans have left (see hilberta_plan_destroy, which puts it there).  Requires a dense binding (strides 0).  The
  * copies are asynchronous if the host buffers are pinned; the call returns
  * after synchronising `stream`. */
 int hilberta_forward_host(const void *q, const void *k, const void *v, void *out,

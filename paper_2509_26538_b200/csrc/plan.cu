@@ -271,7 +271,7 @@ __global__ void window_compact_kernel(int R, int groups, int size, int offset, i
     win[w] = r;
 }
 
-// Device blocks of destroyed plans and replaced bindings, kept for the next ones: allocating and freeing a
+// Device blocks of destroyed plans (tables, workspaces) and replaced bindings, kept for the next ones: allocating and freeing a
 // plan's two blocks took 0.6 ms of the 1.2 ms of a plan, bind and destroy at 1024^2.  At most 16 blocks and
 // 64 MB a device, the newest ones; all of them go back to their devices when an allocation fails and with
 // hilberta_trim.  Launches may still read a block when it is put aside; it is handed out only after a wait for
@@ -423,7 +423,7 @@ static void free_plan(hilberta_plan_t *p) {
     for (cudaEvent_t e : p->ev_done) cudaEventDestroy(e);
     if (p->s_in) cudaStreamDestroy(p->s_in);
     if (p->s_out) cudaStreamDestroy(p->s_out);
-    cudaFree(p->ws);
+    give_block(p->device, p->ws, p->ws_bytes);
     delete p;
 }
 
@@ -873,11 +873,12 @@ extern "C" int hilberta_forward_host(const void *q, const void *k, const void *v
     const size_t bytes = (size_t)p->batch * p->heads * p->S * p->head_dim * esz_out;   // the larger of the two
     const size_t slot = (bytes + 255) & ~(size_t)255;
     if (p->ws_bytes < 4 * slot) {
-        cudaFree(p->ws);
+        give_block(p->device, p->ws, p->ws_bytes);
         p->ws = nullptr;
         p->ws_bytes = 0;
-        HB_CUDA(cudaMalloc(&p->ws, 4 * slot));
-        p->ws_bytes = 4 * slot;
+        size_t got = 4 * slot;
+        HB_CUDA(take_block(p->device, &p->ws, &got));
+        p->ws_bytes = got;
     }
     // fp32 bindings have no slice schedule to build: chunk_heads is only set by the bf16 path
     const int hc = (p->dtype != HILBERTA_FP32 && p->chunk_heads > 0) ? p->chunk_heads : p->heads;

@@ -74,3 +74,21 @@ def test_kept_memory_is_bounded_recent_and_given_back():
     for p in plans:
         p.destroy()
     assert 48 << 20 <= hb.trim() <= 64 << 20
+
+
+def test_the_workspace_of_host_calls_is_kept_too():
+    """The first host-buffer call on a plan finds the workspace that an earlier plan's calls have left."""
+    hb.trim()
+    host = [torch.randn((1, 2, 64 * 64, 128)).bfloat16().pin_memory() for _ in range(4)]
+    want = None
+    for i in range(3):
+        plan = hb.Plan(64, 64, 256, 9, 4, 0)
+        plan.bind(1, 2, 128, hb.BF16)
+        before = torch.cuda.mem_get_info()[0]
+        plan.forward_host(*host)
+        if i:
+            assert torch.cuda.mem_get_info()[0] == before
+            assert torch.equal(host[3].view(torch.int16), want.view(torch.int16))
+        want = host[3].clone()
+        plan.destroy()
+    assert hb.trim() >= 4 * host[0].nbytes
