@@ -703,6 +703,8 @@ extern "C" int hilberta_plan_bind(hilberta_plan_t *p, int batch, int heads, int 
     if (dtype == HILBERTA_BF16 && ((stride_b | stride_h | stride_s) & 7)) return HILBERTA_ERR_INVALID;
     if (dtype == HILBERTA_FP8_E4M3 && ((stride_b | stride_h | stride_s) & 15)) return HILBERTA_ERR_INVALID;
     if ((int64_t)batch * heads > 65535) return HILBERTA_ERR_INVALID;
+    // the kernels' attributes and the number of clusters that run at once are the plan's device's
+    const OnDevice on(p->device);
     p->bound = false;
     p->batch = batch;
     p->heads = heads;

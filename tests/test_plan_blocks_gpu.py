@@ -92,3 +92,18 @@ def test_the_workspace_of_host_calls_is_kept_too():
         want = host[3].clone()
         plan.destroy()
     assert hb.trim() >= 4 * host[0].nbytes
+
+
+@pytest.mark.skipif(torch.cuda.device_count() < 2, reason="two devices")
+def test_a_plan_is_bound_on_its_own_device():
+    """Whichever device is current: tables, kernel attributes and results are those of the plan's device, which a
+    bind elsewhere must not have marked as set up."""
+    with torch.cuda.device(1):
+        plan = hb.Plan(24, 24, 64, 5, 2, 40)
+        x = [torch.randn((1, 2, plan.S, 128), device="cuda") for _ in range(3)]
+    plan.bind_like(x[0])   # device 0 is current; fp32 of head dim 128 needs the opt-in to large shared memory
+    assert torch.cuda.current_device() == 0
+    with torch.cuda.device(1):
+        out = plan.forward(*x, torch.full_like(x[0], float("nan")))
+        assert torch.isfinite(out).all() and plan.status() == 0
+    plan.destroy()
