@@ -7,10 +7,11 @@
 // With P = exp(s Q K^T - LSE), dP = dO V^T, delta = rowsum(dO * O) and
 // dS = P * (dP - delta):   dQ = s dS K,   dK = s dS^T Q,   dV = P^T dO.
 //
-// Three launches: a bandwidth-bound pass that writes (LSE * log2 e, delta) per row,
-// then one tensor-core kernel in two modes that share all code but a few lines; DKV first, and DQ on the
-// SMs that DKV leaves idle (programmatic dependent launch: 64 x 64 + 128 tokens, 16 heads, forward +
-// backward 161 -> 141 us).
+// Two launches: a bandwidth-bound pass that writes (LSE * log2 e, delta) per row, then one tensor-core
+// kernel whose CTAs work in one of two modes that share all code but a few lines: the first half of the grid
+// is DKV, the second DQ, which takes the SMs that DKV leaves idle.  One grid and not a launch of each: as a
+// dependent launch DQ would have to read the statistics before its own wait if it is to start early (16 x 16
+// + 20 tokens, 2 heads, forward + backward 24.8 us that way, 22.6 as one grid; 64 x 64 + 512, 24 heads, 527 both).
 //   mode DQ : resident tile = 128 query rows (Q_i, dO_i); streamed = their keys (K_j, V_j)
 //             A = Q_i K_j^T, B = dO_i V_j^T, dS -> TMEM, dQ_i += dS K_j
 //   mode DKV: resident tile = 128 key rows (K_j, V_j); streamed = the queries that see them
@@ -83,8 +84,7 @@ struct Params {
     long long stride_b, stride_h, stride_s;  // elements
     const float *lse2;    // [batch * heads * S] lse * log2 e
     const float *delta;   // [batch * heads * S] rowsum(dO * O)
-    __nv_bfloat16 *out_a; // DQ: dq; DKV: dk
-    __nv_bfloat16 *out_b; // DKV: dv
+    __nv_bfloat16 *dq, *dk, *dv;
     float scale, scale_log2;
     int S;
     int out_align32;      // outputs and strides 32-byte aligned: 32-byte stores allowed
@@ -126,7 +126,7 @@ __device__ __forceinline__ void issue_at(uint32_t tmem_out, uint32_t tmem_b, uin
 }
 
 // Rows [rank 128 / C, ...) of an item from the C partial sums of the cluster (at sPart in every CTA: COLS fp32
-// columns a row, the first HD of them out_a's), in rank order.  The loads of one 16-byte chunk are in
+// columns a row, the first HD of them dk's in DKV mode, then dv's), in rank order.  The loads of one 16-byte chunk are in
 // flight at a time per lane; neighbouring lanes take neighbouring chunks.
 template <int C, int MODE, int HD>
 __device__ __forceinline__ void merge_parts(const Params &prm, const WorkItem &wi, int r, int rank, long long off, uint32_t sPart) {
@@ -154,7 +154,7 @@ __device__ __forceinline__ void merge_parts(const Params &prm, const WorkItem &w
         if (row < wi.q_rows) {
             const bool second = MODE == MODE_DKV && pair * 8 >= HD;
             const float mul = second ? 1.f : prm.scale;
-            *reinterpret_cast<uint4 *>((second ? prm.out_b - HD : prm.out_a) + off + (long long)row * prm.stride_s + pair * 8) =
+            *reinterpret_cast<uint4 *>((second ? prm.dv - HD : MODE == MODE_DKV ? prm.dk : prm.dq) + off + (long long)row * prm.stride_s + pair * 8) =
                 make_uint4(pack_bf16(a[0].x * mul, a[0].y * mul), pack_bf16(a[0].z * mul, a[0].w * mul),
                            pack_bf16(a[1].x * mul, a[1].y * mul), pack_bf16(a[1].z * mul, a[1].w * mul));
         }
@@ -166,17 +166,16 @@ __device__ __forceinline__ void merge_parts(const Params &prm, const WorkItem &w
 // leaves its sums in the space of its tiles and the epilogue warps of rank c add up rows c 128 / C ... of
 // all shares through distributed shared memory.  Measured (B200, forward + backward): 1 head, 16 x 96 x 96
 // tokens, 4920 -> 693 us; 5 heads, 128 x 128, 585 -> 164 us.
+// cta: this CTA's number among those of its mode.
 template <int MODE, int HD, bool SPLIT>
-__global__ void __launch_bounds__(THREADS, 1)
-attn_bwd_kernel(const __grid_constant__ CUtensorMap tmR1, const __grid_constant__ CUtensorMap tmR2,
-                const __grid_constant__ CUtensorMap tmT1, const __grid_constant__ CUtensorMap tmT2,
-                const Params prm) {
+__device__ __forceinline__ void bwd_cta(const CUtensorMap &tmR1, const CUtensorMap &tmR2, const CUtensorMap &tmT1,
+                                        const CUtensorMap &tmT2, const Params &prm, int cta) {
     extern __shared__ uint8_t smem_raw[];
 #ifdef HB_STAMPS
     if (threadIdx.x == 0) {
         unsigned long long ns;
         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(ns));
-        prm.status[1024 + MODE * 1024 + 4 * blockIdx.x] = (int)(ns & 0x7fffffff);
+        prm.status[1024 + MODE * 1024 + 4 * cta] = (int)(ns & 0x7fffffff);
     }
 #endif
     constexpr uint32_t REG_A = 0, REG_B = 128, OUT_A = 256, OUT_B = 384;   // TMEM columns
@@ -219,13 +218,10 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmR1, const __grid_constant_
     __syncthreads();
     tc_fence_after();
     if (SPLIT) cluster_sync_all();   // the peers' barriers are initialised
-    // The two launches of a call need nothing from each other.  The first (DKV) waits for the pass that writes
-    // the row statistics and then lets the second start on SMs as they fall idle; the second waits for the
-    // first only at its end, so that whatever follows it in the stream follows both.
-    if (MODE == MODE_DKV) wait_for_previous();
     allow_next();
+    wait_for_previous();
     const uint32_t tmem = *tmem_slot;
-    const int u_begin = prm.cta_begin[blockIdx.x], u_end = prm.cta_begin[blockIdx.x + 1];
+    const int u_begin = prm.cta_begin[cta], u_end = prm.cta_begin[cta + 1];
 
     if (warp >= 8) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
@@ -397,7 +393,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmR1, const __grid_constant_
                 tmem_ld32(tmem + lane_addr + (c >= CPO ? OUT_B + (c - CPO) * 32 : OUT_A + c * 32), o);
                 tmem_wait_ld();
                 if (row_ok) {
-                    __nv_bfloat16 *orow = (c >= CPO ? prm.out_b : prm.out_a) + roff + (c % CPO) * 32;
+                    __nv_bfloat16 *orow = (c >= CPO ? prm.dv : MODE == MODE_DKV ? prm.dk : prm.dq) + roff + (c % CPO) * 32;
                     const float mul = c >= CPO ? 1.f : prm.scale;
                     uint32_t w[16];
 #pragma unroll
@@ -617,14 +613,25 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmR1, const __grid_constant_
     __syncwarp();
     if (SPLIT) cluster_sync_all();   // peers signal this CTA's barriers until their last split unit is done
     if (warp == 8) tmem_dealloc(tmem, TMEM_COLS);
-    if (MODE == MODE_DQ) wait_for_previous();
 #ifdef HB_STAMPS
     if (threadIdx.x == 0) {
         unsigned long long ns;
         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(ns));
-        prm.status[1024 + MODE * 1024 + 4 * blockIdx.x + 1] = (int)(ns & 0x7fffffff);
+        prm.status[1024 + MODE * 1024 + 4 * cta + 1] = (int)(ns & 0x7fffffff);
     }
 #endif
+}
+
+// The first half of the CTAs work in DKV mode, whose blocks take longer, the second half in DQ mode; both
+// have the same schedule.
+template <int HD, bool SPLIT>
+__global__ void __launch_bounds__(THREADS, 1)
+attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmdO,
+                const __grid_constant__ Params prm) {
+    const int half = (int)gridDim.x / 2, cta = (int)blockIdx.x;
+    if (cta < half) bwd_cta<MODE_DKV, HD, SPLIT>(tmK, tmV, tmQ, tmdO, prm, cta);
+    else bwd_cta<MODE_DQ, HD, SPLIT>(tmQ, tmdO, tmK, tmV, prm, cta - half);
 }
 
 // lse2[row] = lse[row] * log2 e, delta[row] = sum_d dO[row, d] * O[row, d]: HD / 8 lanes per row
@@ -688,13 +695,9 @@ static int attn_bwd_opt_in(int device, const int **clusters) {
     if (device < 0 || device >= 64) return HILBERTA_ERR_INVALID;
     *clusters = active[device];
     if (attr_done[device]) return HILBERTA_OK;
-    const void *kernels[8] = {
-        (const void *)attn_bwd_kernel<MODE_DQ, 128, false>, (const void *)attn_bwd_kernel<MODE_DKV, 128, false>,
-        (const void *)attn_bwd_kernel<MODE_DQ, 64, false>,  (const void *)attn_bwd_kernel<MODE_DKV, 64, false>,
-        (const void *)attn_bwd_kernel<MODE_DQ, 128, true>,  (const void *)attn_bwd_kernel<MODE_DKV, 128, true>,
-        (const void *)attn_bwd_kernel<MODE_DQ, 64, true>,   (const void *)attn_bwd_kernel<MODE_DKV, 64, true>};
-    for (int i = 0; i < 8; ++i)
-        HB_CUDA(cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+    const void *kernels[4] = {(const void *)attn_bwd_kernel<128, false>, (const void *)attn_bwd_kernel<64, false>,
+                              (const void *)attn_bwd_kernel<128, true>, (const void *)attn_bwd_kernel<64, true>};
+    for (const void *k : kernels) HB_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
     for (int i = 0; i < 3; ++i) {
         cudaLaunchConfig_t cfg{};
         cudaLaunchAttribute attr{};
@@ -706,7 +709,7 @@ static int attn_bwd_opt_in(int device, const int **clusters) {
         cfg.dynamicSmemBytes = SMEM_BYTES;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
-        HB_CUDA(cudaOccupancyMaxActiveClusters(&active[device][i], kernels[5], &cfg));
+        HB_CUDA(cudaOccupancyMaxActiveClusters(&active[device][i], kernels[2], &cfg));
     }
     attr_done[device] = true;
     return HILBERTA_OK;
@@ -737,7 +740,7 @@ int attn_bwd_prepare(hilberta_plan_t *p, BindImage &image) {
     int rc = attn_bwd_opt_in(p->device, &clusters);
     if (rc != HILBERTA_OK) return rc;
     SplitChoice choice;
-    // The two launches share the chip, so a cut has to gain more than in the forward pass (geometric mean of 36
+    // The two modes share the chip, so a cut has to gain more than in the forward pass (geometric mean of 36
     // problems of all sizes, forward included: 90.2 us without this, 86.9 with 100, 87.9 with 300, 101.6 uncut)
     choice.merge_extra = 100;
     choose_split(items, cost, unpaired, bh, p->sm_count, clusters, BK, choice);
@@ -785,23 +788,15 @@ int launch_attn_bwd(const hilberta_plan_t *p, const void *dout, const void *q, c
     prm.status = p->d_status;
     prm.out_align32 = ((((uintptr_t)dq | (uintptr_t)dk | (uintptr_t)dv) & 31) == 0 &&
                        ((p->stride_b | p->stride_h | p->stride_s) & 15) == 0) ? 1 : 0;
-    auto launch = [&](auto mode, const CUtensorMap &r1, const CUtensorMap &r2, const CUtensorMap &t1, const CUtensorMap &t2) {
-        constexpr int MODE = decltype(mode)::value;
-        auto go = [&](auto kernel) {
-            return launch_overlapping(kernel, (unsigned)p->n_bwd_cta, THREADS, SMEM_BYTES, (unsigned)p->bwd_cluster, stream, true, r1, r2,
-                                      t1, t2, prm);
-        };
-        if (p->bwd_cluster > 1)
-            return p->head_dim == 128 ? go(attn_bwd_kernel<MODE, 128, true>) : go(attn_bwd_kernel<MODE, 64, true>);
-        return p->head_dim == 128 ? go(attn_bwd_kernel<MODE, 128, false>) : go(attn_bwd_kernel<MODE, 64, false>);
+    prm.dq = (__nv_bfloat16 *)dq;
+    prm.dk = (__nv_bfloat16 *)dk;
+    prm.dv = (__nv_bfloat16 *)dv;
+    auto go = [&](auto kernel) {
+        return launch_overlapping(kernel, 2u * (unsigned)p->n_bwd_cta, THREADS, SMEM_BYTES, (unsigned)p->bwd_cluster, stream, true,
+                                  mq, mk, mv, mdo, prm);
     };
-    prm.out_a = (__nv_bfloat16 *)dk;
-    prm.out_b = (__nv_bfloat16 *)dv;
-    HB_CUDA(launch(std::integral_constant<int, MODE_DKV>{}, mk, mv, mq, mdo));
-    HB_LAUNCHED();
-    prm.out_a = (__nv_bfloat16 *)dq;
-    prm.out_b = nullptr;
-    HB_CUDA(launch(std::integral_constant<int, MODE_DQ>{}, mq, mdo, mk, mv));
+    if (p->bwd_cluster > 1) HB_CUDA(p->head_dim == 128 ? go(attn_bwd_kernel<128, true>) : go(attn_bwd_kernel<64, true>));
+    else HB_CUDA(p->head_dim == 128 ? go(attn_bwd_kernel<128, false>) : go(attn_bwd_kernel<64, false>));
     HB_LAUNCHED();
     return HILBERTA_OK;
 }
@@ -809,7 +804,7 @@ int launch_attn_bwd(const hilberta_plan_t *p, const void *dout, const void *q, c
 }  // namespace hilberta
 
 // ---------------------------------------------------------------------------
-// hilberta_backward_static: the same three launches with the delta scratch in a
+// hilberta_backward_static: the same launches with the delta scratch in a
 // fixed array that is part of the library image instead of memory obtained from
 // the CUDA allocator.  The array lives on every device that loads the library.
 // In host code its name is only a handle; the device address is looked up once
@@ -866,7 +861,7 @@ extern "C" int hilberta_backward_static(const void *dout, const void *q, const v
     float *delta = nullptr;
     const int rc = static_delta_address(dev, &delta);
     if (rc != HILBERTA_OK) return rc;
-    // delta_kernel overwrites every entry the two tensor-core kernels read, so whatever an
+    // delta_kernel overwrites every entry that the tensor-core kernel reads, so whatever an
     // earlier call left in the array is never seen and nothing has to be cleared
     return hilberta::launch_attn_bwd(p, dout, q, k, v, out, lse, dq, dk, dv, delta, (cudaStream_t)stream);
 }

@@ -164,8 +164,8 @@ namespace hilberta {
 // Programmatic dependent launch: the library's kernels allow the next one in the stream to be set up while
 // they drain (allow_next: once every CTA has said so), and each reads and writes nothing that an earlier
 // kernel could still touch before wait_for_previous has returned -- until then only its plan's tables, which
-// no kernel writes after the plan and its binding are made.  Every kernel waits, so its end implies the end
-// of all before it.  Saves the launch latency and the prologue between kernels, 1 ... 2 us each (one fused
+// no kernel writes after the plan and its binding are made.  Every kernel launched this way waits (some thread
+// of it at least) and the others are launched plainly, so a kernel's end implies the end of all before it.  Saves the launch latency and the prologue between kernels, 1 ... 2 us each (one fused
 // launch after another, 512^2 and 8 heads: 18.7 -> 16.6 us).  overlap = false: an ordinary launch.
 __device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
