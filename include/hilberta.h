@@ -367,6 +367,38 @@ int hilberta_check_work_list(const int32_t *items, int n_items, int S, int item_
 int hilberta_schedule_units(int n_items, const int64_t *cost, const int64_t *cost_two_heads, int bh, int n_cta,
                             int32_t *units, int32_t *cta_begin, int64_t *largest_load);
 
+/* How hilberta_plan_bind cuts the longest work items over clusters of CTAs, and the schedule that comes of it,
+ * computed as there (no GPU involved; exposed so that it can be tested and inspected).  A cut item's keys are
+ * shared out over the CTAs of a cluster, which run their shares at the same time and merge them; that the
+ * CTAs of a cluster list the same cut units, first and in the same order, keeps them from waiting for one
+ * another in vain.  (Algorithm 1 gives every query block to one program.)
+ *   items            n_items records as for hilberta_check_work_list, by descending cost
+ *   cost, cost_two_heads, bh
+ *                    as for hilberta_schedule_units (cost_two_heads may be NULL)
+ *   sm_count         CTAs that run at once; clusters[3]: clusters of 2, 4 and 8 CTAs that do (at most sm_count
+ *                    CTAs each)
+ *   block            keys per block; merge_extra: added to the cost of a share
+ *   chosen[3]        receives the cluster size (1: nothing is cut), the number of cut items -- the first ones
+ *                    of the list -- and the number of CTAs, a multiple of the cluster size
+ *   shares           receives chosen[0] records per cut item, in rank order (room for 8 n_items)
+ *   units            receives three int32 per unit, grouped by CTA: (item, index, second index or -1), or for
+ *                    a share (n_items + its record's number, index, -2); max_units: room, else ERR_BUFFER
+ *   cta_begin        receives sm_count + 1 offsets into units; CTA c has rank c modulo the cluster size
+ *   largest_load     if not NULL, the largest CTA load
+ * Errors: ERR_INVALID, ERR_BUFFER. */
+int hilberta_cut_schedule(const int32_t *items, int n_items, const int64_t *cost, const int64_t *cost_two_heads,
+                          int bh, int sm_count, const int32_t *clusters, int block, int64_t merge_extra,
+                          int32_t *chosen, int32_t *shares, int32_t *units, int max_units, int32_t *cta_begin,
+                          int64_t *largest_load);
+
+/* Host-side check of the shares of cut items (no GPU involved; hilberta_plan_bind runs it on those it makes and
+ * fails with ERR_INVALID rather than upload bad ones).  items: n_items records as for
+ * hilberta_check_work_list; shares: `cluster` records for each of them, in rank order.  Returns HILBERTA_OK iff
+ * every share has its item's rows, at least one key and the right number of blocks, and the key ranges of an
+ * item's shares, one after another, are the item's (Algorithm 1: every key counts once).  Otherwise
+ * ERR_INVALID. */
+int hilberta_check_shares(const int32_t *items, int n_items, const int32_t *shares, int cluster, int block);
+
 /* Host-side aliasing test the attention calls run on their pointer arguments (no GPU involved).
  * Two tensors of the layout [batch, heads, S, row] with the same BYTE strides and rows of row_bytes
  * contiguous bytes, at base addresses a and b: returns 1 if they share at least one byte, else 0.

@@ -31,7 +31,8 @@ SYMBOLS = (
     "hilberta_backward_static", "hilberta_permute",
     "hilberta_unpermute",
     "hilberta_forward_host",
-    "hilberta_check_work_list", "hilberta_check_overlap", "hilberta_schedule_units",
+    "hilberta_check_work_list", "hilberta_check_overlap", "hilberta_schedule_units", "hilberta_cut_schedule",
+    "hilberta_check_shares",
     "hilberta_plan_status", "hilberta_selftest_timeout", "hilberta_launch_count", "hilberta_status_string", "hilberta_version",
     "hilberta_last_cuda_error",
 )
@@ -98,6 +99,10 @@ def lib():
     L.hilberta_check_overlap.restype = i32
     L.hilberta_schedule_units.argtypes = [i32, vp, vp, i32, i32, vp, vp, vp]
     L.hilberta_schedule_units.restype = i32
+    L.hilberta_cut_schedule.argtypes = [vp, i32, vp, vp, i32, i32, vp, i32, i64, vp, vp, vp, i32, vp, vp]
+    L.hilberta_cut_schedule.restype = i32
+    L.hilberta_check_shares.argtypes = [vp, i32, vp, i32, i32]
+    L.hilberta_check_shares.restype = i32
     L.hilberta_selftest_timeout.argtypes = [vp, vp]
     L.hilberta_selftest_timeout.restype = i32
     L.hilberta_plan_status.argtypes = [vp]
@@ -137,6 +142,34 @@ def schedule_units(cost, cost_two_heads, bh: int, n_cta: int):
     _check(lib().hilberta_schedule_units(len(c1), c1.ctypes.data, None if c2 is None else c2.ctypes.data, int(bh), int(n_cta),
                                          units.ctypes.data, begin.ctypes.data, ctypes.addressof(load)), "hilberta_schedule_units")
     return units[:begin[-1]], begin, int(load.value)
+
+
+def cut_schedule(items, cost, cost_two_heads, bh: int, sm_count: int, clusters, block: int, merge_extra: int = 0):
+    """hilberta_cut_schedule (host only): (cluster, cut items, CTAs, shares [cut items * cluster, 10], units [n, 3],
+    cta_begin [CTAs + 1], largest load)."""
+    a = np.ascontiguousarray(items, dtype=np.int32).reshape(-1, 10)
+    n = a.shape[0]
+    c1 = np.ascontiguousarray(cost, dtype=np.int64)
+    c2 = None if cost_two_heads is None else np.ascontiguousarray(cost_two_heads, dtype=np.int64)
+    cl = np.ascontiguousarray(clusters, dtype=np.int32)
+    chosen, shares = np.zeros(3, dtype=np.int32), np.zeros((8 * n, 10), dtype=np.int32)
+    units, begin = np.zeros((8 * n * int(bh), 3), dtype=np.int32), np.zeros(int(sm_count) + 1, dtype=np.int32)
+    load = ctypes.c_int64(0)
+    _check(lib().hilberta_cut_schedule(a.ctypes.data, n, c1.ctypes.data, None if c2 is None else c2.ctypes.data, int(bh),
+                                       int(sm_count), cl.ctypes.data, int(block), int(merge_extra), chosen.ctypes.data,
+                                       shares.ctypes.data, units.ctypes.data, len(units), begin.ctypes.data,
+                                       ctypes.addressof(load)), "hilberta_cut_schedule")
+    cluster, cut, n_cta = (int(x) for x in chosen)
+    return cluster, cut, n_cta, shares[:cut * cluster], units[:begin[n_cta]], begin[:n_cta + 1], int(load.value)
+
+
+def check_shares(items, shares, cluster: int, block: int) -> int:
+    """Status of hilberta_check_shares for [n, 10] items and their [n * cluster, 10] shares (host only)."""
+    a = np.ascontiguousarray(items, dtype=np.int32).reshape(-1, 10)
+    b = np.ascontiguousarray(shares, dtype=np.int32).reshape(-1, 10)
+    if len(b) != len(a) * int(cluster):
+        raise ValueError("cluster shares for every item")
+    return int(lib().hilberta_check_shares(a.ctypes.data, len(a), b.ctypes.data, int(cluster), int(block)))
 
 
 def _check(status: int, where: str):

@@ -1199,7 +1199,8 @@ int attn_bf16_prepare(hilberta_plan_t *p, BindImage &image) {
     // How the longest items are cut over clusters is decided once, for the whole problem: a slice of heads
     // then gives every row the same sums in the same order.
     SplitChoice choice;
-    choose_split(items, cost, cost_two_heads, p->batch * p->heads, p->sm_count, split_clusters(p->device), BN, choice);
+    rc = choose_split(items, cost, cost_two_heads, p->batch * p->heads, p->sm_count, split_clusters(p->device), BN, choice);
+    if (rc != HILBERTA_OK) return rc;
     p->split_cluster = choice.cluster;
     for (const WorkItem &it : choice.shares) items.push_back(it);
     image.add(items, &p->d_work);

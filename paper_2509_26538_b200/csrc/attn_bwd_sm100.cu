@@ -743,7 +743,8 @@ int attn_bwd_prepare(hilberta_plan_t *p, BindImage &image) {
     // The two modes share the chip, so a cut has to gain more than in the forward pass (geometric mean of 36
     // problems of all sizes, forward included: 90.2 us without this, 86.9 with 100, 87.9 with 300, 101.6 uncut)
     choice.merge_extra = 100;
-    choose_split(items, cost, unpaired, bh, p->sm_count, clusters, BK, choice);
+    rc = choose_split(items, cost, unpaired, bh, p->sm_count, clusters, BK, choice);
+    if (rc != HILBERTA_OK) return rc;
     p->bwd_cluster = choice.cluster;
     for (const WorkItem &it : choice.shares) items.push_back(it);
     image.add(items, &p->d_bwd_work);

@@ -206,6 +206,7 @@ int launch_attn_bf16(const hilberta_plan_t *p, const void *q, const void *k, con
 std::vector<WorkItem> build_work_items(const hilberta_plan_t *p, int item_rows, int block);
 // HILBERTA_OK iff the list is safe to hand to a kernel (ranges inside [0, S), rows covered exactly once)
 int check_work_items(const WorkItem *items, int n, int S, int item_rows, int block);
+int check_shares(const WorkItem *items, int n, const WorkItem *shares, int cluster, int block);
 // How a schedule cuts its longest items (the first n_items of the list) over clusters of `cluster` CTAs;
 // shares: cluster entries per cut item, in rank order, appended to the uploaded work list.
 struct SplitChoice {
@@ -215,10 +216,10 @@ struct SplitChoice {
     std::vector<WorkItem> shares;
 };
 // clusters: how many clusters of 2, 4 and 8 CTAs run at once.  items sorted by descending cost.  Of
-// `choice` only merge_extra is read.
-void choose_split(const std::vector<WorkItem> &items, const std::vector<long long> &cost,
-                  const std::vector<long long> &cost_two_heads, int bh, int sm_count, const int *clusters, int block,
-                  SplitChoice &choice);
+// `choice` only merge_extra is read.  Not HILBERTA_OK: the shares are not safe to hand to a kernel.
+int choose_split(const std::vector<WorkItem> &items, const std::vector<long long> &cost,
+                 const std::vector<long long> &cost_two_heads, int bh, int sm_count, const int *clusters, int block,
+                 SplitChoice &choice);
 // The schedule of such a choice (units null: none is written); returns the largest CTA load.
 // cost_two_heads: empty, or per item the cost of running it for TWO (batch, head) indices in one unit
 // (0: the item is not paired); such items become units of two consecutive indices.

@@ -85,6 +85,35 @@ int check_work_items(const WorkItem *items, int n, int S, int item_rows, int blo
     return next == S ? HILBERTA_OK : HILBERTA_ERR_INVALID;
 }
 
+// The same for the shares of cut items (cluster entries per item, in rank order): the rows of the item, and
+// key ranges that make up the item's when read one after another, a block at least in every share.
+int check_shares(const WorkItem *items, int n, const WorkItem *shares, int cluster, int block) {
+    if (n < 0 || cluster < 1 || block < 1 || (n > 0 && (!items || !shares))) return HILBERTA_ERR_INVALID;
+    for (int i = 0; i < n; ++i) {
+        const WorkItem &it = items[i];
+        int seg = 0, done = 0;   // the keys before position `done` of the item's range `seg` have been taken
+        for (int r = 0; r < cluster; ++r) {
+            const WorkItem &s = shares[i * cluster + r];
+            if (s.q_start != it.q_start || s.q_rows != it.q_rows || s.n_seg < 1 || s.n_seg > 3) return HILBERTA_ERR_INVALID;
+            long long blocks = 0;
+            for (int a = 0; a < s.n_seg; ++a) {
+                if (seg >= it.n_seg || s.seg_len[a] < 1 || s.seg_len[a] > it.seg_len[seg] - done ||
+                    s.seg_start[a] != it.seg_start[seg] + done)
+                    return HILBERTA_ERR_INVALID;
+                done += s.seg_len[a];
+                if (done == it.seg_len[seg]) {
+                    ++seg;
+                    done = 0;
+                }
+                blocks += (s.seg_len[a] + block - 1) / block;
+            }
+            if (blocks != s.kv_blocks) return HILBERTA_ERR_INVALID;
+        }
+        if (seg != it.n_seg) return HILBERTA_ERR_INVALID;   // keys that no share has
+    }
+    return HILBERTA_OK;
+}
+
 // ---------------------------------------------------------------------------
 // Items cut over clusters.  A prefix item's key list is the whole sequence; with few heads a handful of
 // them outlasts everything else (3 heads at 2048^2: 9 units of 132 blocks against 26 blocks per SM of
@@ -213,9 +242,9 @@ static WorkItem share_of(const WorkItem &it, int lo, int hi, int block) {
     return s;
 }
 
-void choose_split(const std::vector<WorkItem> &items, const std::vector<long long> &cost,
-                  const std::vector<long long> &cost_two_heads, int bh, int sm_count, const int *clusters, int block,
-                  SplitChoice &choice) {
+int choose_split(const std::vector<WorkItem> &items, const std::vector<long long> &cost,
+                 const std::vector<long long> &cost_two_heads, int bh, int sm_count, const int *clusters, int block,
+                 SplitChoice &choice) {
     const long long merge_extra = choice.merge_extra;
     choice = SplitChoice();
     choice.merge_extra = merge_extra;
@@ -230,7 +259,7 @@ void choose_split(const std::vector<WorkItem> &items, const std::vector<long lon
     };
     long long best = load_of(choice);
     // within 3 % of a perfect balance nothing is to be gained
-    if (best * sm_count <= total + total / 32) return;
+    if (best * sm_count <= total + total / 32) return HILBERTA_OK;
     // (units per head instead of per two only matter where there are CTAs to take them)
     const bool few = n_units < 2ll * sm_count;
     if (few) {
@@ -279,6 +308,7 @@ void choose_split(const std::vector<WorkItem> &items, const std::vector<long lon
             choice.shares.push_back(share_of(items[i], (int)((long long)n * r / choice.cluster),
                                              (int)((long long)n * (r + 1) / choice.cluster), block));
     }
+    return check_shares(items.data(), choice.n_items, choice.shares.data(), choice.cluster, block);
 }
 
 // Adds the units grouped by CTA and the n_cta + 1 offsets to the image.
@@ -319,6 +349,42 @@ extern "C" int hilberta_schedule_units(int n_items, const int64_t *cost, const i
         units[3 * i + 2] = u[i].bh2;
     }
     for (int c = 0; c <= n_cta; ++c) cta_begin[c] = c < (int)cb.size() ? cb[c] : (int)u.size();
+    if (largest_load) *largest_load = m;
+    return HILBERTA_OK;
+}
+
+extern "C" int hilberta_check_shares(const int32_t *items, int n_items, const int32_t *shares, int cluster, int block) {
+    return hilberta::check_shares(reinterpret_cast<const hilberta::WorkItem *>(items), n_items,
+                                  reinterpret_cast<const hilberta::WorkItem *>(shares), cluster, block);
+}
+
+extern "C" int hilberta_cut_schedule(const int32_t *items, int n_items, const int64_t *cost, const int64_t *cost_two_heads,
+                                     int bh, int sm_count, const int32_t *clusters, int block, int64_t merge_extra,
+                                     int32_t *chosen, int32_t *shares, int32_t *units, int max_units, int32_t *cta_begin,
+                                     int64_t *largest_load) {
+    if (n_items < 1 || bh < 1 || sm_count < 1 || block < 1 || !items || !cost || !clusters || !chosen || !shares || !units ||
+        !cta_begin || (long long)n_items * bh > (1ll << 27))
+        return HILBERTA_ERR_INVALID;
+    for (int k = 0; k < 3; ++k)
+        if ((long long)clusters[k] << (k + 1) > sm_count) return HILBERTA_ERR_INVALID;
+    const hilberta::WorkItem *list = reinterpret_cast<const hilberta::WorkItem *>(items);
+    const std::vector<hilberta::WorkItem> its(list, list + n_items);
+    std::vector<long long> c1(cost, cost + n_items), c2((size_t)n_items, 0);
+    if (cost_two_heads) c2.assign(cost_two_heads, cost_two_heads + n_items);
+    hilberta::SplitChoice choice;
+    choice.merge_extra = merge_extra;
+    const int rc = hilberta::choose_split(its, c1, c2, bh, sm_count, clusters, block, choice);
+    if (rc != HILBERTA_OK) return rc;
+    std::vector<hilberta::WorkUnit> u;
+    std::vector<int> cb;
+    const long long m = hilberta::build_schedule(c1, c2, bh, sm_count, choice, &u, &cb);
+    if ((int)u.size() > max_units) return HILBERTA_ERR_BUFFER;
+    memcpy(units, u.data(), sizeof(hilberta::WorkUnit) * u.size());
+    if (!choice.shares.empty()) memcpy(shares, choice.shares.data(), sizeof(hilberta::WorkItem) * choice.shares.size());
+    for (int c = 0; c <= sm_count; ++c) cta_begin[c] = c < (int)cb.size() ? cb[c] : (int)u.size();
+    chosen[0] = choice.cluster;
+    chosen[1] = choice.n_items;
+    chosen[2] = (int)cb.size() - 1;
     if (largest_load) *largest_load = m;
     return HILBERTA_OK;
 }
