@@ -237,7 +237,7 @@ int hilberta_forward_lse(const void *q, const void *k, const void *v, void *out,
  * dq, dk, dv         : device pointers, written; same shape and strides as q; must
  *                      not alias each other or any input.  Every row is written.
  * All pointers 16-byte aligned (lse: 4).  Asynchronous on `stream`; two kernel
- * launches; no allocation, no synchronisation.  A per-row scratch array
+ * launches (fp32 bindings with windows of a few tokens: three); no allocation, no synchronisation.  A per-row scratch array
  * (2 * batch * heads * S floats, owned by the plan, allocated by hilberta_plan_bind)
  * carries lse * log2(e) and delta between the launches, so two backward calls on
  * the same plan must not overlap on the device.

@@ -23,13 +23,12 @@ constexpr int kDeltaRows = 4;
 template <int D>
 __global__ void __launch_bounds__(kDeltaRows * 32)
 delta_fp32_kernel(const float *__restrict__ dout, const float *__restrict__ out, float *__restrict__ delta,
-                  long long stride_b, long long stride_h, long long stride_s, int heads, int S, long long rows) {
+                  long long stride_b, long long stride_h, long long stride_s, int heads, int S) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long at = (long long)blockIdx.x * kDeltaRows + warp;   // (batch * head, row)
+    const int bh = blockIdx.y, row = (int)blockIdx.x * kDeltaRows + warp;
     allow_next();
     wait_for_previous();
-    if (at >= rows) return;
-    const int bh = (int)(at / S), row = (int)(at % S);
+    if (row >= S) return;
     const long long off = (long long)(bh / heads) * stride_b + (long long)(bh % heads) * stride_h +
                           (long long)row * stride_s;
     float acc = 0.f;
@@ -37,7 +36,7 @@ delta_fp32_kernel(const float *__restrict__ dout, const float *__restrict__ out,
     for (int e = 0; e < D / 32; ++e) acc = fmaf(dout[off + lane + 32 * e], out[off + lane + 32 * e], acc);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) delta[at] = acc;
+    if (lane == 0) delta[(long long)bh * S + row] = acc;
 }
 
 template <int D>
@@ -200,21 +199,102 @@ attn_fp32_bwd_kernel(const float *__restrict__ q, const float *__restrict__ k, c
         bwd_tile<D, 0>(q + base, dout + base, k + base, v + base, lse, delta, dq + base, nullptr, stride_s, it, share, scale);
 }
 
+// The rows of short lists, one mode for one warp: the row in registers, the streamed rows one after another.
+template <int D, int MODE>
+__device__ __forceinline__ void bwd_row(const float *r1, const float *r2, const float *t1, const float *t2, const float *lse,
+                                        const float *delta, float *out_a, float *out_b, long long stride_s,
+                                        const SingleRow &it, float scale) {
+    constexpr int E = D / 32;
+    const int lane = threadIdx.x & 31;
+    const long long at = (long long)it.row * stride_s + lane;
+    float a1[E], a2[E], acc_a[E], acc_b[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        a1[e] = r1[at + 32 * e];
+        a2[e] = r2[at + 32 * e];
+        acc_a[e] = acc_b[e] = 0.f;
+    }
+    const float row_lse = lse[it.row], row_delta = delta[it.row];
+    for (int s = 0; s < 3; ++s) {
+        const int end = it.start[s] + it.len[s];
+        for (int j = it.start[s]; j < end; ++j) {
+            const float *x1 = t1 + (long long)j * stride_s + lane, *x2 = t2 + (long long)j * stride_s + lane;
+            float b1[E], b2[E], dot1 = 0.f, dot2 = 0.f;
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                b1[e] = __ldg(x1 + 32 * e);
+                b2[e] = __ldg(x2 + 32 * e);
+                dot1 = fmaf(a1[e], b1[e], dot1);
+                dot2 = fmaf(a2[e], b2[e], dot2);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                dot1 += __shfl_xor_sync(0xffffffffu, dot1, o);
+                dot2 += __shfl_xor_sync(0xffffffffu, dot2, o);
+            }
+            // the statistics belong to the QUERY of the pair
+            const float p = expf(fmaf(dot1, scale, -(MODE == 0 ? row_lse : __ldg(lse + j))));
+            const float ds = p * (dot2 - (MODE == 0 ? row_delta : __ldg(delta + j)));
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                acc_a[e] = fmaf(ds, b1[e], acc_a[e]);                   // dq += dS k  |  dk += dS q
+                if (MODE == 1) acc_b[e] = fmaf(p, b2[e], acc_b[e]);     //             |  dv += P dO
+            }
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        out_a[at + 32 * e] = acc_a[e] * scale;
+        if (MODE == 1) out_b[at + 32 * e] = acc_b[e];
+    }
+}
+
+// Bound by the shuffles and, with few keys a row, by how fast CTAs start, hence eight rows to a CTA, as few
+// registers as let 64 warps run on an SM, and a row's ranges in its own record (48 x 48 tokens, tiles of 4, 48 heads
+// of 64, with the row statistics: 139 us; four rows, 40 registers and a table lookup 173; 32: 120, 128). z: the direction,
+// the one with more work per pair first.
+constexpr int kBwdRows = 8;
+template <int D>
+__global__ void __launch_bounds__(kBwdRows * 32, D == 128 ? 5 : 8)
+attn_fp32_bwd_rows_kernel(const float *__restrict__ q, const float *__restrict__ k, const float *__restrict__ v,
+                          const float *__restrict__ dout, const float *__restrict__ lse, const float *__restrict__ delta,
+                          float *__restrict__ dq, float *__restrict__ dk, float *__restrict__ dv, long long stride_b,
+                          long long stride_h, long long stride_s, int heads, int S, int P,
+                          const Fp32Row *__restrict__ rows, int n_rows, float scale) {
+    const SingleRow it(rows, n_rows, P, (int)blockIdx.x * kBwdRows + (int)(threadIdx.x >> 5));
+    allow_next();
+    wait_for_previous();
+    if (it.row < 0) return;
+    const int bh = blockIdx.y;
+    const long long base = (long long)(bh / heads) * stride_b + (long long)(bh % heads) * stride_h;
+    lse += (long long)bh * S;
+    delta += (long long)bh * S;
+    if (blockIdx.z == 0) bwd_row<D, 1>(k + base, v + base, q + base, dout + base, lse, delta, dk + base, dv + base, stride_s, it, scale);
+    else bwd_row<D, 0>(q + base, dout + base, k + base, v + base, lse, delta, dq + base, nullptr, stride_s, it, scale);
+}
+
 template <int D>
 int launch(const hilberta_plan_t *p, const float *dout, const float *q, const float *k, const float *v,
            const float *out, const float *lse, float *dq, float *dk, float *dv, float *delta, cudaStream_t stream) {
-    if (p->n_f32_work == 0) return HILBERTA_OK;
-    const long long rows = (long long)p->batch * p->heads * p->S;
-    HB_CUDA(launch_overlapping(delta_fp32_kernel<D>, (unsigned)((rows + kDeltaRows - 1) / kDeltaRows), kDeltaRows * 32, 0, 1, stream, true, dout,
-                               out, delta, p->stride_b, p->stride_h, p->stride_s, p->heads, p->S, rows));
+    const Fp32Work &w = p->f32_bwd;
+    const int bhs = p->batch * p->heads;
+    const long long ctas = items_grid(w, 2 * bhs);
+    if (ctas > 0x7fffffffll) return HILBERTA_ERR_INVALID;
+    HB_CUDA(launch_overlapping(delta_fp32_kernel<D>, dim3((p->S + kDeltaRows - 1) / kDeltaRows, bhs), kDeltaRows * 32, 0, 1, stream,
+                               true, dout, out, delta, p->stride_b, p->stride_h, p->stride_s, p->heads, p->S));
     HB_LAUNCHED();
-    const long long ctas = grid_of(p, 2);
-    if (ctas > 0x7fffffffll || (rows + kDeltaRows - 1) / kDeltaRows > 0x7fffffffll) return HILBERTA_ERR_INVALID;
-    HB_CUDA(launch_overlapping(attn_fp32_bwd_kernel<D>, (unsigned)ctas, kThreads, bwd_smem<D>(), (unsigned)p->f32_cluster, stream, may_overlap(p, ctas), q, k, v,
-                               dout, lse, delta, dq, dk, dv, p->stride_b, p->stride_h, p->stride_s, p->heads,
-                               p->batch * p->heads, p->S, p->d_f32_work, p->n_f32_work, p->n_f32_split, p->f32_cluster,
-                               p->scale));
-    HB_LAUNCHED();
+    if (ctas > 0) {
+        HB_CUDA(launch_overlapping(attn_fp32_bwd_kernel<D>, (unsigned)ctas, kThreads, bwd_smem<D>(), (unsigned)w.cluster, stream,
+                                   may_overlap(p, ctas), q, k, v, dout, lse, delta, dq, dk, dv, p->stride_b, p->stride_h,
+                                   p->stride_s, p->heads, bhs, p->S, w.items, w.n_items, w.n_split, w.cluster, p->scale));
+        HB_LAUNCHED();
+    }
+    if (w.n_rows > 0) {
+        HB_CUDA(launch_overlapping(attn_fp32_bwd_rows_kernel<D>, dim3((w.n_rows + kBwdRows - 1) / kBwdRows, bhs, 2), kBwdRows * 32, 0, 1,
+                                   stream, true, q, k, v, dout, lse, delta, dq, dk, dv, p->stride_b, p->stride_h, p->stride_s,
+                                   p->heads, p->S, p->P, w.rows, w.n_rows, p->scale));
+        HB_LAUNCHED();
+    }
     return HILBERTA_OK;
 }
 

@@ -214,11 +214,27 @@ __device__ __forceinline__ void load_block(float *tile, const float *base, long 
     }
 }
 
-// CTAs of a launch over a plan's fp32 work list: `directions` instances per (batch, head) and item, whole clusters.
-inline long long grid_of(const hilberta_plan_t *p, int directions) {
-    const long long c = p->f32_cluster, columns = (long long)p->batch * p->heads * directions;
-    const long long single = (p->n_f32_work - p->n_f32_split) * columns;
-    return p->n_f32_split * columns * c + (single + c - 1) / c * c;
+// Rows whose key lists are so short that a CTA of 64 is not worth while have a warp each, kRowsPerCta to a CTA.
+constexpr int kRowsPerCta = kThreads / 32;
+struct SingleRow {
+    int row;   // < 0: none left
+    int start[3], len[3];
+    __device__ __forceinline__ SingleRow(const Fp32Row *rows, int n_rows, int P, int at) {
+        const Fp32Row r = rows[min(at, n_rows - 1)];
+        row = at < n_rows ? r.row : -1;
+        start[0] = 0;
+        len[0] = P;
+        start[1] = r.seg0_start;
+        len[1] = r.seg0_len;
+        start[2] = r.seg1_start;
+        len[2] = r.seg1_len;
+    }
+};
+
+// CTAs of a launch over the items: `columns` instances of each, whole clusters.
+inline long long items_grid(const Fp32Work &w, long long columns) {
+    const long long c = w.cluster, single = (w.n_items - w.n_split) * columns;
+    return w.n_split * columns * c + (single + c - 1) / c * c;
 }
 
 // Several CTAs of these kernels share an SM.  One that is set up while the kernel before it still runs goes

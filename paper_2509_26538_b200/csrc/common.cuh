@@ -61,6 +61,19 @@ struct WorkUnit {
     int bh2;
 };
 
+// What one direction of an fp32 binding works through: items of up to 64 rows by descending key count, of
+// which the first n_split are cut over clusters of `cluster` CTAs; and single rows, those of windows too short
+// for an item of their own, with a warp each.
+struct __align__(16) Fp32Row {
+    int row, seg0_start, seg0_len, seg1_start, seg1_len, unused[3];   // the window's ranges by value: one trip to memory
+};
+struct Fp32Work {
+    WorkItem *items;
+    int n_items, n_split, cluster;
+    Fp32Row *rows;
+    int n_rows;
+};
+
 // Tables of a binding, gathered on the host: one allocation and one copy for all of them (every
 // cudaMalloc, cudaFree and pageable copy is tens of microseconds of a bind).  `where` receives the device
 // address; scratch lies behind the tables, uninitialised.
@@ -148,10 +161,7 @@ struct hilberta_plan_s {
     int *d_bwd_cta_begin;
     int n_bwd_cta, bwd_cluster;
     float *d_delta;               // [batch * heads * S]
-    // fp32 bindings: items of 64 rows by descending key count; the first n_f32_split of them are cut over
-    // clusters of f32_cluster CTAs
-    hilberta::WorkItem *d_f32_work;
-    int n_f32_work, n_f32_split, f32_cluster;
+    hilberta::Fp32Work f32_fwd, f32_bwd;   // fp32 bindings
     int *d_status;  // [4] error word + diagnostics written by bounded waits
     // workspace of hilberta_forward_host
     void *ws;
@@ -171,7 +181,7 @@ __device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.laun
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <class... Params, class... Args>
-cudaError_t launch_overlapping(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, unsigned cluster,
+cudaError_t launch_overlapping(void (*kernel)(Params...), dim3 grid, unsigned block, size_t smem, unsigned cluster,
                                cudaStream_t stream, bool overlap, const Args &...args) {
     cudaLaunchAttribute attr[2] = {};
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -180,7 +190,7 @@ cudaError_t launch_overlapping(void (*kernel)(Params...), unsigned grid, unsigne
     attr[1].val.clusterDim.x = cluster;
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t config{};
-    config.gridDim = dim3(grid);
+    config.gridDim = grid;
     config.blockDim = dim3(block);
     config.dynamicSmemBytes = smem;
     config.stream = stream;
