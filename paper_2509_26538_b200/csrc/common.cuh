@@ -118,7 +118,6 @@ struct hilberta_plan_s {
     int *d_hil_d2t, *d_hil_t2d;      // [HW]
     int *d_c;                        // [NP + 1] real non-shared cells with padded Hilbert index below d
     int *d_phys2orig, *d_orig2phys;  // [S]
-    int *d_row_window;               // [S] window id of a physical row, -1 for prefix rows
     hilberta::Window *d_windows;     // [T]
     // host mirrors of the small tables
     std::vector<hilberta::Window> h_windows;

@@ -193,20 +193,15 @@ __global__ void cell_scan_kernel(const unsigned char *__restrict__ kind_by_pd, i
 // Appendix A layout: text first, then shared tokens, then the rest, each image
 // group by ascending Hilbert index.  One thread per original token.  Also the
 // rank tables (Hilbert index among the real cells <-> cell).
-// compact_R > 0 selects the group arithmetic of Algorithm 1: tile ids follow the position
-// in the non-shared sequence (c_ns) instead of the position on the padded curve.
-__global__ void layout_kernel(int HW, int NP, int n_text, int P, int tile, int offset, int compact_R,
-                              const int *__restrict__ pd_of_cell, const int *__restrict__ c_ns,
+__global__ void layout_kernel(int HW, int n_text, int P, const int *__restrict__ pd_of_cell, const int *__restrict__ c_ns,
                               const int *__restrict__ c_real, const unsigned char *__restrict__ kind_by_pd,
                               int *__restrict__ hil_d2t, int *__restrict__ hil_t2d,
-                              int *__restrict__ phys2orig, int *__restrict__ orig2phys,
-                              int *__restrict__ row_window) {
+                              int *__restrict__ phys2orig, int *__restrict__ orig2phys) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n_text + HW) return;
     if (t < n_text) {
         phys2orig[t] = t;
         orig2phys[t] = t;
-        row_window[t] = -1;
         return;
     }
     const int cell = t - n_text;
@@ -215,14 +210,7 @@ __global__ void layout_kernel(int HW, int NP, int n_text, int P, int tile, int o
     hil_t2d[cell] = rank;
     hil_d2t[rank] = cell;
     const int below = c_ns[d];
-    int phys;
-    if (kind_by_pd[d] == CELL_SHARED) {
-        phys = n_text + (rank - below);
-        row_window[phys] = -1;
-    } else {
-        phys = P + below;
-        row_window[phys] = compact_R > 0 ? ((below + offset) % compact_R) / tile : ((d + offset) % NP) / tile;
-    }
+    const int phys = kind_by_pd[d] == CELL_SHARED ? n_text + (rank - below) : P + below;
     phys2orig[phys] = t;
     orig2phys[t] = phys;
 }
@@ -440,7 +428,7 @@ static int build_plan(hilberta_plan_t *p) {
     };
     const size_t windows = sizeof(Window) * p->T;
     const size_t o_d2t = place(sizeof(int) * HW), o_t2d = place(sizeof(int) * HW), o_c = place(sizeof(int) * (NP + 1));
-    const size_t o_p2o = place(sizeof(int) * S), o_o2p = place(sizeof(int) * S), o_rw = place(sizeof(int) * S);
+    const size_t o_p2o = place(sizeof(int) * S), o_o2p = place(sizeof(int) * S);
     const size_t o_status = place(sizeof(int) * 4096), o_win = place(windows + (size_t)NP), o_kind = o_win + windows;
     const size_t o_pd = place(sizeof(int) * HW), o_real = place(sizeof(int) * (NP + 1));   // needed here only
     p->plan_bytes = bytes;
@@ -451,7 +439,6 @@ static int build_plan(hilberta_plan_t *p) {
     p->d_c = (int *)(base + o_c);
     p->d_phys2orig = (int *)(base + o_p2o);
     p->d_orig2phys = (int *)(base + o_o2p);
-    p->d_row_window = (int *)(base + o_rw);
     p->d_status = (int *)(base + o_status);
     p->d_windows = (Window *)(base + o_win);
     unsigned char *d_kind = (unsigned char *)(base + o_kind);
@@ -470,9 +457,8 @@ static int build_plan(hilberta_plan_t *p) {
     g_launches.fetch_add(1);
     cell_scan_kernel<<<1, 1024>>>(d_kind, NP, p->d_c, d_c_real);
     g_launches.fetch_add(1);
-    layout_kernel<<<(S + 255) / 256, 256>>>(HW, NP, p->n_text, p->P, p->tile, p->offset, p->compact ? S - p->P : 0,
-                                            d_pd_of_cell, p->d_c, d_c_real, d_kind, p->d_hil_d2t, p->d_hil_t2d,
-                                            p->d_phys2orig, p->d_orig2phys, p->d_row_window);
+    layout_kernel<<<(S + 255) / 256, 256>>>(HW, p->n_text, p->P, d_pd_of_cell, p->d_c, d_c_real, d_kind, p->d_hil_d2t,
+                                            p->d_hil_t2d, p->d_phys2orig, p->d_orig2phys);
     g_launches.fetch_add(1);
     if (p->compact)
         window_compact_kernel<<<(p->T + 127) / 128, 128>>>(S - p->P, p->T, p->tile, p->offset, p->P, p->d_windows);
