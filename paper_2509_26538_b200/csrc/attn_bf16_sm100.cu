@@ -231,12 +231,15 @@ __device__ __forceinline__ void merge_parts(const Params &prm, const WorkItem &w
 #pragma unroll
     for (int p = 1; p < C; ++p) m = fmaxf(m, st[p].x);
     float l = 0.f, l_fix = 0.f, w[C];
+    bool none[C];
 #pragma unroll
     for (int p = 0; p < C; ++p) {
-        // weight 0: not even a NaN of that share counts (a share of nothing but -inf scores has no maximum)
+        // A share of nothing but -inf scores has no maximum, and its sums are NaN; beside other shares it counts for
+        // nothing.  A NaN of any other share reaches the result, however small that share's weight.
+        none[p] = st[p].x == -INFINITY && m != -INFINITY;
         w[p] = ex2(st[p].x - m);
-        l = w[p] != 0.f ? fmaf(st[p].y, w[p], l) : l;
-        l_fix = w[p] != 0.f ? fmaf(st[p].z, w[p], l_fix) : l_fix;
+        l = none[p] ? l : fmaf(st[p].y, w[p], l);
+        l_fix = none[p] ? l_fix : fmaf(st[p].z, w[p], l_fix);
     }
     const float inv = 1.f / (l + l_fix);
 #pragma unroll
@@ -250,7 +253,7 @@ __device__ __forceinline__ void merge_parts(const Params &prm, const WorkItem &w
                 a[e] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                 for (int p = 0; p < C; ++p) {
-                    if (w[p] == 0.f) continue;
+                    if (none[p]) continue;
                     a[e].x = fmaf(x[g][p][e].x, w[p], a[e].x);
                     a[e].y = fmaf(x[g][p][e].y, w[p], a[e].y);
                     a[e].z = fmaf(x[g][p][e].z, w[p], a[e].z);

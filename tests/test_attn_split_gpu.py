@@ -78,3 +78,38 @@ def test_two_streams_share_a_plan():
     for w, outs in zip(want, got):
         assert all(torch.equal(w.view(torch.int16), t.view(torch.int16)) for t in outs)
     plan.destroy()
+
+
+@pytest.mark.parametrize("D,fp8", [(128, False), (64, False), (128, True)])
+def test_values_that_are_not_finite(D, fp8):
+    """Keys of the first half score far below those of the second, so that their share of the weight is exactly zero:
+    a NaN among their values is in the result all the same, and scores of -inf there are not."""
+    H = W = 64
+    plan = hb.Plan(H, W, 512, 0, 8, 512)
+    S, P, heads = plan.S, 512 + 64, 3
+    g = torch.Generator(device="cuda")
+    g.manual_seed(2)
+    dt = torch.float8_e4m3fn if fp8 else torch.bfloat16
+    d = torch.randn(D, generator=g, device="cuda").sign()
+    q = (12 * d).expand(1, heads, S, D).contiguous()
+    k = torch.where(torch.arange(S, device="cuda")[:, None] < S // 2, -12 * d, 12 * d).expand(1, heads, S, D).contiguous()
+    v = torch.randn((1, heads, S, D), generator=g, device="cuda")
+    q, k, v = q.to(dt), k.to(dt), v.to(dt)
+    plan.bind_like(q)
+    out = torch.empty((1, heads, S, D), dtype=torch.bfloat16, device="cuda")
+    plan.forward(q, k, v, out)
+    want = v[:, :, S // 2:].double().mean(2, keepdim=True)   # the second half's keys weigh the same
+    assert (out[:, :, :P].double() - want).abs().max() <= 2 ** -6
+    for at in (0, 600, S // 2 - 1, S - 1):
+        bad = v.clone()
+        bad.view(torch.uint8 if fp8 else torch.int16)[0, 1, at, 5] = 0x7f if fp8 else 0x7fc0
+        plan.forward(q, k, bad, out)
+        assert torch.isnan(out[0, 1, :P, 5].float()).all(), at
+        assert torch.isfinite(out[0, 0, :P].float()).all() and torch.isfinite(out[0, 2, :P].float()).all()
+    if not fp8:   # finite keys whose scores overflow
+        k[:, :, S // 2:] = 0   # the others score 0
+        k[:, :, S - 200:S - 100] = (-3e38 * d).to(dt)
+        plan.forward(q, k, v, out)
+        assert torch.isfinite(out[:, :, :P].float()).all()
+    assert plan.status() == 0
+    plan.destroy()
