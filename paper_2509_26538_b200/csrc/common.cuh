@@ -5,6 +5,7 @@
 #include <string.h>
 
 #include <atomic>
+#include <new>
 #include <vector>
 
 #include "hilberta.h"
@@ -28,6 +29,17 @@ extern std::atomic<uint64_t> g_launches;
         ::hilberta::g_launches.fetch_add(1);           \
         HB_CUDA(cudaGetLastError());                   \
     } while (0)
+
+// The body of a C entry point that builds tables on the host: no exception leaves the library (the containers throw
+// when memory runs out or a size is beyond them, nothing else here does).
+template <class F>
+int guarded(F body) noexcept {
+    try {
+        return body();
+    } catch (...) {
+        return HILBERTA_ERR_NOMEM;
+    }
+}
 
 // One slid tile of the partition (Sec. 3.2) in physical coordinates: the
 // non-shared members of Hilbert interval [lo, lo + tile) mod HW occupy seg0

@@ -379,15 +379,16 @@ cudaError_t take_block(int device, void **ptr, size_t *bytes) {
 void give_block(int device, void *ptr, size_t bytes) {
     if (!ptr) return;
     std::vector<Block> out;
-    {
+    const int rc = guarded([&] {
         std::lock_guard<std::mutex> lock(g_blocks_mutex);
-        size_t held = bytes, n = 1;
+        out.reserve(g_blocks.size() + 1);
+        g_blocks.push_back(Block{device, ptr, bytes, g_blocks_given++, false});
+        size_t held = 0, n = 0;
         for (const Block &b : g_blocks)
             if (b.device == device) {
                 held += b.bytes;
                 ++n;
             }
-        g_blocks.push_back(Block{device, ptr, bytes, g_blocks_given++, false});
         for (size_t i = 0; (held > kKeepBytes || n > kKeepBlocks) && i < g_blocks.size();) {   // the oldest first
             if (g_blocks[i].device != device) {
                 ++i;
@@ -398,7 +399,9 @@ void give_block(int device, void *ptr, size_t bytes) {
             out.push_back(g_blocks[i]);
             g_blocks.erase(g_blocks.begin() + (long)i);
         }
-    }
+        return HILBERTA_OK;
+    });
+    if (rc != HILBERTA_OK) cudaFree(ptr);   // no room to note it down
     free_blocks(out);
 }
 }  // namespace
@@ -580,7 +583,7 @@ static int make_plan(int frames, int H, int W, int tile, int groups, int layer_o
     p->S = n_text + HW;
     p->P = n_text + p->n_shared;
     p->bound = false;
-    int rc = build_plan(p);
+    const int rc = guarded([&] { return build_plan(p); });
     if (rc != HILBERTA_OK) {
         free_plan(p);
         return rc;
@@ -617,11 +620,20 @@ extern "C" int hilberta_plan_video(int frames, int H, int W, int tile, int layer
 }
 
 extern "C" int hilberta_plan_destroy(hilberta_plan_t *plan) {
-    free_plan(plan);
-    return HILBERTA_OK;
+    return guarded([&] {
+        free_plan(plan);
+        return HILBERTA_OK;
+    });
 }
 
-extern "C" size_t hilberta_trim(void) { return free_kept(); }
+extern "C" size_t hilberta_trim(void) {
+    size_t bytes = 0;
+    guarded([&] {
+        bytes = free_kept();
+        return HILBERTA_OK;
+    });
+    return bytes;
+}
 
 extern "C" int hilberta_plan_export(const hilberta_plan_t *p, int what, void *host_buf, size_t bytes,
                                     size_t *needed) {
@@ -672,8 +684,8 @@ extern "C" int hilberta_plan_export(const hilberta_plan_t *p, int what, void *ho
     return HILBERTA_OK;
 }
 
-extern "C" int hilberta_plan_bind(hilberta_plan_t *p, int batch, int heads, int head_dim, int dtype,
-                                  int64_t stride_b, int64_t stride_h, int64_t stride_s, float scale) {
+static int bind_plan(hilberta_plan_t *p, int batch, int heads, int head_dim, int dtype, int64_t stride_b, int64_t stride_h,
+                     int64_t stride_s, float scale) {
     if (!p || batch < 1 || heads < 1 || head_dim < 1) return HILBERTA_ERR_INVALID;
     if (dtype != HILBERTA_BF16 && dtype != HILBERTA_FP32 && dtype != HILBERTA_FP8_E4M3) return HILBERTA_ERR_INVALID;
     if (dtype == HILBERTA_BF16 && head_dim != 128 && head_dim != 64) return HILBERTA_ERR_UNSUPPORTED;
@@ -723,6 +735,11 @@ extern "C" int hilberta_plan_bind(hilberta_plan_t *p, int batch, int heads, int 
         *at.where = (char *)p->d_bind + at.at + (at.in_scratch ? image.bytes.size() : 0);
     p->bound = true;
     return HILBERTA_OK;
+}
+
+extern "C" int hilberta_plan_bind(hilberta_plan_t *p, int batch, int heads, int head_dim, int dtype,
+                                  int64_t stride_b, int64_t stride_h, int64_t stride_s, float scale) {
+    return guarded([&] { return bind_plan(p, batch, heads, head_dim, dtype, stride_b, stride_h, stride_s, scale); });
 }
 
 // Do two tensors of the layout [batch, heads, S, row] share a byte?  Both use the byte strides sb, sh,
@@ -873,6 +890,12 @@ extern "C" int hilberta_forward_host(const void *q, const void *k, const void *v
     const int n_chunks = p->heads / hc;
     if (!p->s_in) HB_CUDA(cudaStreamCreateWithFlags(&p->s_in, cudaStreamNonBlocking));
     if (!p->s_out) HB_CUDA(cudaStreamCreateWithFlags(&p->s_out, cudaStreamNonBlocking));
+    if (guarded([&] {
+            p->ev_in.reserve((size_t)n_chunks + 1);
+            p->ev_done.reserve((size_t)n_chunks + 1);
+            return HILBERTA_OK;
+        }) != HILBERTA_OK)
+        return HILBERTA_ERR_NOMEM;
     while ((int)p->ev_in.size() < n_chunks + 1) {
         cudaEvent_t e0, e1;
         HB_CUDA(cudaEventCreateWithFlags(&e0, cudaEventDisableTiming));

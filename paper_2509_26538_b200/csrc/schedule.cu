@@ -341,7 +341,8 @@ int add_schedule(BindImage &image, const std::vector<long long> &cost, const std
 static_assert(sizeof(hilberta::WorkItem) == 10 * sizeof(int32_t), "hilberta_check_work_list takes ten ints per item");
 
 extern "C" int hilberta_check_work_list(const int32_t *items, int n_items, int S, int item_rows, int block) {
-    return hilberta::check_work_items(reinterpret_cast<const hilberta::WorkItem *>(items), n_items, S, item_rows, block);
+    return hilberta::guarded(
+        [&] { return hilberta::check_work_items(reinterpret_cast<const hilberta::WorkItem *>(items), n_items, S, item_rows, block); });
 }
 
 static_assert(sizeof(hilberta::WorkUnit) == 3 * sizeof(int32_t), "hilberta_schedule_units writes three ints per unit");
@@ -350,19 +351,21 @@ extern "C" int hilberta_schedule_units(int n_items, const int64_t *cost, const i
                                        int32_t *units, int32_t *cta_begin, int64_t *largest_load) {
     if (n_items < 0 || bh < 1 || n_cta < 1 || (n_items > 0 && !cost) || !units || !cta_begin) return HILBERTA_ERR_INVALID;
     if ((long long)n_items * bh > (1ll << 30)) return HILBERTA_ERR_INVALID;
-    std::vector<long long> c1(cost, cost + n_items), c2;
-    if (cost_two_heads) c2.assign(cost_two_heads, cost_two_heads + n_items);
-    std::vector<hilberta::WorkUnit> u;
-    std::vector<int> cb;
-    const long long m = hilberta::build_schedule(c1, c2, bh, n_cta, hilberta::SplitChoice(), &u, &cb);
-    for (size_t i = 0; i < u.size(); ++i) {
-        units[3 * i] = u[i].item;
-        units[3 * i + 1] = u[i].bh;
-        units[3 * i + 2] = u[i].bh2;
-    }
-    for (int c = 0; c <= n_cta; ++c) cta_begin[c] = c < (int)cb.size() ? cb[c] : (int)u.size();
-    if (largest_load) *largest_load = m;
-    return HILBERTA_OK;
+    return hilberta::guarded([&] {
+        std::vector<long long> c1(cost, cost + n_items), c2;
+        if (cost_two_heads) c2.assign(cost_two_heads, cost_two_heads + n_items);
+        std::vector<hilberta::WorkUnit> u;
+        std::vector<int> cb;
+        const long long m = hilberta::build_schedule(c1, c2, bh, n_cta, hilberta::SplitChoice(), &u, &cb);
+        for (size_t i = 0; i < u.size(); ++i) {
+            units[3 * i] = u[i].item;
+            units[3 * i + 1] = u[i].bh;
+            units[3 * i + 2] = u[i].bh2;
+        }
+        for (int c = 0; c <= n_cta; ++c) cta_begin[c] = c < (int)cb.size() ? cb[c] : (int)u.size();
+        if (largest_load) *largest_load = m;
+        return HILBERTA_OK;
+    });
 }
 
 extern "C" int hilberta_check_shares(const int32_t *items, int n_items, const int32_t *shares, int cluster, int block) {
@@ -379,24 +382,26 @@ extern "C" int hilberta_cut_schedule(const int32_t *items, int n_items, const in
         return HILBERTA_ERR_INVALID;
     for (int k = 0; k < 3; ++k)
         if ((long long)clusters[k] << (k + 1) > sm_count) return HILBERTA_ERR_INVALID;
-    const hilberta::WorkItem *list = reinterpret_cast<const hilberta::WorkItem *>(items);
-    const std::vector<hilberta::WorkItem> its(list, list + n_items);
-    std::vector<long long> c1(cost, cost + n_items), c2((size_t)n_items, 0);
-    if (cost_two_heads) c2.assign(cost_two_heads, cost_two_heads + n_items);
-    hilberta::SplitChoice choice;
-    choice.merge_extra = merge_extra;
-    const int rc = hilberta::choose_split(its, c1, c2, bh, sm_count, clusters, block, choice);
-    if (rc != HILBERTA_OK) return rc;
-    std::vector<hilberta::WorkUnit> u;
-    std::vector<int> cb;
-    const long long m = hilberta::build_schedule(c1, c2, bh, sm_count, choice, &u, &cb);
-    if ((int)u.size() > max_units) return HILBERTA_ERR_BUFFER;
-    memcpy(units, u.data(), sizeof(hilberta::WorkUnit) * u.size());
-    if (!choice.shares.empty()) memcpy(shares, choice.shares.data(), sizeof(hilberta::WorkItem) * choice.shares.size());
-    for (int c = 0; c <= sm_count; ++c) cta_begin[c] = c < (int)cb.size() ? cb[c] : (int)u.size();
-    chosen[0] = choice.cluster;
-    chosen[1] = choice.n_items;
-    chosen[2] = (int)cb.size() - 1;
-    if (largest_load) *largest_load = m;
-    return HILBERTA_OK;
+    return hilberta::guarded([&] {
+        const hilberta::WorkItem *list = reinterpret_cast<const hilberta::WorkItem *>(items);
+        const std::vector<hilberta::WorkItem> its(list, list + n_items);
+        std::vector<long long> c1(cost, cost + n_items), c2((size_t)n_items, 0);
+        if (cost_two_heads) c2.assign(cost_two_heads, cost_two_heads + n_items);
+        hilberta::SplitChoice choice;
+        choice.merge_extra = merge_extra;
+        const int rc = hilberta::choose_split(its, c1, c2, bh, sm_count, clusters, block, choice);
+        if (rc != HILBERTA_OK) return rc;
+        std::vector<hilberta::WorkUnit> u;
+        std::vector<int> cb;
+        const long long m = hilberta::build_schedule(c1, c2, bh, sm_count, choice, &u, &cb);
+        if ((int)u.size() > max_units) return HILBERTA_ERR_BUFFER;
+        memcpy(units, u.data(), sizeof(hilberta::WorkUnit) * u.size());
+        if (!choice.shares.empty()) memcpy(shares, choice.shares.data(), sizeof(hilberta::WorkItem) * choice.shares.size());
+        for (int c = 0; c <= sm_count; ++c) cta_begin[c] = c < (int)cb.size() ? cb[c] : (int)u.size();
+        chosen[0] = choice.cluster;
+        chosen[1] = choice.n_items;
+        chosen[2] = (int)cb.size() - 1;
+        if (largest_load) *largest_load = m;
+        return HILBERTA_OK;
+    });
 }

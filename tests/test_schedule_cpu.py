@@ -1,10 +1,14 @@
 """hilberta_schedule_units: the host-side assignment of (work item, batch * head) units to CTAs.
 
 What any correct schedule must satisfy, and what longest-first list scheduling guarantees."""
+import os
+
 import numpy as np
 import pytest
 
 from paper_2509_26538_b200 import binding as hb
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def _loads(units, begin, cost, two):
@@ -74,3 +78,20 @@ def test_argument_errors():
     assert L.hilberta_schedule_units(1, c.ctypes.data, None, 1, 0, buf.ctypes.data, buf.ctypes.data, None) == hb.ERR_INVALID
     assert L.hilberta_schedule_units(1, None, None, 1, 4, buf.ctypes.data, buf.ctypes.data, None) == hb.ERR_INVALID
     assert L.hilberta_schedule_units(1, c.ctypes.data, None, 1, 4, None, buf.ctypes.data, None) == hb.ERR_INVALID
+
+
+def test_memory_that_runs_out_is_a_status():
+    """2^27 units do not fit into the address space left: an error code, and the process goes on."""
+    import subprocess
+    import sys
+    code = """
+import resource, numpy as np
+from paper_2509_26538_b200 import binding as hb
+L = hb.lib()
+used = int(open("/proc/self/statm").read().split()[0]) * 4096
+resource.setrlimit(resource.RLIMIT_AS, (used + (256 << 20),) * 2)
+c, out = np.ones(1 << 13, dtype=np.int64), np.zeros(1 << 10, dtype=np.int32)
+assert L.hilberta_schedule_units(1 << 13, c.ctypes.data, None, 1 << 14, 4, out.ctypes.data, out.ctypes.data, None) == hb.ERR_NOMEM
+assert L.hilberta_schedule_units(8, c.ctypes.data, None, 2, 4, out.ctypes.data, out.ctypes.data, None) == hb.OK
+"""
+    assert subprocess.run([sys.executable, "-c", code], cwd=ROOT).returncode == 0
