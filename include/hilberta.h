@@ -80,6 +80,7 @@ extern "C" {
 #define HILBERTA_EXPORT_NNZ 6         /* uint64[1]   number of (query, key) pairs the mask keeps */
 #define HILBERTA_EXPORT_INFO 7        /* int32[11]   H, W, tile, offset mod NP, shared_region, n_text, n_shared, T, padded side n, frames, shared_frames */
 #define HILBERTA_EXPORT_LAUNCH_CLOCK 8 /* int32[2]  SM cycles and nanoseconds that the first CTA of the plan's latest tensor-core forward launch was resident: cycles / ns = the SM clock (GHz) that launch ran at; synchronises the device */
+#define HILBERTA_EXPORT_CUTS 9        /* int32[2][3] of the binding, forward and backward: CTAs per cluster (1: no list of keys is cut), work items that are cut, the most cut units in the list of one CTA */
 
 typedef struct hilberta_plan_s hilberta_plan_t;
 

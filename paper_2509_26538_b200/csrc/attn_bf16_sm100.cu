@@ -1207,8 +1207,8 @@ int attn_bf16_prepare(hilberta_plan_t *p, BindImage &image) {
     p->split_cluster = choice.cluster;
     for (const WorkItem &it : choice.shares) items.push_back(it);
     image.add(items, &p->d_work);
-    rc = add_schedule(image, cost, cost_two_heads, p->batch * p->heads, p->sm_count, choice, &p->d_units,
-                            &p->d_cta_begin, &p->n_cta);
+    rc = add_schedule(image, cost, cost_two_heads, p->batch * p->heads, p->sm_count, choice, &p->d_units, &p->d_cta_begin,
+                      &p->n_cta, &p->cuts[0]);
     if (rc != HILBERTA_OK) return rc;
     if (p->chunk_heads < p->heads) {
         rc = add_schedule(image, cost, cost_two_heads, p->batch * p->chunk_heads, p->sm_count, choice,

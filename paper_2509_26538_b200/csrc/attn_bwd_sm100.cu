@@ -748,7 +748,8 @@ int attn_bwd_prepare(hilberta_plan_t *p, BindImage &image) {
     p->bwd_cluster = choice.cluster;
     for (const WorkItem &it : choice.shares) items.push_back(it);
     image.add(items, &p->d_bwd_work);
-    rc = add_schedule(image, cost, {}, bh, p->sm_count, choice, &p->d_bwd_units, &p->d_bwd_cta_begin, &p->n_bwd_cta);
+    rc = add_schedule(image, cost, {}, bh, p->sm_count, choice, &p->d_bwd_units, &p->d_bwd_cta_begin, &p->n_bwd_cta,
+                      &p->cuts[1]);
     if (rc != HILBERTA_OK) return rc;
     image.add_scratch(2 * (size_t)bh * p->S, &p->d_delta);
     return HILBERTA_OK;

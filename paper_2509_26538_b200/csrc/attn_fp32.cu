@@ -362,6 +362,9 @@ int attn_fp32_prepare(hilberta_plan_t *p, BindImage &image) {
         Fp32Work &w = backward ? p->f32_bwd : p->f32_fwd;
         const std::vector<Fp32Row> rows = take_short_rows(p, mine, most, fp32_cost(p->head_dim, backward), w);
         w.n_rows = (int)rows.size();
+        p->cuts[backward][0] = w.n_split > 0 ? w.cluster : 1;
+        p->cuts[backward][1] = w.n_split;
+        p->cuts[backward][2] = w.n_split > 0 ? 1 : 0;
         image.add(mine, &w.items);
         image.add(rows, &w.rows);
     }

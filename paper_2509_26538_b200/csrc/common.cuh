@@ -173,6 +173,7 @@ struct hilberta_plan_s {
     int n_bwd_cta, bwd_cluster;
     float *d_delta;               // [batch * heads * S]
     hilberta::Fp32Work f32_fwd, f32_bwd;   // fp32 bindings
+    int cuts[2][3];               // forward, backward: CTAs per cluster, cut items, the most cut units of a CTA
     int *d_status;  // [4] error word + diagnostics written by bounded waits
     // workspace of hilberta_forward_host
     void *ws;
@@ -247,7 +248,8 @@ int choose_split(const std::vector<WorkItem> &items, const std::vector<long long
 long long build_schedule(const std::vector<long long> &cost, const std::vector<long long> &cost_two_heads, int bh, int sm_count,
                          const SplitChoice &choice, std::vector<WorkUnit> *units, std::vector<int> *cta_begin);
 int add_schedule(BindImage &image, const std::vector<long long> &cost, const std::vector<long long> &cost_two_heads, int bh,
-                 int sm_count, const SplitChoice &choice, WorkUnit **d_units, int **d_cta_begin, int *n_cta_out);
+                 int sm_count, const SplitChoice &choice, WorkUnit **d_units, int **d_cta_begin, int *n_cta_out,
+                 int (*cuts)[3] = nullptr);
 // The forward kernel that the environment variable HILBERTA_FORWARD_KERNEL selects, read once: 'p' (pairs
 // of SMs), 's' (one query tile per CTA) or 0 (the default kernel).
 char forward_kernel_choice();

@@ -663,6 +663,11 @@ extern "C" int hilberta_plan_export(const hilberta_plan_t *p, int what, void *ho
             need = sizeof(int) * tmp.size();
             hsrc = tmp.data();
             break;
+        case HILBERTA_EXPORT_CUTS:
+            if (!p->bound) return HILBERTA_ERR_UNBOUND;
+            need = sizeof(p->cuts);
+            hsrc = p->cuts;
+            break;
         case HILBERTA_EXPORT_LAUNCH_CLOCK:
             need = sizeof(int) * 2;
             dsrc = p->d_status + 32;
@@ -704,6 +709,7 @@ static int bind_plan(hilberta_plan_t *p, int batch, int heads, int head_dim, int
     // the kernels' attributes and the number of clusters that run at once are the plan's device's
     const OnDevice on(p->device);
     p->bound = false;
+    memset(p->cuts, 0, sizeof(p->cuts));
     p->batch = batch;
     p->heads = heads;
     p->head_dim = head_dim;

@@ -325,12 +325,22 @@ int choose_split(const std::vector<WorkItem> &items, const std::vector<long long
 
 // Adds the units grouped by CTA and the n_cta + 1 offsets to the image.
 int add_schedule(BindImage &image, const std::vector<long long> &cost, const std::vector<long long> &cost_two_heads, int bh,
-                 int sm_count, const SplitChoice &choice, WorkUnit **d_units, int **d_cta_begin, int *n_cta_out) {
+                 int sm_count, const SplitChoice &choice, WorkUnit **d_units, int **d_cta_begin, int *n_cta_out, int (*cuts)[3]) {
     if ((long long)cost.size() * bh > (1ll << 30)) return HILBERTA_ERR_INVALID;
     std::vector<WorkUnit> units;
     std::vector<int> cta_begin;
     build_schedule(cost, cost_two_heads, bh, sm_count, choice, &units, &cta_begin);
     *n_cta_out = (int)cta_begin.size() - 1;
+    if (cuts) {
+        (*cuts)[0] = choice.cluster;
+        (*cuts)[1] = choice.n_items;
+        (*cuts)[2] = 0;
+        for (int c = 0; c < *n_cta_out; ++c) {
+            int n = cta_begin[c];
+            while (n < cta_begin[c + 1] && units[n].bh2 == -2) ++n;
+            (*cuts)[2] = std::max((*cuts)[2], n - cta_begin[c]);
+        }
+    }
     image.add(units, d_units);
     image.add(cta_begin, d_cta_begin);
     return HILBERTA_OK;

@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("H,W,tile,o,hs,nt,B,heads,D,fp8", [
-    (16, 32, 256, 100, 2, 20, 1, 1, 128, False),    # few units: everything that can be is cut
+    (16, 32, 256, 100, 2, 20, 1, 1, 128, False),    # few units, but too short to be cut
     (32, 32, 256, 128, 4, 64, 1, 8, 128, False),    # one-tile prefix items beside uncut window items
     (32, 32, 256, 128, 4, 64, 1, 8, 64, False),
     (32, 32, 256, 128, 4, 64, 1, 8, 128, True),

@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("H,W,tile,o,hs,nt,B,heads,D", [
-    (16, 32, 256, 100, 2, 20, 1, 1, 128),     # few units: everything that can be is cut
+    (16, 32, 256, 100, 2, 20, 1, 1, 128),     # few units, but too short to be cut
     (32, 32, 256, 128, 4, 64, 1, 8, 128),     # prefix items cut, window items not
     (32, 32, 256, 128, 4, 64, 1, 8, 64),
     (48, 40, 1024, 77, 8, 226, 1, 2, 128),    # prefix of two full tiles and a rest
