@@ -238,8 +238,9 @@ inline long long items_grid(const Fp32Work &w, long long columns) {
 }
 
 // Several CTAs of these kernels share an SM.  One that is set up while the kernel before it still runs goes
-// where there is room and not where the load is even: four layers of 25 x 34 + 333 tokens, 6 heads of 32 (228
-// CTAs), 318 us overlapping against 262 in turn; 112 CTAs of head dim 128 68 against 62; 80 CTAs 46 against 49.
+// where there is room and not where the load is even.  Four layers, overlapping / in turn (B200, us): 80 CTAs 46 /
+// 49, 96 34.7 / 35.7, 112 of head dim 128 68 / 62, 200 of 128 83 / 86, 264 of 32 305 / 230, 352 98 / 80 and 86 / 75,
+// 384 49.5 / 49.5, 410 1510 / 1243, 608 142 / 145 and 213 / 201: up to the line it gains, beyond it mostly loses.
 inline bool may_overlap(const hilberta_plan_t *p, long long ctas) { return 5 * ctas <= 3 * p->sm_count; }
 
 }  // namespace fp32t

@@ -141,7 +141,7 @@ struct hilberta_plan_s {
     float scale;
     hilberta::WorkItem *d_work;
     int n_work;
-    hilberta::WorkUnit *d_units;  // [n_work * batch * heads], grouped by CTA
+    hilberta::WorkUnit *d_units;  // grouped by CTA: an (item, batch * head), two heads of an item, or a share of one
     int *d_cta_begin;             // [n_cta + 1]
     int n_cta;
     // a second schedule over a slice of chunk_heads heads (all batches), for the host-buffer entry
@@ -165,13 +165,13 @@ struct hilberta_plan_s {
     cudaStream_t s_in, s_out;           // copy streams of hilberta_forward_host (created on first use)
     std::vector<cudaEvent_t> ev_in, ev_done;
     // backward pass: 128-row items over the same key lists, their schedule, and the
-    // per-row scratch delta = rowsum(dO * O) that both backward kernels read
+    // per-row scratch (lse * log2 e, then delta = rowsum(dO * O)) that the backward kernel reads
     hilberta::WorkItem *d_bwd_work;
     int n_bwd_work;
     hilberta::WorkUnit *d_bwd_units;
     int *d_bwd_cta_begin;
     int n_bwd_cta, bwd_cluster;
-    float *d_delta;               // [batch * heads * S]
+    float *d_delta;               // [2 * batch * heads * S]
     hilberta::Fp32Work f32_fwd, f32_bwd;   // fp32 bindings
     int cuts[2][3];               // forward, backward: CTAs per cluster, cut items, the most cut units of a CTA
     int *d_status;  // [4] error word + diagnostics written by bounded waits
@@ -187,8 +187,9 @@ namespace hilberta {
 // they drain (allow_next: once every CTA has said so), and each reads and writes nothing that an earlier
 // kernel could still touch before wait_for_previous has returned -- until then only its plan's tables, which
 // no kernel writes after the plan and its binding are made.  Every kernel launched this way waits (some thread
-// of it at least) and the others are launched plainly, so a kernel's end implies the end of all before it.  Saves the launch latency and the prologue between kernels, 1 ... 2 us each (one fused
-// launch after another, 512^2 and 8 heads: 18.7 -> 16.6 us).  overlap = false: an ordinary launch.
+// of it at least) and the others are launched plainly, so a kernel's end implies the end of all before it.
+// Saves the launch latency and the prologue between kernels, 1 ... 2 us each (one fused launch after another,
+// 512^2 and 8 heads: 18.7 -> 16.6 us).  overlap = false: an ordinary launch.
 __device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -9,8 +9,11 @@ namespace hilberta {
 constexpr int kGatherThreads = 256;
 constexpr int kGatherUnroll = 4;
 // Gathers of up to this many bytes may overlap the kernel before them.  They run for a few microseconds each,
-// and launch latency is part of that (3 heads at 2048^2, three gathers and a forward: 99 -> 92 us); three
-// gathers of 104 MB that run into one another leave the forward after them less of K and V in L2 (607 -> 619 us).
+// and launch latency is part of that; large ones that run into one another leave the forward after them less of
+// K and V in L2.  Three gathers and a forward, overlapping / plain, by the bytes of one gather (B200, us, two runs
+// each): 3.5 MB 43 / 48, 13 MB 90 / 98, 28 MB 143 / 146, 29 MB 130 ... 137 / 138, 43 MB 231 ... 248 / 234, 69 MB
+// 370 ... 398 / 405, 101 MB 1019 ... 1057 / 1023 ... 1050, 104 MB 617 ... 633 / 597 ... 611.  The line lies where every run
+// gains.
 constexpr size_t kOverlapBytes = 32u << 20;
 
 // dst[b, r, :] = src[b, index[r], :]; a row is `vecs` 16-byte vectors.

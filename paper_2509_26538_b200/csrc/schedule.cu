@@ -52,7 +52,7 @@ std::vector<WorkItem> build_work_items(const hilberta_plan_t *p, int item_rows, 
 }
 
 // Every kernel reads the key ranges and query rows of its work items without further checks, so the
-// lists are validated on the host before anything is uploaded: each item's rows and key ranges lie
+// lists are validated on the host before anything is uploaded (the shares of cut items by check_shares): each item's rows and key ranges lie
 // inside [0, S), its key ranges do not overlap, its block count matches them, and the items' query
 // ranges cover [0, S) exactly once.
 int check_work_items(const WorkItem *items, int n, int S, int item_rows, int block) {

@@ -1,6 +1,11 @@
 """How the path spreads over several GPUs: every (batch, head) pair is an
 independent unit with the same plan, so ranks take disjoint contiguous slices
-of the batch*heads axis and never exchange data (no collective in the path)."""
+of the batch*heads axis and never exchange data (no collective in the path).
+
+A slice is bound as a problem of its own, and which long key lists are cut over clusters, hence the order of
+their sums, is chosen from the number of heads bound: the heads of a slice equal the same heads of the whole
+problem up to rounding (one bf16 step at most as measured), not bit for bit.  The same slice gives the same
+bits."""
 from __future__ import annotations
 
 
