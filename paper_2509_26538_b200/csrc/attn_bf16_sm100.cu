@@ -1208,7 +1208,7 @@ int attn_bf16_prepare(hilberta_plan_t *p, BindImage &image) {
     for (const WorkItem &it : choice.shares) items.push_back(it);
     image.add(items, &p->d_work);
     rc = add_schedule(image, cost, cost_two_heads, p->batch * p->heads, p->sm_count, choice, &p->d_units, &p->d_cta_begin,
-                      &p->n_cta, &p->cuts[0]);
+                      &p->n_cta, &p->cuts[0], &p->fwd_load);
     if (rc != HILBERTA_OK) return rc;
     if (p->chunk_heads < p->heads) {
         rc = add_schedule(image, cost, cost_two_heads, p->batch * p->chunk_heads, p->sm_count, choice,
@@ -1289,10 +1289,18 @@ int launch_attn_bf16(const hilberta_plan_t *p, const void *q, const void *k, con
     gprm.gv = v;
     KernelParams<false> pprm;
     static_cast<Params &>(pprm) = prm;
+    // A launch overlaps the one before it where its lists are cut, which leaves CTAs to spare, and where it is short.
+    // Set up while the kernel before it drains, its CTAs go to the SMs in the order in which these fall idle, and long
+    // uncut launches lose more by that than the launch latency is worth.  By largest load, overlapping / plain (B200,
+    // us, launches of 24 ... 96 heads right behind each other): both gathers fused in, load 77 12.6 / 14.2, 103 19.2 / 20.4,
+    // 208 31.0 / 33.5, 229 33.8 / 33.5, 260 36.4 / 34.6, 328 50.6 / 47.9, 439 72.4 / 63.2, 733 130 / 102, 980 120 / 106,
+    // 1860 243 / 194, 2260 294 / 231; behind three gathers, 260 41.2 / 43.5, 280 36.1 / 38.9, 454 64.9 / 68.1, 595 92.0 /
+    // 90.4, 868 90.4 / 85.9, 3325 307 / 288, 256 x 256 tokens in tiles of 64, 16 heads 2416 / 2170.
+    const bool overlap = p->split_cluster > 1 || p->fwd_load <= (in_map ? 210 : 500);
     auto launch = [&](auto split) {
         constexpr bool SPLIT = decltype(split)::value;
         auto go = [&](auto kernel, int smem, const auto &params) {
-            return launch_overlapping(kernel, (unsigned)n_cta, THREADS, (size_t)smem, (unsigned)p->split_cluster, stream, true, mq, mk, mv,
+            return launch_overlapping(kernel, (unsigned)n_cta, THREADS, (size_t)smem, (unsigned)p->split_cluster, stream, overlap, mq, mk, mv,
                                       mo, params);
         };
         if (in_map) {

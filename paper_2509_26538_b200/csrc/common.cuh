@@ -148,6 +148,7 @@ struct hilberta_plan_s {
     // point, which pipelines copies and launches slice by slice; chunk_heads == heads: no slicing
     int chunk_heads;
     int split_cluster;            // CTAs per cluster of the forward launches (1: no clusters, no split units)
+    long long fwd_load;           // largest CTA load of the forward schedule, in twentieths of a key block (1.45 us)
     hilberta::WorkUnit *d_units_chunk;
     int *d_cta_begin_chunk;
     int n_cta_chunk;
@@ -250,7 +251,7 @@ long long build_schedule(const std::vector<long long> &cost, const std::vector<l
                          const SplitChoice &choice, std::vector<WorkUnit> *units, std::vector<int> *cta_begin);
 int add_schedule(BindImage &image, const std::vector<long long> &cost, const std::vector<long long> &cost_two_heads, int bh,
                  int sm_count, const SplitChoice &choice, WorkUnit **d_units, int **d_cta_begin, int *n_cta_out,
-                 int (*cuts)[3] = nullptr);
+                 int (*cuts)[3] = nullptr, long long *largest_load = nullptr);
 // The forward kernel that the environment variable HILBERTA_FORWARD_KERNEL selects, read once: 'p' (pairs
 // of SMs), 's' (one query tile per CTA) or 0 (the default kernel).
 char forward_kernel_choice();

@@ -325,11 +325,13 @@ int choose_split(const std::vector<WorkItem> &items, const std::vector<long long
 
 // Adds the units grouped by CTA and the n_cta + 1 offsets to the image.
 int add_schedule(BindImage &image, const std::vector<long long> &cost, const std::vector<long long> &cost_two_heads, int bh,
-                 int sm_count, const SplitChoice &choice, WorkUnit **d_units, int **d_cta_begin, int *n_cta_out, int (*cuts)[3]) {
+                 int sm_count, const SplitChoice &choice, WorkUnit **d_units, int **d_cta_begin, int *n_cta_out, int (*cuts)[3],
+                 long long *largest_load) {
     if ((long long)cost.size() * bh > (1ll << 30)) return HILBERTA_ERR_INVALID;
     std::vector<WorkUnit> units;
     std::vector<int> cta_begin;
-    build_schedule(cost, cost_two_heads, bh, sm_count, choice, &units, &cta_begin);
+    const long long load = build_schedule(cost, cost_two_heads, bh, sm_count, choice, &units, &cta_begin);
+    if (largest_load) *largest_load = load;
     *n_cta_out = (int)cta_begin.size() - 1;
     if (cuts) {
         (*cuts)[0] = choice.cluster;
