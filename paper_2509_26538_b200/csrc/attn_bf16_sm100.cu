@@ -1295,7 +1295,8 @@ int launch_attn_bf16(const hilberta_plan_t *p, const void *q, const void *k, con
     // us, launches of 24 ... 96 heads right behind each other): both gathers fused in, load 77 12.6 / 14.2, 103 19.2 / 20.4,
     // 208 31.0 / 33.5, 229 33.8 / 33.5, 260 36.4 / 34.6, 328 50.6 / 47.9, 439 72.4 / 63.2, 733 130 / 102, 980 120 / 106,
     // 1860 243 / 194, 2260 294 / 231; behind three gathers, 260 41.2 / 43.5, 280 36.1 / 38.9, 454 64.9 / 68.1, 595 92.0 /
-    // 90.4, 868 90.4 / 85.9, 3325 307 / 288, 256 x 256 tokens in tiles of 64, 16 heads 2416 / 2170.
+    // 90.4, 868 90.4 / 85.9, 3325 307 / 288, 256 x 256 tokens in tiles of 64, 16 heads 2416 / 2170.  (Above the line,
+    // without fused entry gathers: windows of one query tile lose 3 ... 13 %, those of two gain up to 2 or lose up to 5.)
     const bool overlap = p->split_cluster > 1 || p->fwd_load <= (in_map ? 210 : 500);
     auto launch = [&](auto split) {
         constexpr bool SPLIT = decltype(split)::value;
