@@ -33,6 +33,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 #include <functional>
 #include <mutex>
@@ -89,7 +90,10 @@ constexpr float P_SHIFT_FP8 = 4.0f;
 #define HB_POLY_DEG_FP8 2
 #endif
 #ifndef HB_HOST_SLICES
-#define HB_HOST_SLICES 8   // hilberta_forward_host pipelines its copies and launches over about this many slices of heads
+#define HB_HOST_SLICES 8   // hilberta_forward_host pipelines its copies and launches over about this many slices of heads at most
+#endif
+#ifndef HB_HOST_MB
+#define HB_HOST_MB 1.77    // ... and about the square root of the output in units of this many megabytes
 #endif
 #ifndef HB_SPLIT_AT
 #define HB_SPLIT_AT 2    // P goes to the MMA issuer in two parts: 32-key chunks 0..HB_SPLIT_AT, then the rest (2: 96 + 32 keys; measured 0.4-0.6 % faster than 64 + 64)
@@ -1192,13 +1196,19 @@ int attn_bf16_prepare(hilberta_plan_t *p, BindImage &image) {
     int rc = attn_bf16_opt_in(p->device);
     if (rc != HILBERTA_OK) return rc;
 
-    // slice of heads for the pipelined host-buffer path: the largest divisor of `heads` not above heads / HB_HOST_SLICES (rounded up)
+    // Slice of heads for the pipelined host-buffer path.  Every slice costs some 70 us on the way (copies that start and
+    // end, events), and what runs after the last copy in -- a slice's launch and its way out -- shrinks with their
+    // number n, so n goes with the square root of the tensor's size.  Pinned buffers (B200, us), always about eight slices /
+    // this rule: 24 heads of 128, 7 MB a tensor 755 / 600, 28 MB 2107 / 2000, 60 MB 4103 / 3845, 104 MB 6480 / 6460; 8 heads,
+    // 2 MB 365 / 210; 3 heads of 64, 0.1 MB 87 / 57.  Batches want more of them (two and four batch items, 38 and 19 MB: with
+    // n as for one item 2535 / 2585 and 1221 / 1267).  n is the divisor of `heads` nearest in proportion.
+    const double out_mb = 2e-6 * p->batch * p->heads * (double)p->S * p->head_dim;
+    const double want = std::min((double)HB_HOST_SLICES, std::max(1.0, std::sqrt(out_mb * p->batch / HB_HOST_MB)));
     p->chunk_heads = p->heads;
-    for (int d = (p->heads + HB_HOST_SLICES - 1) / HB_HOST_SLICES; d >= 1; --d)
-        if (p->heads % d == 0) {
-            p->chunk_heads = d;
-            break;
-        }
+    for (int n = 2; n <= p->heads; ++n) {
+        const double now = (double)p->heads / p->chunk_heads;
+        if (p->heads % n == 0 && std::max(n / want, want / n) < std::max(now / want, want / now)) p->chunk_heads = p->heads / n;
+    }
     // How the longest items are cut over clusters is decided once, for the whole problem: a slice of heads
     // then gives every row the same sums in the same order.
     SplitChoice choice;

@@ -11,10 +11,9 @@ constexpr int kGatherThreads = 256;
 constexpr int kGatherUnroll = 4;
 // Gathers of up to this many bytes may overlap the kernel before them.  They run for a few microseconds each,
 // and launch latency is part of that; large ones that run into one another leave the forward after them less of
-// K and V in L2.  Three gathers and a forward, overlapping / plain, by the bytes of one gather (B200, us, two runs
-// each): 3.5 MB 43 / 48, 13 MB 90 / 98, 28 MB 143 / 146, 29 MB 130 ... 137 / 138, 43 MB 231 ... 248 / 234, 69 MB
-// 370 ... 398 / 405, 101 MB 1019 ... 1057 / 1023 ... 1050, 104 MB 617 ... 633 / 597 ... 611.  The line lies where every run
-// gains.
+// K and V in L2.  Three gathers and a forward, overlapping / plain, by the bytes of one gather (B200, us): 2 MB 21.6 /
+// 27.8, 5 MB 31.3 / 32.9, 13 MB 89 / 97, 28 MB 158 / 160, 33 MB 182.6 / 182.3, 47 MB 257.8 / 257.2, 52 MB (e4m3) 438 / 441,
+// 52 MB (head dim 64) 421 / 423, 70 MB 374 / 369, 104 MB 625 / 612, 415 MB 4190 / 4120.
 constexpr size_t kOverlapBytes = 32u << 20;
 
 // n / d for n < 2^31 by a multiplication (Granlund and Montgomery, 1994): with s = ceil(log2 d),

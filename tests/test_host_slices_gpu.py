@@ -1,0 +1,32 @@
+"""hilberta_forward_host at sizes from one slice of heads to eight, prime numbers of heads and batches among them, equals
+the fused launch on device buffers bit for bit (a slice's rows are summed in the same order)."""
+import pytest
+import torch
+
+from paper_2509_26538_b200 import binding as hb
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("H,text,batch,heads,dim,dtype", [
+    (8, 0, 1, 1, 64, "bf16"), (16, 5, 1, 7, 128, "bf16"), (16, 0, 3, 6, 64, "bf16"),   # one slice
+    (40, 77, 1, 13, 128, "bf16"),                                                      # 13 heads: one slice or 13
+    (64, 512, 1, 24, 128, "bf16"), (64, 512, 1, 24, 128, "fp8"), (48, 33, 4, 10, 128, "bf16"),
+    (96, 512, 2, 16, 128, "bf16"),                                                     # eight
+])
+def test_host_slices(H, text, batch, heads, dim, dtype):
+    kind = torch.float8_e4m3fn if dtype == "fp8" else torch.bfloat16
+    plan = hb.Plan(H, H, 64, 16, 2, text)
+    g = torch.Generator(device="cuda").manual_seed(H + heads)
+    q, k, v = (torch.randn((batch, heads, plan.S, dim), generator=g, device="cuda").to(kind) for _ in range(3))
+    plan.bind_like(q)
+    want = torch.empty(q.shape, dtype=torch.bfloat16, device="cuda")
+    plan.forward_fused(q, k, v, want)
+    hq, hk, hv = (t.cpu().pin_memory() for t in (q, k, v))
+    out = torch.empty(q.shape, dtype=torch.bfloat16).pin_memory()
+    for _ in range(2):
+        out.fill_(7.0)
+        plan.forward_host(hq, hk, hv, out)
+        assert torch.equal(out, want.cpu())
+    assert plan.status() == 0
+    plan.destroy()
