@@ -22,7 +22,10 @@
 // into weights as soon as A is written and releases A at once, so the scores of the NEXT block
 // are computed while phase 2 (which needs B) and the output MMAs of this block run; phase 2
 // overwrites B in place with P and dS (bf16), each thread inside the 32 columns it has just
-// read.  Per block the tensor pipe sees  A(s+1) | out(s) | B(s+1)  back to back.
+// read.  Per block the tensor pipe sees  A(s+1) | out(s) | B(s+1)  back to back.  Phase 2 lies on the chain
+// B(s) -> phase 2 -> out(s) -> B(s+1), so P and dS are handed over in two halves and the first half's output MMAs run
+// beside the second half's arithmetic (backward call, B200, us, as a whole / in halves: 128 x 128 + 512 tokens, 24 heads
+// 1513 / 1470, 64 x 64 + 512 in tiles of 256 255 / 251, 32 x 32 + 64, 8 heads 26.9 / 26.2).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -59,8 +62,8 @@ enum Bar {
     S_FULL,       // region A written
     A_DONE,       // region A read by every element-wise thread (256 arrivals)
     DP_FULL,      // region B written
-    P_READY,      // P / dS written over region B (256 arrivals)
-    T1_FULL, T1_EMPTY = T1_FULL + NT1,
+    P_READY,      // [part]: P / dS of the first, then of the last 32 columns of each warpgroup written over region B (256 arrivals)
+    T1_FULL = P_READY + 2, T1_EMPTY = T1_FULL + NT1,
     T2_FULL = T1_EMPTY + NT1, T2_EMPTY = T2_FULL + NT2,
     // split units: the whole cluster's partial sums are in shared memory / have been read (4 warps per CTA)
     PART_READY = T2_EMPTY + NT2, PART_READ,
@@ -113,16 +116,19 @@ __device__ __forceinline__ void issue_rt(uint32_t tmem_acc, uint32_t sR, uint32_
 
 // out (+)= A T: A (128 x 128, bf16) from TMEM, the streamed block row-major in smem (N-major
 // operand: 128 rows of K, two 64-column slabs of N).  The bf16 pairs of streamed rows
-// [32 g, 32 g + 32) sit 16 columns wide at column 32 g of region B (+ a_off).
+// [32 g, 32 g + 32) sit 16 columns wide at column 32 g of region B (+ a_off).  In two parts, as the
+// element-wise step hands them over: g = 0, 2, then 1, 3.
 template <int HD>
-__device__ __forceinline__ void issue_at(uint32_t tmem_out, uint32_t tmem_b, uint32_t a_off, uint32_t sT,
+__device__ __forceinline__ void issue_at(uint32_t tmem_out, uint32_t tmem_b, uint32_t a_off, uint32_t sT, int part,
                                          bool accumulate) {
     constexpr uint32_t IDESC = idesc_bf16_f32(BM, HD, 0, 1);
     const uint64_t db = smem_desc_sw128(sT, SLAB_BYTES, 1024);
 #pragma unroll
-    for (int k = 0; k < BK / 16; ++k)
+    for (int i = 0; i < BK / 32; ++i) {
+        const int k = (i >> 1) * 4 + part * 2 + (i & 1);
         mma_ts(tmem_out, tmem_b + (k >> 1) * 32 + a_off + (k & 1) * 8, db + (uint64_t)((k * 2048) >> 4), IDESC,
-               (accumulate || k > 0) ? 1u : 0u);
+               (accumulate || part > 0 || i > 0) ? 1u : 0u);
+    }
 }
 
 // Rows [rank 128 / C, ...) of an item from the C partial sums of the cluster (at sPart in every CTA: COLS fp32
@@ -202,7 +208,7 @@ __device__ __forceinline__ void bwd_cta(const CUtensorMap &tmR1, const CUtensorM
         for (int i = 0; i < NUM_BARS; ++i) {
             uint32_t count = 1;
             if (i == EPI_DONE) count = 128;
-            if (i == A_DONE || i == P_READY) count = 256;
+            if (i == A_DONE || i == P_READY || i == P_READY + 1) count = 256;
             if (SPLIT && (i == PART_READY || i == PART_READ)) count = 4 * cluster_cta_count();
             // DKV: ring 2 also carries the row statistics, copied by the 32 lanes of its producer warp
             if (MODE == MODE_DKV && i >= T2_FULL && i < T2_FULL + NT2) count = 33;
@@ -455,11 +461,15 @@ __device__ __forceinline__ void bwd_cta(const CUtensorMap &tmR1, const CUtensorM
                         ok = wait_or_abort(bar(EPI_DONE), (uc - 1) & 1, abort_flag, prm.status, 0x506);
                         if (!ok) break;
                     }
-                    ok = wait_or_abort(bar(P_READY), e & 1, abort_flag, prm.status, 0x507);
+#pragma unroll
+                    for (int part = 0; part < 2; ++part) {
+                        ok = wait_or_abort(bar(P_READY + part), e & 1, abort_flag, prm.status, 0x507);
+                        if (!ok) break;
+                        tc_fence_after();
+                        issue_at<HD>(tmem + OUT_A, tmem + REG_B, 16, t1(e), part, s > 0);                       // dS  x T1
+                        if (MODE == MODE_DKV) issue_at<HD>(tmem + OUT_B, tmem + REG_B, 0, t2(e), part, s > 0);   // P^T x T2
+                    }
                     if (!ok) break;
-                    tc_fence_after();
-                    issue_at<HD>(tmem + OUT_A, tmem + REG_B, 16, t1(e), s > 0);                       // dS  x T1
-                    if (MODE == MODE_DKV) issue_at<HD>(tmem + OUT_B, tmem + REG_B, 0, t2(e), s > 0);   // P^T x T2
                     mma_commit(bar(T1_EMPTY + e % NT1));
                     if (MODE == MODE_DKV) mma_commit(bar(T2_EMPTY + e % NT2));
                     if (more) {
@@ -596,13 +606,13 @@ __device__ __forceinline__ void bwd_cta(const CUtensorMap &tmR1, const CUtensorM
                             // the 32 columns just read take P (16 columns of bf16 pairs) and dS (16)
                             if (MODE == MODE_DKV) tmem_st16(tB + h2 * 32, pk);
                             tmem_st16(tB + h2 * 32 + 16, dk);
+                            tmem_wait_st();
+                            tc_fence_before();
+                            mbar_arrive(bar(P_READY + h2));
                         }
                     };
                     if (ragged) phase2(std::true_type{});
                     else phase2(std::false_type{});
-                    tmem_wait_st();
-                    tc_fence_before();
-                    mbar_arrive(bar(P_READY));
                 }
             }
         }
