@@ -125,17 +125,36 @@ int check_shares(const WorkItem *items, int n, const WorkItem *shares, int clust
 // B200: 22.7 us uncut, 21.3 in shares of two and 20.8 in shares of four, i.e. 6 and 8 us a merge.
 static long long merge_cost(int cluster) { return cluster == 2 ? 85 : cluster == 4 ? 110 : 135; }
 
-// Greedy assignment to the least loaded of n machines (of equally loaded ones the lowest number).
+// Greedy assignment to the least loaded of n machines (of equally loaded ones the lowest number).  While machines are
+// idle the next of them is the least loaded one, so the heap is only built when all have work, and a schedule of fewer
+// units than machines needs none.  Plan, bind, export and destroy on a B200's host: 44 x 47 tokens, 2 x 12 heads 165 -> 122 us, 64 x 64 + 512, 24 heads 221 -> 184, 128 x 128 + 512 621 -> 580.
 struct LeastLoaded {
     typedef std::pair<long long, int> Load;   // (load, machine)
     std::vector<Load> heap;
+    size_t idle = 0;   // machines from this number on are idle, and the heap is not one yet; heap.size(): it is
     explicit LeastLoaded(const std::vector<long long> &load) {
-        for (size_t i = 0; i < load.size(); ++i) heap.push_back(Load(load[i], (int)i));
+        heap.reserve(load.size());
+        bool any = false;
+        for (size_t i = 0; i < load.size(); ++i) {
+            heap.push_back(Load(load[i], (int)i));
+            any = any || load[i] != 0;
+        }
+        if (any) build();
+    }
+    void build() {
         std::make_heap(heap.begin(), heap.end(), std::greater<Load>());
+        idle = heap.size();
     }
     // adds `cost` to the least loaded machine; returns its new load and its number
     Load add(long long cost) {
         const size_t n = heap.size();
+        if (idle < n && cost > 0) {
+            heap[idle].first = cost;
+            const Load at = heap[idle];
+            if (++idle == n) build();
+            return at;
+        }
+        if (idle < n) build();
         const Load top(heap[0].first + cost, heap[0].second);
         size_t i = 0;
         for (;;) {   // sift the grown top down
