@@ -127,7 +127,8 @@ static long long merge_cost(int cluster) { return cluster == 2 ? 85 : cluster ==
 
 // Greedy assignment to the least loaded of n machines (of equally loaded ones the lowest number).  While machines are
 // idle the next of them is the least loaded one, so the heap is only built when all have work, and a schedule of fewer
-// units than machines needs none.  Plan, bind, export and destroy on a B200's host: 44 x 47 tokens, 2 x 12 heads 165 -> 122 us, 64 x 64 + 512, 24 heads 221 -> 184, 128 x 128 + 512 621 -> 580.
+// units than machines needs none.  Plan, bind, export and destroy on a B200's host: 44 x 47 tokens, 2 x 12 heads
+// 165 -> 122 us, 64 x 64 + 512, 24 heads 221 -> 184, 128 x 128 + 512 621 -> 580.
 struct LeastLoaded {
     typedef std::pair<long long, int> Load;   // (load, machine)
     std::vector<Load> heap;
