@@ -892,7 +892,16 @@ extern "C" int hilberta_forward_host(const void *q, const void *k, const void *v
         p->ws_bytes = got;
     }
     // fp32 bindings have no slice schedule to build: chunk_heads is only set by the bf16 path
-    const int hc = (p->dtype != HILBERTA_FP32 && p->chunk_heads > 0) ? p->chunk_heads : p->heads;
+    int hc = (p->dtype != HILBERTA_FP32 && p->chunk_heads > 0) ? p->chunk_heads : p->heads;
+    // A copy to pageable memory returns when it is done, so the next slice's copies in would not be queued before and
+    // slices only add their fixed costs: 24 heads of 128, 28 MB a tensor, one / four / eight slices 9018 / 9525 / 10195 us
+    // with all four buffers pageable and 3234 / 3677 / 4336 with `out` alone.  Pageable inputs are staged beside the
+    // launches and copies out of earlier slices and keep theirs (8163 / 7330 / 7365).
+    if (hc < p->heads) {
+        cudaPointerAttributes attr;
+        HB_CUDA(cudaPointerGetAttributes(&attr, out));
+        if (attr.type == cudaMemoryTypeUnregistered) hc = p->heads;
+    }
     const int n_chunks = p->heads / hc;
     if (!p->s_in) HB_CUDA(cudaStreamCreateWithFlags(&p->s_in, cudaStreamNonBlocking));
     if (!p->s_out) HB_CUDA(cudaStreamCreateWithFlags(&p->s_out, cudaStreamNonBlocking));

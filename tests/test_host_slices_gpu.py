@@ -30,3 +30,22 @@ def test_host_slices(H, text, batch, heads, dim, dtype):
         assert torch.equal(out, want.cpu())
     assert plan.status() == 0
     plan.destroy()
+
+
+@pytest.mark.parametrize("pinned", [(True, False), (False, True), (False, False)])
+def test_pageable_buffers(pinned):
+    """A copy to pageable memory ends before the next one begins: one slice, while pageable inputs keep theirs."""
+    plan = hb.Plan(64, 64, 64, 16, 2, 512)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    q, k, v = (torch.randn((1, 24, plan.S, 128), generator=g, device="cuda").bfloat16() for _ in range(3))
+    plan.bind_like(q)
+    want = plan.forward_fused(q, k, v, torch.empty_like(q)).cpu()
+    ins = [t.cpu().pin_memory() if pinned[0] else t.cpu() for t in (q, k, v)]
+    out = torch.full(q.shape, 7.0, dtype=torch.bfloat16)
+    out = out.pin_memory() if pinned[1] else out
+    before = hb.launch_count()
+    plan.forward_host(*ins, out)
+    launches = hb.launch_count() - before
+    assert torch.equal(out, want)
+    assert launches == 1 if not pinned[1] else launches > 1
+    plan.destroy()
