@@ -90,7 +90,7 @@ constexpr float P_SHIFT_FP8 = 4.0f;
 #define HB_POLY_DEG_FP8 2
 #endif
 #ifndef HB_HOST_SLICES
-#define HB_HOST_SLICES 8   // hilberta_forward_host pipelines its copies and launches over about this many slices of heads at most
+#define HB_HOST_SLICES 8   // hilberta_forward_host pipelines its copies and launches over this many slices of heads at most
 #endif
 #ifndef HB_HOST_MB
 #define HB_HOST_MB 1.77    // ... and about the square root of the output in units of this many megabytes
@@ -1188,7 +1188,6 @@ int attn_bf16_prepare(hilberta_plan_t *p, BindImage &image) {
         // the second stream's tile loads.
         cost_two_heads.push_back(it.q_rows > BM ? 0 : (long long)it.kv_blocks * 21 + 40);
     }
-    p->n_cta_chunk = 0;
     p->n_work = (int)items.size();
     p->n_cta = 0;
     p->split_cluster = 1;
@@ -1196,19 +1195,19 @@ int attn_bf16_prepare(hilberta_plan_t *p, BindImage &image) {
     int rc = attn_bf16_opt_in(p->device);
     if (rc != HILBERTA_OK) return rc;
 
-    // Slice of heads for the pipelined host-buffer path.  Every slice costs some 70 us on the way (copies that start and
-    // end, events), and what runs after the last copy in -- a slice's launch and its way out -- shrinks with their
-    // number n, so n goes with the square root of the tensor's size.  Pinned buffers (B200, us), always about eight slices /
-    // this rule: 24 heads of 128, 7 MB a tensor 755 / 600, 28 MB 2107 / 2000, 60 MB 4103 / 3845, 104 MB 6480 / 6460; 8 heads,
-    // 2 MB 365 / 210; 3 heads of 64, 0.1 MB 87 / 57.  Batches want more of them (two and four batch items, 38 and 19 MB: with
-    // n as for one item 2535 / 2585 and 1221 / 1267).  n is the divisor of `heads` nearest in proportion.
+    // Slices of heads for the pipelined host-buffer path, of sizes that differ by one head at most, so that any number of
+    // heads goes into any number n of slices.  What runs after the last copy in, a slice's launch and its way out, shrinks
+    // with n, and a slice costs 10 ... 50 us of copies that start and end, so n goes with the square root of the output's
+    // size.  HB_HOST_MB is from a sweep over n = 1 ... 12 of 31 problems with pinned buffers (B200; outputs of 0.1 ... 104 MB,
+    // one to four batch items, bf16 and e4m3): 1.2 ... 2.2 cost 1.5 ... 1.8 % on average over the best n of each problem, and
+    // this value 1.6.  One / eight slices / this rule (us): 8 heads of 128, 2 MB 214 / 288 / 214; 24 heads, 28 MB 2206 /
+    // 2137 / 1972, 60 MB 4605 / 4138 / 3973, 104 MB 8038 / 6472 / 6472; 13 heads, 15 MB 1212 / 1205 / 1096; 61 heads, 72 MB 5501 /
+    // 4714 / 4659; e4m3, 24 heads, 28 MB 1404 / 1291 / 1225, 104 MB 5075 / 4111 / 4111 (where five would take 3812).  Batches:
+    // 2 x 12 heads, 27 MB 2109 / 1890 / 1817, 4 x 10, 24 MB 1830 / 1766 / 1752, 4 x 24, 58 MB 4444 / 3959 / 3959; without the
+    // factor `batch` they cost the same on average, the first 1929, the others 1686 and 3860.
     const double out_mb = 2e-6 * p->batch * p->heads * (double)p->S * p->head_dim;
     const double want = std::min((double)HB_HOST_SLICES, std::max(1.0, std::sqrt(out_mb * p->batch / HB_HOST_MB)));
-    p->chunk_heads = p->heads;
-    for (int n = 2; n <= p->heads; ++n) {
-        const double now = (double)p->heads / p->chunk_heads;
-        if (p->heads % n == 0 && std::max(n / want, want / n) < std::max(now / want, want / now)) p->chunk_heads = p->heads / n;
-    }
+    p->n_slices = std::min(p->heads, (int)std::lround(want));
     // How the longest items are cut over clusters is decided once, for the whole problem: a slice of heads
     // then gives every row the same sums in the same order.
     SplitChoice choice;
@@ -1220,9 +1219,10 @@ int attn_bf16_prepare(hilberta_plan_t *p, BindImage &image) {
     rc = add_schedule(image, cost, cost_two_heads, p->batch * p->heads, p->sm_count, choice, &p->d_units, &p->d_cta_begin,
                       &p->n_cta, &p->cuts[0], &p->fwd_load);
     if (rc != HILBERTA_OK) return rc;
-    if (p->chunk_heads < p->heads) {
-        rc = add_schedule(image, cost, cost_two_heads, p->batch * p->chunk_heads, p->sm_count, choice,
-                                &p->d_units_chunk, &p->d_cta_begin_chunk, &p->n_cta_chunk);
+    for (int more = 0; more < 2 && p->n_slices > 1; ++more) {
+        if (more && p->heads % p->n_slices == 0) break;
+        rc = add_schedule(image, cost, cost_two_heads, p->batch * (p->heads / p->n_slices + more), p->sm_count, choice,
+                          &p->d_units_slice[more], &p->d_cta_begin_slice[more], &p->n_cta_slice[more]);
         if (rc != HILBERTA_OK) return rc;
     }
     // the alternative kernels' tables: only where they are selected
@@ -1240,33 +1240,35 @@ char forward_kernel_choice() {
 }
 
 int launch_attn_bf16(const hilberta_plan_t *p, const void *q, const void *k, const void *v, void *out,
-                     float *lse, const int *out_map, const int *in_map, cudaStream_t stream, int chunk) {
+                     float *lse, const int *out_map, const int *in_map, cudaStream_t stream, int slice) {
     if (p->n_work == 0) return HILBERTA_OK;
     // bf16 with head dim 128 and inputs in physical order can also run on pairs of SMs
     // (attn_bf16_pair_sm100.cu) or with one query tile per CTA (attn_bf16_solo_sm100.cu).  Those kernels
     // are correct but measure slower than this one, so they are opt-in: the environment variable
     // HILBERTA_FORWARD_KERNEL=pair or =solo selects them (read once, by the first bind).
-    if (forward_kernel_choice() == 'p' && !in_map && chunk < 0 && p->n_pair > 0)
+    if (forward_kernel_choice() == 'p' && !in_map && slice < 0 && p->n_pair > 0)
         return launch_attn_bf16_pair(p, q, k, v, out, lse, out_map, stream);
-    if (forward_kernel_choice() == 's' && !in_map && chunk < 0 && p->n_solo > 0)
+    if (forward_kernel_choice() == 's' && !in_map && slice < 0 && p->n_solo > 0)
         return launch_attn_bf16_solo(p, q, k, v, out, lse, out_map, stream);
     int heads = p->heads, n_cta = p->n_cta;
     const WorkUnit *units = p->d_units;
     const int *cta_begin = p->d_cta_begin;
     const bool fp8 = p->dtype == HILBERTA_FP8_E4M3;
-    if (chunk >= 0 && p->chunk_heads < p->heads) {
-        // a slice of heads: same strides, shifted base pointers, the slice's own schedule
-        if (lse) return HILBERTA_ERR_INVALID;
-        heads = p->chunk_heads;
-        const long long off = (long long)chunk * heads * p->stride_h;   // elements
+    if (slice >= 0) {
+        // a slice of heads: same strides, shifted base pointers, a schedule of its own
+        if (lse || slice >= p->n_slices || p->n_slices < 2) return HILBERTA_ERR_INVALID;
+        const int first = p->slice_begin(slice, p->n_slices);
+        heads = p->slice_begin(slice + 1, p->n_slices) - first;
+        const long long off = first * p->stride_h;   // elements
         const long long esz_in = fp8 ? 1 : 2;
         q = (const char *)q + off * esz_in;
         k = (const char *)k + off * esz_in;
         v = (const char *)v + off * esz_in;
         out = (__nv_bfloat16 *)out + off;
-        units = p->d_units_chunk;
-        cta_begin = p->d_cta_begin_chunk;
-        n_cta = p->n_cta_chunk;
+        const int more = heads > p->heads / p->n_slices;
+        units = p->d_units_slice[more];
+        cta_begin = p->d_cta_begin_slice[more];
+        n_cta = p->n_cta_slice[more];
     }
     CUtensorMap mq, mk, mv;
     int rc;

@@ -409,10 +409,10 @@ static int launch_fwd(const hilberta_plan_t *p, const float *q, const float *k, 
 }
 
 int launch_attn_fp32(const hilberta_plan_t *p, const void *q, const void *k, const void *v, void *out,
-                     float *lse, const int *out_map, const int *in_map, cudaStream_t stream, int chunk) {
+                     float *lse, const int *out_map, const int *in_map, cudaStream_t stream, int slice) {
     const uintptr_t bits = (uintptr_t)q | (uintptr_t)k | (uintptr_t)v | (uintptr_t)out;
     if ((bits & 15) || ((p->stride_b | p->stride_h | p->stride_s) & 3)) return HILBERTA_ERR_INVALID;
-    if (chunk >= 0) return HILBERTA_ERR_INVALID;   // fp32 bindings have no slices of heads
+    if (slice >= 0) return HILBERTA_ERR_INVALID;   // fp32 bindings have no slices of heads
     switch (p->head_dim) {
         case 32: return launch_fwd<32>(p, (const float *)q, (const float *)k, (const float *)v, (float *)out, lse, out_map, in_map, stream);
         case 64: return launch_fwd<64>(p, (const float *)q, (const float *)k, (const float *)v, (float *)out, lse, out_map, in_map, stream);

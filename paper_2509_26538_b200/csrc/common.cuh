@@ -144,14 +144,16 @@ struct hilberta_plan_s {
     hilberta::WorkUnit *d_units;  // grouped by CTA: an (item, batch * head), two heads of an item, or a share of one
     int *d_cta_begin;             // [n_cta + 1]
     int n_cta;
-    // a second schedule over a slice of chunk_heads heads (all batches), for the host-buffer entry
-    // point, which pipelines copies and launches slice by slice; chunk_heads == heads: no slicing
-    int chunk_heads;
+    // The host-buffer entry point pipelines copies and launches over n_slices slices of heads (of all batch items): the
+    // first heads % n_slices of them have a head more than the others, and a schedule of their own.
+    int n_slices;
+    // first head of slice c of n
+    int slice_begin(int c, int n) const { return c * (heads / n) + (c < heads % n ? c : heads % n); }
     int split_cluster;            // CTAs per cluster of the forward launches (1: no clusters, no split units)
     long long fwd_load;           // largest CTA load of the forward schedule, in twentieths of a key block (1.45 us)
-    hilberta::WorkUnit *d_units_chunk;
-    int *d_cta_begin_chunk;
-    int n_cta_chunk;
+    hilberta::WorkUnit *d_units_slice[2];   // [1]: of the slices with a head more
+    int *d_cta_begin_slice[2];
+    int n_cta_slice[2];
     // the pair kernel's work list and schedule (bf16, head dim 128): items of 256 rows, one per
     // pair of SMs; n_pair == 0: the shape is served by the single-CTA kernel
     hilberta::WorkItem *d_work_pair;
@@ -219,12 +221,12 @@ cudaError_t launch_overlapping(void (*kernel)(Params...), dim3 grid, unsigned bl
 // (natural log), indexed like `out` rows.
 // in_map: nullptr = q, k, v are in physical order; else they are in ORIGINAL order and physical
 // row p is read from row in_map[p] (the entry gather fused into the loads).
-// chunk: -1 = the whole bound problem; c >= 0 = heads [c * chunk_heads, (c + 1) * chunk_heads) of
-// every batch item only (lse must be null then).
+// slice: -1 = the whole bound problem; c >= 0 = slice c of n_slices > 1, its heads
+// of every batch item only (lse must be null then).
 int launch_attn_fp32(const hilberta_plan_t *p, const void *q, const void *k, const void *v, void *out,
-                     float *lse, const int *out_map, const int *in_map, cudaStream_t stream, int chunk = -1);
+                     float *lse, const int *out_map, const int *in_map, cudaStream_t stream, int slice = -1);
 int launch_attn_bf16(const hilberta_plan_t *p, const void *q, const void *k, const void *v, void *out,
-                     float *lse, const int *out_map, const int *in_map, cudaStream_t stream, int chunk = -1);
+                     float *lse, const int *out_map, const int *in_map, cudaStream_t stream, int slice = -1);
 // schedule.cu: work lists (runs of item_rows rows with their up to three key ranges, counted in
 // blocks of `block` rows) and the static longest-first assignment of (item, batch * head) units to CTAs
 std::vector<WorkItem> build_work_items(const hilberta_plan_t *p, int item_rows, int block);

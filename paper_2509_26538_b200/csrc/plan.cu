@@ -710,6 +710,7 @@ static int bind_plan(hilberta_plan_t *p, int batch, int heads, int head_dim, int
     const OnDevice on(p->device);
     p->bound = false;
     memset(p->cuts, 0, sizeof(p->cuts));
+    p->n_slices = 1;   // fp32 bindings have no others
     p->batch = batch;
     p->heads = heads;
     p->head_dim = head_dim;
@@ -796,7 +797,7 @@ bool bound_tensors_overlap(const hilberta_plan_t *p, const void *out, size_t esz
 
 static int forward_impl(const void *q, const void *k, const void *v, void *out, float *lse,
                         const hilberta_plan_t *p, const int *out_map, const int *in_map, void *stream,
-                        int chunk = -1) {
+                        int slice = -1) {
     if (!p || !q || !k || !v || !out) return HILBERTA_ERR_INVALID;
     if (!p->bound) return HILBERTA_ERR_UNBOUND;
     {
@@ -811,10 +812,10 @@ static int forward_impl(const void *q, const void *k, const void *v, void *out, 
     HB_CUDA(cudaGetDevice(&dev));
     if (dev != p->device) return HILBERTA_ERR_INVALID;  // the plan's tables live on another device
     cudaStream_t st = (cudaStream_t)stream;
-    if (p->dtype == HILBERTA_FP32) return launch_attn_fp32(p, q, k, v, out, lse, out_map, in_map, st, chunk);
+    if (p->dtype == HILBERTA_FP32) return launch_attn_fp32(p, q, k, v, out, lse, out_map, in_map, st, slice);
     const uintptr_t bits = (uintptr_t)q | (uintptr_t)k | (uintptr_t)v | (uintptr_t)out;
     if (bits & 15) return HILBERTA_ERR_INVALID;
-    return launch_attn_bf16(p, q, k, v, out, lse, out_map, in_map, st, chunk);
+    return launch_attn_bf16(p, q, k, v, out, lse, out_map, in_map, st, slice);
 }
 
 extern "C" int hilberta_forward(const void *q, const void *k, const void *v, void *out,
@@ -891,27 +892,25 @@ extern "C" int hilberta_forward_host(const void *q, const void *k, const void *v
         HB_CUDA(take_block(p->device, &p->ws, &got));
         p->ws_bytes = got;
     }
-    // fp32 bindings have no slice schedule to build: chunk_heads is only set by the bf16 path
-    int hc = (p->dtype != HILBERTA_FP32 && p->chunk_heads > 0) ? p->chunk_heads : p->heads;
     // A copy to pageable memory returns when it is done, so the next slice's copies in would not be queued before and
     // slices only add their fixed costs: 24 heads of 128, 28 MB a tensor, one / four / eight slices 9018 / 9525 / 10195 us
     // with all four buffers pageable and 3234 / 3677 / 4336 with `out` alone.  Pageable inputs are staged beside the
     // launches and copies out of earlier slices and keep theirs (8163 / 7330 / 7365).
-    if (hc < p->heads) {
+    int n = p->n_slices;
+    if (n > 1) {
         cudaPointerAttributes attr;
         HB_CUDA(cudaPointerGetAttributes(&attr, out));
-        if (attr.type == cudaMemoryTypeUnregistered) hc = p->heads;
+        if (attr.type == cudaMemoryTypeUnregistered) n = 1;
     }
-    const int n_chunks = p->heads / hc;
     if (!p->s_in) HB_CUDA(cudaStreamCreateWithFlags(&p->s_in, cudaStreamNonBlocking));
     if (!p->s_out) HB_CUDA(cudaStreamCreateWithFlags(&p->s_out, cudaStreamNonBlocking));
     if (guarded([&] {
-            p->ev_in.reserve((size_t)n_chunks + 1);
-            p->ev_done.reserve((size_t)n_chunks + 1);
+            p->ev_in.reserve((size_t)n + 1);
+            p->ev_done.reserve((size_t)n + 1);
             return HILBERTA_OK;
         }) != HILBERTA_OK)
         return HILBERTA_ERR_NOMEM;
-    while ((int)p->ev_in.size() < n_chunks + 1) {
+    while ((int)p->ev_in.size() < n + 1) {
         cudaEvent_t e0, e1;
         HB_CUDA(cudaEventCreateWithFlags(&e0, cudaEventDisableTiming));
         HB_CUDA(cudaEventCreateWithFlags(&e1, cudaEventDisableTiming));
@@ -923,27 +922,26 @@ extern "C" int hilberta_forward_host(const void *q, const void *k, const void *v
     void *in[3] = {ws, ws + slot, ws + 2 * slot};
     char *out_dev = ws + 3 * slot;
     const void *host_in[3] = {q, k, v};
-    // a slice of hc heads of every batch item: `batch` rows of row_bytes, one tensor of heads apart
-    const size_t row_bytes = (size_t)hc * p->S * p->head_dim * esz;
-    const size_t pitch = (size_t)p->heads * p->S * p->head_dim * esz;
-    const size_t row_bytes_out = row_bytes / esz * esz_out, pitch_out = pitch / esz * esz_out;
+    // a slice of the heads of every batch item: `batch` rows of some heads' bytes, one tensor of heads apart
+    const size_t head = (size_t)p->S * p->head_dim;
+    const size_t pitch = p->heads * head * esz, pitch_out = p->heads * head * esz_out;
     // work already queued on the caller's stream comes first
-    HB_CUDA(cudaEventRecord(p->ev_in[n_chunks], st));
-    HB_CUDA(cudaStreamWaitEvent(p->s_in, p->ev_in[n_chunks], 0));
-    for (int c = 0; c < n_chunks; ++c) {
-        const size_t off = (size_t)c * row_bytes;
+    HB_CUDA(cudaEventRecord(p->ev_in[n], st));
+    HB_CUDA(cudaStreamWaitEvent(p->s_in, p->ev_in[n], 0));
+    for (int c = 0; c < n; ++c) {
+        const size_t first = (size_t)p->slice_begin(c, n) * head, elems = (size_t)p->slice_begin(c + 1, n) * head - first;
+        const size_t off = first * esz, off_out = first * esz_out;
         for (int i = 0; i < 3; ++i)
-            HB_CUDA(cudaMemcpy2DAsync((char *)in[i] + off, pitch, (const char *)host_in[i] + off, pitch, row_bytes,
+            HB_CUDA(cudaMemcpy2DAsync((char *)in[i] + off, pitch, (const char *)host_in[i] + off, pitch, elems * esz,
                                       p->batch, cudaMemcpyHostToDevice, p->s_in));
         HB_CUDA(cudaEventRecord(p->ev_in[c], p->s_in));
         HB_CUDA(cudaStreamWaitEvent(st, p->ev_in[c], 0));
         const int rc = forward_impl(in[0], in[1], in[2], out_dev, nullptr, p, p->d_phys2orig, p->d_phys2orig, st,
-                                    n_chunks > 1 ? c : -1);
+                                    n > 1 ? c : -1);
         if (rc != HILBERTA_OK) return rc;
         HB_CUDA(cudaEventRecord(p->ev_done[c], st));
         HB_CUDA(cudaStreamWaitEvent(p->s_out, p->ev_done[c], 0));
-        const size_t off_out = (size_t)c * row_bytes_out;
-        HB_CUDA(cudaMemcpy2DAsync((char *)out + off_out, pitch_out, out_dev + off_out, pitch_out, row_bytes_out, p->batch,
+        HB_CUDA(cudaMemcpy2DAsync((char *)out + off_out, pitch_out, out_dev + off_out, pitch_out, elems * esz_out, p->batch,
                                   cudaMemcpyDeviceToHost, p->s_out));
     }
     HB_CUDA(cudaStreamSynchronize(p->s_out));

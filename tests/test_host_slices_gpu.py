@@ -1,5 +1,5 @@
-"""hilberta_forward_host at sizes from one slice of heads to eight, prime numbers of heads and batches among them, equals
-the fused launch on device buffers bit for bit (a slice's rows are summed in the same order)."""
+"""hilberta_forward_host at sizes from one slice of heads to eight (a launch each), prime numbers of heads and batches among
+them, equals the fused launch on device buffers bit for bit (a slice's rows are summed in the same order)."""
 import pytest
 import torch
 
@@ -8,13 +8,14 @@ from paper_2509_26538_b200 import binding as hb
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("H,text,batch,heads,dim,dtype", [
-    (8, 0, 1, 1, 64, "bf16"), (16, 5, 1, 7, 128, "bf16"), (16, 0, 3, 6, 64, "bf16"),   # one slice
-    (40, 77, 1, 13, 128, "bf16"),                                                      # 13 heads: one slice or 13
-    (64, 512, 1, 24, 128, "bf16"), (64, 512, 1, 24, 128, "fp8"), (48, 33, 4, 10, 128, "bf16"),
-    (96, 512, 2, 16, 128, "bf16"),                                                     # eight
+@pytest.mark.parametrize("H,text,batch,heads,dim,dtype,slices", [
+    (8, 0, 1, 1, 64, "bf16", 1), (16, 5, 1, 7, 128, "bf16", 1), (16, 0, 3, 6, 64, "bf16", 1),
+    (40, 77, 1, 13, 128, "bf16", 2),                                                   # 7 and 6 heads
+    (64, 512, 1, 24, 128, "bf16", 4), (64, 512, 1, 24, 128, "fp8", 4), (48, 33, 4, 10, 128, "bf16", 7),
+    (64, 333, 2, 7, 128, "fp8", 4), (88, 256, 1, 31, 128, "bf16", 6), (64, 512, 1, 67, 64, "bf16", 5),
+    (96, 512, 2, 16, 128, "bf16", 8), (128, 512, 1, 23, 128, "bf16", 7),
 ])
-def test_host_slices(H, text, batch, heads, dim, dtype):
+def test_host_slices(H, text, batch, heads, dim, dtype, slices):
     kind = torch.float8_e4m3fn if dtype == "fp8" else torch.bfloat16
     plan = hb.Plan(H, H, 64, 16, 2, text)
     g = torch.Generator(device="cuda").manual_seed(H + heads)
@@ -26,7 +27,9 @@ def test_host_slices(H, text, batch, heads, dim, dtype):
     out = torch.empty(q.shape, dtype=torch.bfloat16).pin_memory()
     for _ in range(2):
         out.fill_(7.0)
+        before = hb.launch_count()
         plan.forward_host(hq, hk, hv, out)
+        assert hb.launch_count() - before == slices
         assert torch.equal(out, want.cpu())
     assert plan.status() == 0
     plan.destroy()
