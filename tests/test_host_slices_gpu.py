@@ -8,17 +8,9 @@ from paper_2509_26538_b200 import binding as hb
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("H,text,batch,heads,dim,dtype,slices", [
-    (8, 0, 1, 1, 64, "bf16", 1), (16, 5, 1, 7, 128, "bf16", 1), (16, 0, 3, 6, 64, "bf16", 1),
-    (40, 77, 1, 13, 128, "bf16", 2),                                                   # 7 and 6 heads
-    (64, 512, 1, 24, 128, "bf16", 4), (64, 512, 1, 24, 128, "fp8", 4), (48, 33, 4, 10, 128, "bf16", 7),
-    (64, 333, 2, 7, 128, "fp8", 4), (88, 256, 1, 31, 128, "bf16", 6), (64, 512, 1, 67, 64, "bf16", 5),
-    (96, 512, 2, 16, 128, "bf16", 8), (128, 512, 1, 23, 128, "bf16", 7),
-])
-def test_host_slices(H, text, batch, heads, dim, dtype, slices):
+def _check(plan, batch, heads, dim, dtype, slices):
     kind = torch.float8_e4m3fn if dtype == "fp8" else torch.bfloat16
-    plan = hb.Plan(H, H, 64, 16, 2, text)
-    g = torch.Generator(device="cuda").manual_seed(H + heads)
+    g = torch.Generator(device="cuda").manual_seed(plan.S + heads)
     q, k, v = (torch.randn((batch, heads, plan.S, dim), generator=g, device="cuda").to(kind) for _ in range(3))
     plan.bind_like(q)
     want = torch.empty(q.shape, dtype=torch.bfloat16, device="cuda")
@@ -32,6 +24,32 @@ def test_host_slices(H, text, batch, heads, dim, dtype, slices):
         assert hb.launch_count() - before == slices
         assert torch.equal(out, want.cpu())
     assert plan.status() == 0
+
+
+@pytest.mark.parametrize("H,text,batch,heads,dim,dtype,slices", [
+    (8, 0, 1, 1, 64, "bf16", 1), (16, 5, 1, 7, 128, "bf16", 1), (16, 0, 3, 6, 64, "bf16", 1),
+    (40, 77, 1, 13, 128, "bf16", 2),                                                   # 7 and 6 heads
+    (64, 512, 1, 24, 128, "bf16", 4), (64, 512, 1, 24, 128, "fp8", 4), (48, 33, 4, 10, 128, "bf16", 7),
+    (64, 333, 2, 7, 128, "fp8", 4), (88, 256, 1, 31, 128, "bf16", 6), (64, 512, 1, 67, 64, "bf16", 5),
+    (96, 512, 2, 16, 128, "bf16", 8), (128, 512, 1, 23, 128, "bf16", 7),
+])
+def test_host_slices(H, text, batch, heads, dim, dtype, slices):
+    plan = hb.Plan(H, H, 64, 16, 2, text)
+    _check(plan, batch, heads, dim, dtype, slices)
+    plan.destroy()
+
+
+@pytest.mark.parametrize("H,tile,shared,text,batch,heads,dim,dtype,slices", [
+    (128, 1024, 16, 512, 1, 3, 128, "bf16", 3), (128, 1024, 16, 512, 1, 3, 128, "fp8", 3),
+    (128, 1024, 16, 512, 1, 5, 64, "bf16", 2),                                         # 3 and 2 heads
+    (64, 512, 8, 512, 2, 3, 64, "bf16", 2), (64, 512, 8, 512, 3, 2, 128, "bf16", 2),
+])
+def test_host_slices_of_cut_lists(H, tile, shared, text, batch, heads, dim, dtype, slices):
+    """Key lists cut over clusters: the shares are those of the whole problem, the schedules the slices' own."""
+    plan = hb.Plan(H, H, tile, 0, shared, text)
+    _check(plan, batch, heads, dim, dtype, slices)
+    cluster, items, _ = plan.export(hb.EXPORT_CUTS)[0]
+    assert cluster > 1 and items > 0
     plan.destroy()
 
 
