@@ -1195,19 +1195,27 @@ int attn_bf16_prepare(hilberta_plan_t *p, BindImage &image) {
     int rc = attn_bf16_opt_in(p->device);
     if (rc != HILBERTA_OK) return rc;
 
-    // Slices of heads for the pipelined host-buffer path, of sizes that differ by one head at most, so that any number of
-    // heads goes into any number n of slices.  What runs after the last copy in, a slice's launch and its way out, shrinks
-    // with n, and a slice costs 10 ... 50 us of copies that start and end, so n goes with the square root of the output's
-    // size.  HB_HOST_MB is from a sweep over n = 1 ... 12 of 31 problems with pinned buffers (B200; outputs of 0.1 ... 104 MB,
-    // one to four batch items, bf16 and e4m3): 1.2 ... 2.2 cost 1.5 ... 1.8 % on average over the best n of each problem, and
-    // this value 1.6.  One / eight slices / this rule (us): 8 heads of 128, 2 MB 214 / 288 / 214; 24 heads, 28 MB 2206 /
-    // 2137 / 1972, 60 MB 4605 / 4138 / 3973, 104 MB 8038 / 6472 / 6472; 13 heads, 15 MB 1212 / 1205 / 1096; 61 heads, 72 MB 5501 /
-    // 4714 / 4659; e4m3, 24 heads, 28 MB 1404 / 1291 / 1225, 104 MB 5075 / 4111 / 4111 (where five would take 3812).  Batches:
-    // 2 x 12 heads, 27 MB 2109 / 1890 / 1817, 4 x 10, 24 MB 1830 / 1766 / 1752, 4 x 24, 58 MB 4444 / 3959 / 3959; without the
-    // factor `batch` they cost the same on average, the first 1929, the others 1686 and 3860.
+    // Slices of heads for the pipelined host-buffer path.  What runs after the last copy in, a slice's launch and its way
+    // out, shrinks with their number n, and a slice costs 10 ... 50 us of copies that start and end, so n goes with the
+    // square root of the output's size.  HB_HOST_MB is from a sweep over n = 1 ... 8 of 248 problems with pinned buffers (B200;
+    // outputs of 2 ... 75 MB, 2 ... 24 heads, one to four batch items, bf16 and e4m3): 1.2 ... 2.7 cost 3.1 ... 1.9 % on average
+    // over the best n of each problem and this value 2.5; without the factor `batch` 1.3, but some calls 6 % more.
+    // One / eight slices / this rule (us): 8 heads of 128, 2 MB 214 / 288 / 214; 24 heads, 28 MB 2206 / 2137 / 1972, 60 MB
+    // 4605 / 4138 / 3973, 104 MB 8038 / 6472 / 6472; e4m3, 24 heads, 28 MB 1404 / 1291 / 1225, 104 MB 5075 / 4111 / 4111 (where
+    // five would take 3812).  Batches: 2 x 12 heads, 27 MB 2109 / 1890 / 1817, 4 x 10, 24 MB 1830 / 1766 / 1727, 4 x 24, 58 MB
+    // 4444 / 3959 / 3959 (without `batch` 1908, 1679 and 3860).
+    // A divisor of `heads` within a factor of 1.5 is taken where there is one: one schedule then serves all slices, and the
+    // nearest n of any kind is no faster on average (2.2 % over the best) and up to 6 % slower.  Elsewhere slices differ by a
+    // head: 13 heads, 15 MB 1212 / 1205 / 1096, 31 heads, 64 MB 4829 / 4190 / 4040, 61 heads, 72 MB 5501 / 4714 / 4659.
     const double out_mb = 2e-6 * p->batch * p->heads * (double)p->S * p->head_dim;
     const double want = std::min((double)HB_HOST_SLICES, std::max(1.0, std::sqrt(out_mb * p->batch / HB_HOST_MB)));
     p->n_slices = std::min(p->heads, (int)std::lround(want));
+    double off = 1.5;
+    for (int n = 1; n <= std::min(p->heads, HB_HOST_SLICES); ++n)
+        if (p->heads % n == 0 && std::max(n / want, want / n) < off) {
+            off = std::max(n / want, want / n);
+            p->n_slices = n;
+        }
     // How the longest items are cut over clusters is decided once, for the whole problem: a slice of heads
     // then gives every row the same sums in the same order.
     SplitChoice choice;

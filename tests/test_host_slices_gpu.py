@@ -29,9 +29,10 @@ def _check(plan, batch, heads, dim, dtype, slices):
 @pytest.mark.parametrize("H,text,batch,heads,dim,dtype,slices", [
     (8, 0, 1, 1, 64, "bf16", 1), (16, 5, 1, 7, 128, "bf16", 1), (16, 0, 3, 6, 64, "bf16", 1),
     (40, 77, 1, 13, 128, "bf16", 2),                                                   # 7 and 6 heads
-    (64, 512, 1, 24, 128, "bf16", 4), (64, 512, 1, 24, 128, "fp8", 4), (48, 33, 4, 10, 128, "bf16", 7),
+    (64, 512, 1, 24, 128, "bf16", 4), (64, 512, 1, 24, 128, "fp8", 4), (48, 33, 4, 10, 128, "bf16", 5),
     (64, 333, 2, 7, 128, "fp8", 4), (88, 256, 1, 31, 128, "bf16", 6), (64, 512, 1, 67, 64, "bf16", 5),
-    (96, 512, 2, 16, 128, "bf16", 8), (128, 512, 1, 23, 128, "bf16", 7),
+    (96, 512, 2, 16, 128, "bf16", 8), (128, 512, 1, 23, 128, "bf16", 7), (96, 512, 1, 10, 128, "bf16", 5),
+    (96, 512, 2, 20, 64, "bf16", 8), (56, 333, 1, 24, 64, "bf16", 3),
 ])
 def test_host_slices(H, text, batch, heads, dim, dtype, slices):
     plan = hb.Plan(H, H, 64, 16, 2, text)
