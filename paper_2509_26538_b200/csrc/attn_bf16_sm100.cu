@@ -1227,15 +1227,31 @@ int attn_bf16_prepare(hilberta_plan_t *p, BindImage &image) {
     rc = add_schedule(image, cost, cost_two_heads, p->batch * p->heads, p->sm_count, choice, &p->d_units, &p->d_cta_begin,
                       &p->n_cta, &p->cuts[0], &p->fwd_load);
     if (rc != HILBERTA_OK) return rc;
-    for (int more = 0; more < 2 && p->n_slices > 1; ++more) {
-        if (more && p->heads % p->n_slices == 0) break;
-        rc = add_schedule(image, cost, cost_two_heads, p->batch * (p->heads / p->n_slices + more), p->sm_count, choice,
-                          &p->d_units_slice[more], &p->d_cta_begin_slice[more], &p->n_cta_slice[more]);
-        if (rc != HILBERTA_OK) return rc;
+    p->slice_bytes = 0;
+    if (p->n_slices > 1) {
+        // a unit for every (batch, head) of the larger slices, and every item or share
+        const size_t units = items.size() * p->batch * (size_t)(p->heads / p->n_slices + 1);
+        p->slice_bytes = 2 * (BindImage::up(sizeof(WorkUnit) * units) + BindImage::up(sizeof(int) * (p->sm_count + 1)));
+        p->fwd_cost.swap(cost);
+        p->fwd_cost_two.swap(cost_two_heads);
+        p->fwd_split = choice;
     }
     // the alternative kernels' tables: only where they are selected
     if (forward_kernel_choice() == 's') return attn_bf16_solo_prepare(p, image);
     if (forward_kernel_choice() == 'p') return attn_bf16_pair_prepare(p, image);
+    return HILBERTA_OK;
+}
+
+int attn_bf16_make_slices(hilberta_plan_t *p, char *where, cudaStream_t stream) {
+    BindImage image;
+    for (int more = 0; more < (p->heads % p->n_slices ? 2 : 1); ++more) {
+        const int rc = add_schedule(image, p->fwd_cost, p->fwd_cost_two, p->batch * (p->heads / p->n_slices + more), p->sm_count,
+                                    p->fwd_split, &p->d_units_slice[more], &p->d_cta_begin_slice[more], &p->n_cta_slice[more]);
+        if (rc != HILBERTA_OK) return rc;
+    }
+    if (image.bytes.size() > p->slice_bytes) return HILBERTA_ERR_BUFFER;
+    HB_CUDA(cudaMemcpyAsync(where, image.bytes.data(), image.bytes.size(), cudaMemcpyHostToDevice, stream));   // returns when staged
+    for (const BindImage::Place &at : image.places) *at.where = where + at.at;
     return HILBERTA_OK;
 }
 

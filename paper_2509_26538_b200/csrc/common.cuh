@@ -86,6 +86,15 @@ struct Fp32Work {
     int n_rows;
 };
 
+// How a schedule cuts its longest items (the first n_items of the list) over clusters of `cluster` CTAs;
+// shares: cluster entries per cut item, in rank order, appended to the uploaded work list.
+struct SplitChoice {
+    int cluster = 1, n_clusters = 0, n_items = 0;
+    bool pair_heads = true;
+    long long merge_extra = 0;   // of a share, on top of what a forward merge costs
+    std::vector<WorkItem> shares;
+};
+
 // Tables of a binding, gathered on the host: one allocation and one copy for all of them (every
 // cudaMalloc, cudaFree and pageable copy is tens of microseconds of a bind).  `where` receives the device
 // address; scratch lies behind the tables, uninitialised.
@@ -149,6 +158,11 @@ struct hilberta_plan_s {
     int n_slices;
     // first head of slice c of n
     int slice_begin(int c, int n) const { return c * (heads / n) + (c < heads % n ? c : heads % n); }
+    // The slices' schedules are made by the first host-buffer call (most bindings see none), in its workspace, from:
+    std::vector<long long> fwd_cost, fwd_cost_two;
+    hilberta::SplitChoice fwd_split;
+    size_t slice_bytes;   // the most that they take
+    bool slices_made;
     int split_cluster;            // CTAs per cluster of the forward launches (1: no clusters, no split units)
     long long fwd_load;           // largest CTA load of the forward schedule, in twentieths of a key block (1.45 us)
     hilberta::WorkUnit *d_units_slice[2];   // [1]: of the slices with a head more
@@ -233,14 +247,6 @@ std::vector<WorkItem> build_work_items(const hilberta_plan_t *p, int item_rows, 
 // HILBERTA_OK iff the list is safe to hand to a kernel (ranges inside [0, S), rows covered exactly once)
 int check_work_items(const WorkItem *items, int n, int S, int item_rows, int block);
 int check_shares(const WorkItem *items, int n, const WorkItem *shares, int cluster, int block);
-// How a schedule cuts its longest items (the first n_items of the list) over clusters of `cluster` CTAs;
-// shares: cluster entries per cut item, in rank order, appended to the uploaded work list.
-struct SplitChoice {
-    int cluster = 1, n_clusters = 0, n_items = 0;
-    bool pair_heads = true;
-    long long merge_extra = 0;   // of a share, on top of what a forward merge costs
-    std::vector<WorkItem> shares;
-};
 // clusters: how many clusters of 2, 4 and 8 CTAs run at once.  items sorted by descending cost.  Of
 // `choice` only merge_extra is read.  Not HILBERTA_OK: the shares are not safe to hand to a kernel.
 int choose_split(const std::vector<WorkItem> &items, const std::vector<long long> &cost,
@@ -258,6 +264,8 @@ int add_schedule(BindImage &image, const std::vector<long long> &cost, const std
 // of SMs), 's' (one query tile per CTA) or 0 (the default kernel).
 char forward_kernel_choice();
 int attn_bf16_prepare(hilberta_plan_t *p, BindImage &image);
+// makes the slices' schedules in slice_bytes bytes at `where`, on `stream`
+int attn_bf16_make_slices(hilberta_plan_t *p, char *where, cudaStream_t stream);
 // attn_bf16_pair_sm100.cu: the forward kernel on pairs of SMs (bf16, head dim 128, inputs in physical order)
 int attn_bf16_pair_prepare(hilberta_plan_t *p, BindImage &image);
 int launch_attn_bf16_pair(const hilberta_plan_t *p, const void *q, const void *k, const void *v, void *out,

@@ -711,6 +711,7 @@ static int bind_plan(hilberta_plan_t *p, int batch, int heads, int head_dim, int
     p->bound = false;
     memset(p->cuts, 0, sizeof(p->cuts));
     p->n_slices = 1;   // fp32 bindings have no others
+    p->slices_made = false;
     p->batch = batch;
     p->heads = heads;
     p->head_dim = head_dim;
@@ -884,14 +885,6 @@ extern "C" int hilberta_forward_host(const void *q, const void *k, const void *v
     const size_t esz_out = p->dtype == HILBERTA_FP8_E4M3 ? 2 : esz;
     const size_t bytes = (size_t)p->batch * p->heads * p->S * p->head_dim * esz_out;   // the larger of the two
     const size_t slot = (bytes + 255) & ~(size_t)255;
-    if (p->ws_bytes < 4 * slot) {
-        give_block(p->device, p->ws, p->ws_bytes);
-        p->ws = nullptr;
-        p->ws_bytes = 0;
-        size_t got = 4 * slot;
-        HB_CUDA(take_block(p->device, &p->ws, &got));
-        p->ws_bytes = got;
-    }
     // A copy to pageable memory returns when it is done, so the next slice's copies in would not be queued before and
     // slices only add their fixed costs: 24 heads of 128, 28 MB a tensor, one / four / eight slices 9018 / 9525 / 10195 us
     // with all four buffers pageable and 3234 / 3677 / 4336 with `out` alone.  Pageable inputs are staged beside the
@@ -901,6 +894,16 @@ extern "C" int hilberta_forward_host(const void *q, const void *k, const void *v
         cudaPointerAttributes attr;
         HB_CUDA(cudaPointerGetAttributes(&attr, out));
         if (attr.type == cudaMemoryTypeUnregistered) n = 1;
+    }
+    const size_t need = 4 * slot + (n > 1 ? p->slice_bytes : 0);
+    if (p->ws_bytes < need) {
+        p->slices_made = false;
+        give_block(p->device, p->ws, p->ws_bytes);
+        p->ws = nullptr;
+        p->ws_bytes = 0;
+        size_t got = need;
+        HB_CUDA(take_block(p->device, &p->ws, &got));
+        p->ws_bytes = got;
     }
     if (!p->s_in) HB_CUDA(cudaStreamCreateWithFlags(&p->s_in, cudaStreamNonBlocking));
     if (!p->s_out) HB_CUDA(cudaStreamCreateWithFlags(&p->s_out, cudaStreamNonBlocking));
@@ -935,6 +938,13 @@ extern "C" int hilberta_forward_host(const void *q, const void *k, const void *v
             HB_CUDA(cudaMemcpy2DAsync((char *)in[i] + off, pitch, (const char *)host_in[i] + off, pitch, elems * esz,
                                       p->batch, cudaMemcpyHostToDevice, p->s_in));
         HB_CUDA(cudaEventRecord(p->ev_in[c], p->s_in));
+        if (c == 0 && n > 1 && !p->slices_made) {   // beside the first copies
+            const int rc = guarded([&] { return attn_bf16_make_slices(p, ws + 4 * slot, st); });
+            if (rc != HILBERTA_OK) {
+                HB_CUDA(cudaStreamSynchronize(p->s_in));
+                return rc;
+            }
+        }
         HB_CUDA(cudaStreamWaitEvent(st, p->ev_in[c], 0));
         const int rc = forward_impl(in[0], in[1], in[2], out_dev, nullptr, p, p->d_phys2orig, p->d_phys2orig, st,
                                     n > 1 ? c : -1);
@@ -946,6 +956,7 @@ extern "C" int hilberta_forward_host(const void *q, const void *k, const void *v
     }
     HB_CUDA(cudaStreamSynchronize(p->s_out));
     HB_CUDA(cudaStreamSynchronize(st));
+    if (n > 1) p->slices_made = true;
     return HILBERTA_OK;
 }
 

@@ -71,3 +71,29 @@ def test_pageable_buffers(pinned):
     assert torch.equal(out, want)
     assert launches == 1 if not pinned[1] else launches > 1
     plan.destroy()
+
+
+def test_slices_after_another_bind():
+    """The slices' schedules belong to the binding: other heads, types and cuts in between, in the same workspace, on
+    other streams and with a pageable output."""
+    plan = hb.Plan(64, 64, 512, 0, 8, 512)
+    shapes = [(1, 13, 128, "bf16", 3), (2, 3, 64, "bf16", 2), (1, 24, 128, "fp8", 4), (1, 5, 128, "bf16", 2)]
+    for shape in shapes + shapes[::-1]:
+        with torch.cuda.stream(torch.cuda.Stream()):
+            _check(plan, *shape)
+    plan.destroy()
+    # the first call on a binding in one slice, the next in two, again in one
+    plan = hb.Plan(64, 64, 512, 0, 8, 512)
+    q, k, v = (torch.randn((1, 5, plan.S, 128), device="cuda").bfloat16() for _ in range(3))
+    plan.bind_like(q)
+    want = plan.forward_fused(q, k, v, torch.empty_like(q)).cpu()
+    pageable = [t.cpu() for t in (q, k, v, torch.zeros_like(q))]
+    pinned = [t.pin_memory() for t in pageable]
+    for buffers, slices in ((pageable, 1), (pinned, 2), (pageable, 1), (pinned, 2)):
+        buffers[3].fill_(7.0)
+        before = hb.launch_count()
+        plan.forward_host(*buffers)
+        assert hb.launch_count() - before == slices
+        assert torch.equal(buffers[3], want)
+    assert plan.status() == 0
+    plan.destroy()
