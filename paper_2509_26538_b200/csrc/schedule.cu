@@ -126,9 +126,10 @@ int check_shares(const WorkItem *items, int n, const WorkItem *shares, int clust
 static long long merge_cost(int cluster) { return cluster == 2 ? 85 : cluster == 4 ? 110 : 135; }
 
 // Greedy assignment to the least loaded of n machines (of equally loaded ones the lowest number).  While machines are
-// idle the next of them is the least loaded one, so the heap is only built when all have work, and a schedule of fewer
-// units than machines needs none.  Plan, bind, export and destroy on a B200's host: 44 x 47 tokens, 2 x 12 heads
-// 165 -> 122 us, 64 x 64 + 512, 24 heads 221 -> 184, 128 x 128 + 512 621 -> 580.
+// idle the next of them is the least loaded one, so the heap is built when the last one gets its first unit (built for the
+// first unit that finds none idle: 0.2 us less of 6 for 54 units, 0.5 more of 12 for 432).  Plan, bind, export and destroy on
+// a B200's host, a heap from the first unit on / this: 44 x 47 tokens, 2 x 12 heads 165 / 122 us, 64 x 64 + 512, 24 heads
+// 221 / 184, 128 x 128 + 512 621 / 580.
 struct LeastLoaded {
     typedef std::pair<long long, int> Load;   // (load, machine)
     std::vector<Load> heap;
